@@ -112,10 +112,11 @@ cudaError_t spectra_tc_launch(int n, int fmt, const void* tables, const float* V
 // Per-map bounds of S3 into r.norm (lo at 0..2, 1/(hi-lo) at 3..5; 0 for a flat map).
 cudaError_t minmax_bounds_launch(const float* S3, long long N, const Reduce& r, cudaStream_t s);
 // Normalised maps from S3 and r.norm; one chain per block of `sections` inline sections (0: one chain);
-// W_out [blocks][3]; err2 (nullable) the squared error of every step in filter order.
+// W_out [blocks][3]; err2 (nullable) the squared error of every step in filter order.  scratch: device memory
+// (8-byte aligned) for the regrouped form of the chains, about 6 bytes a voxel; with less the chains run step by step.
 cudaError_t adapt_launch(const float* S3, const float* D, int T, int X, int Y, int method, double mu, double eps,
                          double lambda, double delta, int sections, const float* norm, float* W_out, float* err2,
-                         cudaStream_t s);
+                         void* scratch, size_t scratch_bytes, cudaStream_t s);
 
 // ---- K2: directional center-surround ----------------------------------------------------------
 // Once per device: the shared-memory size limit of the ring-staged K2 (windows whose ring fits 96 KB).
