@@ -29,6 +29,7 @@ struct sal_handle {
     void* tc_tables = nullptr;  // constant tensor-core operands of K1 (BF16/FP16 forms)
     void* adj_tables = nullptr; // constant tensor-core operands of K5 (FP16)
     float* f32_wt = nullptr;    // Eq. 1 weight table of the FP32 K1 / K5 (n <= 16)
+    float* slide_wt = nullptr;  // Eq. 1 weight table of the sliding FP32 K1 (set where that form applies)
     float* sp_tab = nullptr;    // spatial-domain reading: the Eq. 1 ratio table
     float* vpad = nullptr;      // V with rows padded to ypad floats (tensor-core forms, Y not a multiple of 4)
     int ypad = 0;
@@ -70,6 +71,8 @@ void free_scratch(sal_handle* h) {
     h->tc_tables = h->adj_tables = nullptr;
     if (h->f32_wt) cudaFree(h->f32_wt);
     h->f32_wt = nullptr;
+    if (h->slide_wt) cudaFree(h->slide_wt);
+    h->slide_wt = nullptr;
     if (h->sp_tab) cudaFree(h->sp_tab);
     h->sp_tab = nullptr;
     if (h->vpad) cudaFree(h->vpad);
@@ -133,14 +136,15 @@ cudaError_t launch_k1(sal_handle* h, const float* V, float* E, cudaStream_t st) 
     cudaError_t e;
     if (h->feature == 2) {
         e = sal::spatial_f32_launch(h->n, h->sp_tab, V, E, h->T, h->X, h->Y, h->boundary, h->taper, st);
+    } else if (h->slide_wt) {
+        e = sal::spectra_f32_slide_launch(h->n, h->slide_wt, V, out, h->T, h->X, h->Y, h->boundary, h->feature, st);
     } else if (h->n == 32) {
         e = h->prec == SAL_FP32
-                ? sal::spectra_f32_n32_launch(h->tw, V, out, h->T, h->X, h->Y, h->boundary, h->feature, s, h->taper, st)
+                ? sal::spectra_f32_n32_launch(h->tw, V, out, h->T, h->X, h->Y, h->boundary, h->feature, s, st)
                 : sal::spectra_tc32_launch(h->prec == SAL_BF16 ? 1 : 0, h->tw, V, out, h->T, h->X, h->Y, h->boundary,
                                            h->feature, s, h->err_dev, st);
     } else if (h->prec == SAL_FP32) {
-        e = sal::spectra_f32_launch(h->n, h->tw, h->f32_wt, V, out, h->T, h->X, h->Y, h->boundary, h->feature, s,
-                                    h->taper, st);
+        e = sal::spectra_f32_launch(h->n, h->tw, h->f32_wt, V, out, h->T, h->X, h->Y, h->boundary, h->feature, s, st);
     } else {
         const float* vt = padded_copy(h, V, st, e);
         if (e == cudaSuccess)
@@ -149,6 +153,20 @@ cudaError_t launch_k1(sal_handle* h, const float* V, float* E, cudaStream_t st) 
     }
     if (e != cudaSuccess || s == 1) return e;
     return sal::upsample_launch(h->Ec, E, h->T, h->X, h->Y, s, st);
+}
+
+// sal_create: one of the handle's tables to the device; a failure frees the handle.
+sal_status upload_table(sal_handle* h, const std::vector<float>& t, float** dst) {
+    const size_t bytes = t.size() * sizeof(float);
+    cudaError_t e = cudaMalloc(dst, bytes);
+    const bool oom = e != cudaSuccess;
+    if (!oom) e = cudaMemcpy(*dst, t.data(), bytes, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) return SAL_OK;
+    free_scratch(h);
+    delete h;
+    cudaGetLastError();
+    if (oom) return fail(nullptr, SAL_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+    return cuda_fail(nullptr, e, "cudaMemcpy");
 }
 
 }  // namespace
@@ -312,6 +330,11 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
         if (e == cudaSuccess && h->prec != SAL_FP32) e = sal::spectra_tc_prepare(h->n, h->prec == SAL_BF16 ? 1 : 0);
         if (e == cudaSuccess && h->prec != SAL_FP32) e = sal::spectra_adjoint_tc_prepare(h->n, 0);
     }
+    // the rect cube at stride 1 and n >= 8: the sliding form of the FP32 K1 (a tapered window does not slide, and on a
+    // lattice there is no run of neighbours to slide over)
+    const bool slide = h->prec == SAL_FP32 && h->feature != 2 && h->taper == 0 && h->stride == 1 &&
+                       sal::f32_slide_supported(h->n);
+    if (e == cudaSuccess && slide) e = sal::spectra_f32_slide_prepare(h->n);
     if (e == cudaSuccess && h->feature == 2) e = sal::spatial_f32_prepare();
     if (e == cudaSuccess) e = sal::dcs_prepare();
     if (e == cudaSuccess) e = sal::dcs_adjoint_prepare();
@@ -325,6 +348,7 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
     const size_t adj_bytes = tc_fwd ? sal::spectra_adjoint_tc_tables_bytes(h->n) : 0;
     const bool f32_tab = h->prec == SAL_FP32 && sal::spectra_f32_supported(h->n) && h->feature != 2;
     const size_t wt_bytes = f32_tab ? sal::f32_weight_table_floats(h->n) * sizeof(float) : 0;
+    const size_t sl_bytes = slide ? sal::f32_slide_table_floats(h->n) * sizeof(float) : 0;
     const size_t sp_bytes = h->feature == 2 ? sal::spatial_weight_table_floats(h->n) * sizeof(float) : 0;
     const int sc = p->stride;
     const size_t ec_bytes = sc > 1 ? (size_t)3 * ((T + sc - 1) / sc) * ((X + sc - 1) / sc) * ((Y + sc - 1) / sc) *
@@ -333,7 +357,8 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
     // the tensor-core forms stage interior bricks by TMA from a row-padded copy when rows are not 16-byte multiples
     const int ypad = (Y + 3) & ~3;
     const size_t vpad_bytes = tc_fwd && h->feature != 2 && ypad != Y ? (size_t)T * X * ypad * sizeof(float) : 0;
-    const size_t need = 2 * plane3 + small + tab_bytes + adj_bytes + ec_bytes + wt_bytes + sp_bytes + vpad_bytes;
+    const size_t need = 2 * plane3 + small + tab_bytes + adj_bytes + ec_bytes + wt_bytes + sl_bytes + sp_bytes +
+                        vpad_bytes;
     if (h->budget && need > h->budget) {
         delete h;
         return fail(nullptr, SAL_ERR_OOM, "scratch (" + std::to_string(need) + " B) exceeds hbm_budget_bytes");
@@ -403,17 +428,14 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
     if (f32_tab) {
         std::vector<float> wt(sal::f32_weight_table_floats(h->n));
         sal::f32_weight_table_fill(h->n, h->feature, wt.data());
-        if ((e = cudaMalloc(&h->f32_wt, wt_bytes)) != cudaSuccess) {
-            free_scratch(h);
-            delete h;
-            cudaGetLastError();
-            return fail(nullptr, SAL_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-        }
-        if ((e = cudaMemcpy(h->f32_wt, wt.data(), wt_bytes, cudaMemcpyHostToDevice)) != cudaSuccess) {
-            free_scratch(h);
-            delete h;
-            return cuda_fail(nullptr, e, "cudaMemcpy");
-        }
+        const sal_status us = upload_table(h, wt, &h->f32_wt);
+        if (us != SAL_OK) return us;
+    }
+    if (slide) {
+        std::vector<float> wt(sal::f32_slide_table_floats(h->n));
+        sal::f32_slide_table_fill(h->n, h->feature, wt.data());
+        const sal_status us = upload_table(h, wt, &h->slide_wt);
+        if (us != SAL_OK) return us;
     }
     if (sp_bytes) {
         std::vector<float> rt(sal::spatial_weight_table_floats(h->n));

@@ -66,11 +66,18 @@ struct Reduce {
 // at voxels whose indices are multiples of s; E is then the lattice [3][ceil(T/s)][ceil(X/s)][ceil(Y/s)].
 bool spectra_f32_supported(int n);
 cudaError_t spectra_f32_prepare(int n);
-// taper 0 (rect) at stride 1 takes the sliding form of stage 3 for n >= 8
 // wtab: the Eq. 1 weight table of the FP32 kernels (f32_weight_table_fill), device memory
 cudaError_t spectra_f32_launch(int n, const TwiddleTable& tw, const float* wtab, const float* V, float* E, int T,
-                               int X, int Y, int bnd, int feat, int stride, int taper, cudaStream_t s);
+                               int X, int Y, int bnd, int feat, int stride, cudaStream_t s);
 size_t f32_weight_table_floats(int n);
+// The sliding form of K1 (rect cube, stride 1, n = 8, 16, 32).  wtab: its own weight table
+// (f32_slide_table_fill, host; device copy)
+bool f32_slide_supported(int n);
+size_t f32_slide_table_floats(int n);
+void f32_slide_table_fill(int n, int feat, float* out);
+cudaError_t spectra_f32_slide_prepare(int n);
+cudaError_t spectra_f32_slide_launch(int n, const float* wtab, const float* V, float* E, int T, int X, int Y, int bnd,
+                                     int feat, cudaStream_t s);
 // The spatial-domain reading of the feature step (FP32, n in {2, 4, 8, 16}, stride 1): per-window separable
 // FFTs in shared memory (spatial_f32_prepare sets their shared-memory limits; once per device).  rtab: the
 // Eq. 1 ratio table (spatial_weight_table_fill, host; 16-byte aligned device copy).
@@ -90,9 +97,8 @@ cudaError_t pad_rows_launch(const float* V, float* Vp, long long rows, int Y, in
 
 // K1 for the 32^3 window: FP32 on the SIMT pipes, or on the tensor cores (BF16 fmt = 1, FP16 fmt = 0)
 cudaError_t spectra_f32_n32_prepare();
-// taper 0 (rect) at stride 1 takes the sliding form of stage 3
 cudaError_t spectra_f32_n32_launch(const TwiddleTable& tw, const float* V, float* E, int T, int X, int Y, int bnd,
-                                   int feat, int stride, int taper, cudaStream_t s);
+                                   int feat, int stride, cudaStream_t s);
 cudaError_t spectra_tc32_prepare(int fmt);
 cudaError_t spectra_tc32_launch(int fmt, const TwiddleTable& tw, const float* V, float* E, int T, int X, int Y,
                                 int bnd, int feat, int stride, int* err, cudaStream_t s);

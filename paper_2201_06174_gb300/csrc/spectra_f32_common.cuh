@@ -94,10 +94,9 @@ template <int N_, int BY_, int NT_> struct Brick {
     static constexpr int G_FLOAT2 = H * N * YH;
     static_assert(NT % 32 == 0 && NT >= YH, "staging maps one y position per thread");
 
-    // Halo brick of V into s_in [N][N][YH], border extension applied per axis, minus vshift (a constant
-    // over the brick moves only the DC bin of a rect-tapered cube).
+    // Halo brick of V into s_in [N][N][YH], border extension applied per axis.
     __device__ static void stage_brick(const float* __restrict__ V, float* s_in, int T, int X, int Y, int bnd,
-                                       int t0, int x0, int y_start, float vshift = 0.f) {
+                                       int t0, int x0, int y_start) {
         constexpr int RSTEP = NT / YH;
         constexpr int ITERS = (N * N + RSTEP - 1) / RSTEP;   // rows per thread: all loads issued, then stored
         const int tid = threadIdx.x;
@@ -120,7 +119,7 @@ template <int N_, int BY_, int NT_> struct Brick {
 #pragma unroll
             for (int i = 0; i < ITERS; ++i) {
                 const int r = r0 + i * RSTEP;
-                if (r < N * N) s_in[r * YH + yy] = v[i] - vshift;
+                if (r < N * N) s_in[r * YH + yy] = v[i];
             }
         }
     }

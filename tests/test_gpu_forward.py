@@ -91,6 +91,36 @@ def test_hann_taper_features_match_oracle(sal, n, prec, tol):
         assert rel_l2(g["E"][m], E[m]) <= tol, (m, rel_l2(g["E"][m], E[m]))
 
 
+# the sliding form's bricks (n = 8: 8 x0 by 32 or 8 y0; 16: 12 by 32 or 8; 32: 6 by 16) past their edges, in its
+# short runs (small volumes) and its long ones, cubes larger than the volume, and every border extension
+@pytest.mark.parametrize("feature", ["abs", "energy"])
+@pytest.mark.parametrize("n,shape,boundary", [
+    (8, (3, 9, 9), "symmetric"), (8, (5, 17, 41), "zero"), (8, (33, 25, 65), "periodic"), (8, (30, 33, 67), "zero"),
+    (16, (1, 1, 1), "symmetric"), (16, (3, 13, 9), "periodic"), (16, (20, 25, 33), "symmetric"),
+    (16, (16, 37, 31), "zero"), (32, (2, 7, 5), "symmetric"), (32, (13, 13, 17), "symmetric"),
+    (32, (20, 6, 50), "zero"), (32, (3, 5, 9), "periodic"),
+])
+def test_sliding_bricks_match_oracle(sal, n, shape, boundary, feature):
+    V = np.random.RandomState(n + sum(shape)).randn(*shape).astype(np.float32) + 0.5
+    g = _run(sal, V, sal.Params(n=n, boundary=boundary, feature=feature))
+    E = oracle.features(V, n, boundary=boundary, feature=feature)
+    for m in range(3):   # a few dozen FP32 roundings per bin; a volume of one voxel has no features but 1e-15 of noise
+        err = np.linalg.norm(g["E"][m] - E[m])
+        assert err <= 1e-6 * max(np.linalg.norm(E[m]), 1e-6 * np.linalg.norm(V)), (m, err)
+
+
+def test_sliding_form_keeps_a_nan_to_its_windows(sal):
+    V = np.random.RandomState(2).randn(9, 20, 70).astype(np.float32)
+    E0 = _run(sal, V, sal.Params(n=8))["E"]
+    V[4, 8, 32] = np.nan
+    E1 = _run(sal, V, sal.Params(n=8))["E"]
+    bad = np.isnan(E1).any(0)
+    t, x, y = np.nonzero(bad)
+    assert bad[4, 8, 32] and x.min() >= 8 - 3 and x.max() <= 8 + 4 and y.min() >= 32 - 3 and y.max() <= 32 + 4 + 15
+    # the same up to rounding: the brick whose corner is not finite is staged without a shift
+    assert np.abs(E1[:, ~bad] - E0[:, ~bad]).max() <= 1e-6 * np.abs(E0).max()
+
+
 @pytest.mark.parametrize("n,shape", [(8, (4, 5, 200)), (16, (3, 4, 150))])
 def test_sliding_form_long_rows(sal, n, shape):
     """Rows long enough for many y bricks (ragged last brick): every chunk of the sliding recursion
