@@ -607,11 +607,12 @@ k4_galpha_finalize(const double* __restrict__ part, int nparts, const __grid_con
 // slice u_t of brick t0 lies at t_ext = t0 - n/2 + u_t.
 //   pass 1 (along t): ext[i][brick][x'][y'] = sum over t0 of the slices at t_ext = t_begin - n/2 + i, for
 //     every extended plane i < t_step (t_count - 1) + n -- contiguous slices, read once;
-//   pass 2 (across bricks): gV[q] += sum of ext over the extended positions (t_ext, x_ext, y_ext) that
+//   pass 2 (across bricks): gV[q] += (or =, add = false: the only slab) sum of ext over the extended positions (t_ext, x_ext, y_ext) that
 //     map to q and the bricks that hold them.
 // Both passes sum in a fixed order, so the result is deterministic.
-// Pass 1: one warp per (plane i, brick) row of `slice` contiguous floats (slice4 = slice / 4 16-byte groups:
-// the blocks' slices are padded to a multiple of 4 floats), lanes along the row.
+// Pass 1: (plane i, brick) rows of `slice` contiguous floats (slice4 = slice / 4 16-byte groups: the blocks' slices
+// are padded to a multiple of 4 floats), a warp per 32 groups of a row, each lane's up to 16 loads at once: a warp per
+// whole row left small volumes to the latency of its five to seven rounds (12 x 16 x 20, n = 16: 41 us).
 __global__ void __launch_bounds__(kThreads)
 k5_gather_t(const float4* __restrict__ blocks, float4* __restrict__ ext, int n, int nb, int slice4, int t_count,
             int t_step) {
@@ -621,15 +622,18 @@ k5_gather_t(const float4* __restrict__ blocks, float4* __restrict__ ext, int n, 
     const long long rows = (long long)(t_step * (t_count - 1) + n) * nb;
     // from the slice of brick r to that of brick r + 1 on the same plane: the next t0's block, u_t - t_step
     const long long rstep = (long long)nb * bsz - (long long)t_step * slice4;
-    for (long long w = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5); w < rows;
-         w += (long long)gridDim.x * kWarps) {
+    const int parts = (slice4 + 31) / 32;
+    for (long long item = (long long)blockIdx.x * kWarps + (threadIdx.x >> 5); item < rows * parts;
+         item += (long long)gridDim.x * kWarps) {
+        const long long w = item / parts;
+        const int e = (int)(item - w * parts) * 32 + lane;
         const int brick = (int)(w % nb), i = (int)(w / nb);
         // the bricks r whose slice u_t = i - t_step r (< n) lands on plane i, in increasing r
         const int r_lo = i >= n ? (i - n + t_step) / t_step : 0;
         const int nr = min(t_count - 1, i / t_step) - r_lo + 1;   // at most 16 (n <= 16)
         const float4* src = blocks + ((long long)r_lo * nb + brick) * bsz + (long long)(i - t_step * r_lo) * slice4;
         float4* dst = ext + w * slice4;
-        for (int e = lane; e < slice4; e += 32) {
+        if (e < slice4) {
             float4 v[16];
 #pragma unroll
             for (int j = 0; j < 16; ++j) v[j] = j < nr ? __ldg(src + j * rstep + e) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -649,7 +653,7 @@ k5_gather_t(const float4* __restrict__ blocks, float4* __restrict__ ext, int n, 
 // Pass 2: one thread per voxel; block (32 y, 8 x) of plane t = t_lo + blockIdx.z.
 __global__ void __launch_bounds__(kThreads)
 k5_gather_xy(const float* __restrict__ ext, float* __restrict__ gV, int T, int X, int Y, int bnd, int n, int BX,
-             int XH, int BY, int YH, int slice, int t_begin, int t_count, int t_step, int t_lo) {
+             int XH, int BY, int YH, int slice, int t_begin, int t_count, int t_step, int t_lo, int add) {
     const int h2 = n / 2;
     const int nseg = (Y + BY - 1) / BY;
     const int nxs = (X + BX - 1) / BX;
@@ -685,7 +689,7 @@ k5_gather_xy(const float* __restrict__ ext, float* __restrict__ gV, int T, int X
                     sum += __ldg(plane + (long long)(xs * nseg + sg) * slice + (x - xs * BX + h2) * YH +
                                  (y - sg * BY + h2));
         }
-        gV[q] += sum;
+        gV[q] = add ? gV[q] + sum : 0.f + sum;
         return;
     }
     int et[40], ex[40], ey[40];
@@ -711,7 +715,7 @@ k5_gather_xy(const float* __restrict__ ext, float* __restrict__ gV, int T, int X
             }
         }
     }
-    gV[q] += sum;
+    gV[q] = add ? gV[q] + sum : 0.f + sum;
 }
 
 // gS3[m][p] = coef[m] * gS[p]
@@ -812,13 +816,14 @@ size_t gather_ext_floats(int n, SpectraAdjointGeometry g, int X, int Y, int t_co
 }
 
 cudaError_t gather_add_launch(const float* blocks, float* ext, float* gV, int T, int X, int Y, int bnd, int n,
-                              SpectraAdjointGeometry g, int t_begin, int t_count, int t_step, cudaStream_t s) {
+                              SpectraAdjointGeometry g, int t_begin, int t_count, int t_step, bool add,
+                              cudaStream_t s) {
     if (n > 16 || t_step < 1) return cudaErrorInvalidValue;   // pass 1 unrolls up to 16 bricks per plane
     const int nb = ((X + g.BX - 1) / g.BX) * ((Y + g.BY - 1) / g.BY);
     const long long e_total = (long long)gather_ext_floats(n, g, X, Y, t_count, t_step);
     if (g.slice % 4 != 0) return cudaErrorInvalidValue;   // pass 1 moves 16-byte groups
-    const long long rows1 = e_total / g.slice;   // (plane, brick) rows, a warp each
-    long long b1 = (rows1 + kThreads / 32 - 1) / (kThreads / 32);
+    const long long warps1 = e_total / g.slice * ((g.slice / 4 + 31) / 32);   // 32 groups of a (plane, brick) row each
+    long long b1 = (warps1 + kThreads / 32 - 1) / (kThreads / 32);
     const long long cap1 = 8LL * device_sms();   // grid-stride: 8 blocks per SM
     if (b1 > cap1) b1 = cap1;
     if (b1 < 1) b1 = 1;
@@ -835,7 +840,7 @@ cudaError_t gather_add_launch(const float* blocks, float* ext, float* gV, int T,
     static_assert(kThreads == 32 * 8, "pass 2 blocks are 32 y x 8 x");
     const dim3 grid2((Y + 31) / 32, (X + 7) / 8, t_hi - t_lo);   // T, X <= 65535 (checked at create)
     k5_gather_xy<<<grid2, dim3(32, 8), 0, s>>>(ext, gV, T, X, Y, bnd, n, g.BX, g.XH, g.BY, g.YH, g.slice, t_begin,
-                                              t_count, t_step, t_lo);
+                                              t_count, t_step, t_lo, add ? 1 : 0);
     note_launches(2);
     return cudaGetLastError();
 }

@@ -591,9 +591,11 @@ sal_status ensure_backward_scratch(sal_handle* h) {
 // gV = (dE/dV)^T gE through the brick blocks of K5 and the fixed-order overlap-add, slab by slab.
 sal_status spectral_adjoint(sal_handle* h, const float* V, const float* gE, float* gV, cudaStream_t st) {
     cudaError_t e;
-    if ((e = cudaMemsetAsync(gV, 0, (size_t)h->N * sizeof(float), st)) != cudaSuccess)
-        return cuda_fail(h, e, "spectral adjoint: memset");
     const int sc = h->stride;
+    const int planes = (h->T + sc - 1) / sc;
+    const bool slabs = planes > h->slab_t;   // several slabs add their parts into gV
+    if (slabs && (e = cudaMemsetAsync(gV, 0, (size_t)h->N * sizeof(float), st)) != cudaSuccess)
+        return cuda_fail(h, e, "spectral adjoint: memset");
     if (sc > 1) {
         // stride s: the gradient of the interpolated features back onto the lattice voxels; the cubes of
         // the other voxels were never taken, so only the bricks of the lattice planes run
@@ -603,7 +605,6 @@ sal_status spectral_adjoint(sal_handle* h, const float* V, const float* gE, floa
         gE = h->gEl;
     }
     const sal::SpectraAdjointGeometry g = adjoint_geometry(h);
-    const int planes = (h->T + sc - 1) / sc;
     const float* vt = nullptr;
     if (h->prec != SAL_FP32) {
         vt = padded_copy(h, V, st, e);
@@ -630,7 +631,7 @@ sal_status spectral_adjoint(sal_handle* h, const float* V, const float* gE, floa
                                                  st);
         if (e != cudaSuccess) return cuda_fail(h, e, "spectral adjoint");
         if ((e = sal::gather_add_launch(h->blocks, h->gext, gV, h->T, h->X, h->Y, h->boundary, h->n, g, t_begin, cnt,
-                                        sc, st)) != cudaSuccess)
+                                        sc, slabs, st)) != cudaSuccess)
             return cuda_fail(h, e, "spectral adjoint: overlap-add");
     }
     return SAL_OK;

@@ -190,10 +190,12 @@ cudaError_t dcs_adjoint_galpha_launch(const float* E, const float* gS, long long
                                       size_t tile_part_bytes, double* part, float* galpha, cudaStream_t s);
 cudaError_t expand_gradient_launch(const float* gS, const float* coef, float* gS3, long long N, cudaStream_t s);
 // Overlap-add of one slab's brick blocks into gV through the scratch `ext` (gather_ext_floats floats):
-// first along t (contiguous slices), then across the bricks that overlap each voxel.
+// first along t (contiguous slices), then across the bricks that overlap each voxel.  add = false: the slab holds every
+// plane's bricks, and gV is written instead of added to.
 size_t gather_ext_floats(int n, SpectraAdjointGeometry g, int X, int Y, int t_count, int t_step);
 cudaError_t gather_add_launch(const float* blocks, float* ext, float* gV, int T, int X, int Y, int bnd, int n,
-                              SpectraAdjointGeometry g, int t_begin, int t_count, int t_step, cudaStream_t s);
+                              SpectraAdjointGeometry g, int t_begin, int t_count, int t_step, bool add,
+                              cudaStream_t s);
 
 // One CTA waits, through the tensor-core kernels' bounded mbarrier wait, on a barrier that nobody
 // arrives at, gives up after `tries` tries and sets the error word (failure-detection check).
