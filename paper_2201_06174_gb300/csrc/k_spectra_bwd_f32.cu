@@ -24,21 +24,29 @@
 // One CTA = one brick (t0, x0, y_start .. y_start+BY-1), same mapping as K1:
 //   1. stage brick, forward stages 1 and 2 (shared with K1);
 //   2. per (row, y0): forward stage 3 -> Gamma -> inverse DFT along y (pairing k, n-k), added
-//      into a private accumulation window of the thread (thread-interleaved shared memory); for the rect
-//      cube at n = 8, 16 both y-passes slide over the thread's run of outputs (see SL below);
+//      into a private accumulation window of the thread (thread-interleaved shared memory);
 //   3. windows of the y-chunks summed into Gamma_G2[k_t][k_x][y];
 //   4. adjoint of stage 2 (x) -> Gamma_G1[k_t][u_x][y];
 //   5. adjoint of stage 1 (t), real part -> the brick's block [u_t][u_x][y] of gVext, written to
 //      scratch; a separate gather kernel sums the overlapping blocks in a fixed order.
-#include "spectra_f32_common.cuh"
+#include "spectra_f32_exact.cuh"
 
 namespace sal {
 namespace {
 
+using f32::Exact2f;
+using f32::FF;
+using f32::ff_add;
+using f32::ff_mul;
+using f32::ff_mul1;
+using f32::kSmallBin;
+using f32::kZeroBin;
+using f32::make_exact2f;
+using f32::make_vanish_tab;
 using f32::Tw;
+using f32::vanish_mask;
+using f32::VanishTab;
 
-constexpr float kSmallBin = 1.0f / 65536.0f;       // FP32 |F| / A_p at or below which a bin is resolved exactly
-constexpr float kZeroBin = 1.0f / 68719476736.0f;  // float-float max(|Re F|, |Im F|) / A_p at or below which F = 0
 constexpr int kListQ = 32;   // small bins a CTA may hand to the listed-bin passes (more: it resolves them itself)
 // Layout of the listed-bin scratch of one launch of ncta CTAs (ints): [0] the number of listed bins, [4 ..)
 // the work list (cta << 5 | entry, in no particular order), then per CTA kListStride ints: [0] its count,
@@ -46,104 +54,6 @@ constexpr int kListQ = 32;   // small bins a CTA may hand to the listed-bin pass
 // (Re, Im) of each entry's Gamma, written by the exact pass.
 constexpr int kListStride = 1 + 3 * kListQ;
 __host__ __device__ constexpr size_t list_cta_offset(long long ncta) { return 4 + (size_t)ncta * kListQ; }
-
-// Float-float constants of the exact recompute: cos, sin of 2 pi m / n and the taper h(u), each as a pair
-// (hi, lo) of FP32 values whose sum is the double-precision value.
-template <int N> struct Exact2f {
-    float ch[N], cl[N], sh[N], sl[N], hh[N], hl[N];
-};
-
-// Masks of the bins that vanish for every input, per axis (t, x, y): bit k of the mask of position p
-// (the cube's samples p - n/2 .. p + n/2 - 1 of that axis) is set when bin k of that axis vanishes.
-// Positions whose cube lies inside the axis never vanish; the others are p < n (entries 0 .. n-1) and
-// p >= L - n (entries n .. 2n-1).
-struct VanishTab {
-    uint16_t m[3][32];
-    int L[3];
-};
-
-__device__ __forceinline__ uint32_t vanish_mask(const VanishTab& v, int a, int p, int n) {
-    const int L = v.L[a];
-    if (p - n / 2 >= 0 && p + n / 2 - 1 < L) return 0u;
-    return p < n ? v.m[a][p] : v.m[a][n + (p - (L - n))];
-}
-
-// Host: does bin k of the one-axis cube at position p (axis length L) vanish for every input?  The bin is
-// sum_m h(m) w^(k m) x[src(m)] (w = exp(-2 pi i / n)), so it vanishes for all x iff, for each source
-// sample j, the coefficient sum_{m: src(m) = j} h(m) w^(k m) is 0.  With n a power of two, w has minimal
-// polynomial w^(n/2) + 1, so the coefficient is zero iff its coordinates on w^0 .. w^(n/2-1)
-// (w^(e + n/2) = -w^e) are; they are integers for the rect taper (h = 1) and, scaled by 4, for the
-// periodic Hann taper (4 h(m) w^(km) = 2 w^(km) - w^(km+m) - w^(km-m)).  Exact: no rounding enters.
-inline bool axis_bin_vanishes(int n, int p, int L, int bnd, int taper, int k) {
-    if (p - n / 2 >= 0 && p + n / 2 - 1 < L) return false;
-    int src[32];
-    for (int m = 0; m < n; ++m) src[m] = ext_index(p - n / 2 + m, L, bnd);
-    for (int m = 0; m < n; ++m) {
-        if (src[m] < 0) continue;
-        bool first = true;
-        for (int q = 0; q < m; ++q) first = first && src[q] != src[m];
-        if (!first) continue;
-        int a[16] = {0};
-        for (int q = m; q < n; ++q) {
-            if (src[q] != src[m]) continue;
-            const int e0 = (k * q) % n;
-            const int es[3] = {e0, (e0 + q) % n, (e0 - q + n) % n};
-            const int vs[3] = {taper ? 2 : 1, taper ? -1 : 0, taper ? -1 : 0};
-            for (int r = 0; r < 3; ++r) {
-                if (es[r] < n / 2) a[es[r]] += vs[r];
-                else a[es[r] - n / 2] -= vs[r];
-            }
-        }
-        for (int e = 0; e < n / 2; ++e)
-            if (a[e] != 0) return false;
-    }
-    return true;
-}
-
-inline uint16_t axis_vanish_mask(int n, int p, int L, int bnd, int taper) {
-    uint16_t mk = 0;
-    for (int k = 0; k < n; ++k)
-        if (axis_bin_vanishes(n, p, L, bnd, taper, k)) mk = (uint16_t)(mk | (1u << k));
-    return mk;
-}
-
-inline VanishTab make_vanish_tab(int n, int T, int X, int Y, int bnd, int taper) {
-    VanishTab v{};
-    const int L[3] = {T, X, Y};
-    for (int a = 0; a < 3; ++a) {
-        v.L[a] = L[a];
-        for (int p = 0; p < n && p < L[a]; ++p) v.m[a][p] = axis_vanish_mask(n, p, L[a], bnd, taper);
-        for (int p = L[a] - n > 0 ? L[a] - n : 0; p < L[a]; ++p)
-            v.m[a][n + (p - (L[a] - n))] = axis_vanish_mask(n, p, L[a], bnd, taper);
-    }
-    return v;
-}
-
-// Float-float arithmetic (an unevaluated sum hi + lo of two FP32 values): the error-free transformations
-// two-sum (Knuth) and the FMA product residual, with the usual renormalisation.
-struct FF {
-    float hi, lo;
-};
-__device__ __forceinline__ FF ff_fast_two_sum(float a, float b) {   // |a| >= |b|
-    const float s = a + b;
-    return {s, b - (s - a)};
-}
-__device__ __forceinline__ FF ff_add(FF a, FF b) {
-    const float s = a.hi + b.hi;
-    const float bb = s - a.hi;
-    const float e = (a.hi - (s - bb)) + (b.hi - bb);
-    return ff_fast_two_sum(s, e + a.lo + b.lo);
-}
-__device__ __forceinline__ FF ff_mul(FF a, FF b) {
-    const float p = a.hi * b.hi;
-    float e = fmaf(a.hi, b.hi, -p);
-    e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
-    return ff_fast_two_sum(p, e);
-}
-__device__ __forceinline__ FF ff_mul1(float a, FF b) {   // a exact in FP32
-    const float p = a * b.hi;
-    return ff_fast_two_sum(p, fmaf(a, b.lo, fmaf(a, b.hi, -p)));
-}
 
 template <int N> struct BCfg;
 template <> struct BCfg<2>  { static constexpr int BY = 32, YC = 1, MINB = 4; };
@@ -500,23 +410,15 @@ k5_listed_apply_f32(float* __restrict__ blocks, const int* __restrict__ lists, l
     }
 }
 
-// EN: the energy reading of the feature (Gamma = 2 rho F, no kink band).  SL: both y-passes slide (rect
-// taper, n = 8, 16).  With the phase anchored at the start y_r of the thread's run,
-//   Ft_j[k] = F_{y_r + j}[k] w^(k j) = sum_{y = j}^{j + n - 1} G2[y_r + y] w^(k y),   w = e^(-2 pi i / n),
-// the forward recompute is Ft_0 by the direct sum, then Ft_{j+1} = Ft_j + (G2[y_r + j + n] - G2[y_r + j]) w^(k j),
-// and |Ft| = |F|, so Gamma~_j = Gamma(Ft_j) = Gamma_j w^(k j) (the direction and the energy reading alike).
-// The inverse along y of the run, dG2[y_r + p] = sum_{j <= p < j + n} sum_k Gamma_j[k] e^(2 pi i k (p - j)/n),
-// is then z(P, p) = sum_k P[k] e^(2 pi i k p / n) of the sum P of Gamma~_j over the outputs j whose window
-// holds p: for a run of YC <= n outputs, with the prefix sums P_i = sum_{j <= i} Gamma~_j,
-//   p < YC - 1:  z(P_p, p);     YC - 1 <= p < n:  z(P_{YC-1}, p);     p = n + i:  z(P_{YC-1}, i) - z(P_i, i),
-// (z has period n in p): YC + n - 1 point evaluations of n bins per run instead of YC n.
-// The brick is staged as is: the small-bin level below is relative to the raw window's L1 norm.
-template <int N, bool EN, bool SL>
-__global__ void __launch_bounds__(BGeo<N>::NT, BCfg<N>::MINB)
-k5_spectra_adjoint_f32(const float* __restrict__ V, const float* __restrict__ gE, float* __restrict__ blocks,
-                       int T, int X, int Y, int bnd, int t_begin, int t_step, const float* __restrict__ wtab,
-                       int taper, const __grid_constant__ Tw<N> tw, const __grid_constant__ Exact2f<N> ex,
-                       const __grid_constant__ VanishTab vt, int* __restrict__ lists) {
+// One brick (t0, x0, y_start ..), cta its index among the launch's.  EN: the energy reading of the feature (Gamma = 2 rho
+// F, no kink band).  DENSE: a part of a brick of the sliding form, of geometry dg: outputs past dg.BY are none of its
+// own, every small bin is resolved in place, and the block is added to blk.
+template <int N, bool EN, bool DENSE>
+__device__ __forceinline__ void adjoint_brick(const float* __restrict__ V, const float* __restrict__ gE, float* blk,
+                                              int T, int X, int Y, int bnd, int t0, int x0, int y_start,
+                                              const float* __restrict__ wtab, int taper, const Tw<N>& tw,
+                                              const Exact2f<N>& ex, const VanishTab& vt, int* __restrict__ lists,
+                                              long long cta, long long ncta, const SpectraAdjointGeometry& dg) {
     using G = BGeo<N>;
     using B = typename G::B;
     constexpr int H = G::H, BY = G::BY, YC = G::YC, YH = G::YH, ROWS = G::ROWS, NT = G::NT, WIN = G::WIN;
@@ -533,9 +435,6 @@ k5_spectra_adjoint_f32(const float* __restrict__ V, const float* __restrict__ gE
     int* s_src = reinterpret_cast<int*>(smem_raw + G::IDX_OFF);                   // [2][N] cube rows along t, x
 
     const int tid = threadIdx.x;
-    const int y_start = blockIdx.x * BY;
-    const int x0 = blockIdx.y;
-    const int t0 = t_begin + blockIdx.z * t_step;   // t_step s > 1: the lattice planes of stride-s windows
     const size_t NV = (size_t)T * X * Y;
 
     if (!EN)
@@ -544,7 +443,7 @@ k5_spectra_adjoint_f32(const float* __restrict__ V, const float* __restrict__ gE
     B::stage_brick(V, s_in, T, X, Y, bnd, t0, x0, y_start);
     for (int i = tid; i < 3 * BY; i += NT) {
         const int m = i / BY, yl = i % BY, y = y_start + yl;
-        s_ge[i] = y < Y ? __ldg(gE + m * NV + ((size_t)t0 * X + x0) * Y + y) : 0.f;
+        s_ge[i] = y < Y && (!DENSE || yl < dg.BY) ? __ldg(gE + m * NV + ((size_t)t0 * X + x0) * Y + y) : 0.f;
     }
     __syncthreads();
     // window L1 norms A[y0] = sum_u h(u_t) h(u_x) h(u_y) |V|, as column sums then a y box sum
@@ -569,37 +468,16 @@ k5_spectra_adjoint_f32(const float* __restrict__ V, const float* __restrict__ gE
     const int ych = tid / ROWS;
     float wt[3][H];
     B::row_weights(wtab, row, wt);
-    if constexpr (!SL) {   // the sliding inverse writes every window position itself
 #pragma unroll
-        for (int j = 0; j < WIN; ++j) s_win[j * NT + tid] = make_float2(0.f, 0.f);
-    }
-    static_assert(!SL || YC <= N, "the sliding inverse needs runs of at most n outputs");
+    for (int j = 0; j < WIN; ++j) s_win[j * NT + tid] = make_float2(0.f, 0.f);
     const float2* grow = s_g2 + (size_t)row * YH;
-    float fr[N], fi[N];   // F[k_y] of the current output, all n bins (SL: Ft, the run-anchored phase)
-    // SL: prefix sums over the run's outputs of the pair coefficients below (the pairing is linear)
-    float par[H], pai[H], pbr[H], pbi[H];
-#pragma unroll
-    for (int k = 0; k < H; ++k) par[k] = pai[k] = pbr[k] = pbi[k] = 0.f;
-    // z(P, p): sum_k P[k] e^(2 pi i k p / n) from the pair coefficients of P, at run position p (mod n)
-    auto z_at = [&](int p, float& zr, float& zi) {
-        zr = 0.f;
-        zi = 0.f;
-#pragma unroll
-        for (int k = 0; k < H; ++k) {
-            zr = fmaf(par[k], tw.c[k][p], zr);
-            zi = fmaf(pai[k], tw.c[k][p], zi);
-            if (k != 0 && 2 * k != N) {
-                zr = fmaf(pbr[k], tw.s[k][p], zr);
-                zi = fmaf(pbi[k], tw.s[k][p], zi);
-            }
-        }
-    };
+    float fr[N], fi[N];   // F[k_y] of the current output, all n bins
     // the whole row vanishes when its k_t or its k_x does
     const bool row_vanishes =
         !EN && (((vanish_mask(vt, 0, t0, N) >> (row / N)) | (vanish_mask(vt, 1, x0, N) >> (row % N))) & 1u);
     for (int yi = 0; yi < YC; ++yi) {
         const int yl = ych * YC + yi;
-        if (!SL || yi == 0) {
+        {
             float pr[H], pi[H], qr[H], qi[H];
 #pragma unroll
             for (int k = 0; k < H; ++k) pr[k] = pi[k] = qr[k] = qi[k] = 0.f;
@@ -627,18 +505,6 @@ k5_spectra_adjoint_f32(const float* __restrict__ V, const float* __restrict__ gE
                     fr[N - k] = pr[k] - qi[k];   // F[n-k] = P + iQ
                     fi[N - k] = pi[k] + qr[k];
                 }
-            }
-        } else {
-            // Ft_yi = Ft_{yi-1} + (entering - leaving) w^(k (yi - 1)), w^(k m) = c - i sn
-            const float2 a = grow[yl - 1], b = grow[yl - 1 + N];   // sample leaving, sample entering
-            const float dr = b.x - a.x, di = b.y - a.y;
-            const int m = yi - 1;
-#pragma unroll
-            for (int k = 0; k < N; ++k) {
-                const float c = k <= N / 2 ? tw.c[k][m] : tw.c[N - k][m];
-                const float sn = k <= N / 2 ? tw.s[k][m] : -tw.s[N - k][m];
-                fr[k] = fmaf(dr, c, fmaf(di, sn, fr[k]));
-                fi[k] = fmaf(di, c, fmaf(-dr, sn, fi[k]));
             }
         }
         const float g0 = s_ge[yl], g1 = s_ge[BY + yl], g2 = s_ge[2 * BY + yl];
@@ -680,68 +546,31 @@ k5_spectra_adjoint_f32(const float* __restrict__ V, const float* __restrict__ gE
             if (small != 0u) small &= ~vanish_mask(vt, 2, y_start + yl, N);
             s_small[yi * NT + tid] = (uint16_t)small;
         }
-        if constexpr (SL) {
-            // P_yi = P_{yi-1} + Gamma~_yi; position yi takes z(P_yi, yi), position n + yi its negative (the
-            // full sum's value is added below)
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            float zr = 0.f, zi = 0.f;
 #pragma unroll
             for (int k = 0; k < H; ++k) {
-                par[k] += ar[k];
-                pai[k] += ai[k];
-                pbr[k] += br[k];
-                pbi[k] += bi[k];
-            }
-            if (yi < YC - 1) {
-                float zr, zi;
-                z_at(yi, zr, zi);
-                s_win[yi * NT + tid] = make_float2(zr, zi);
-                s_win[(N + yi) * NT + tid] = make_float2(-zr, -zi);
-            }
-        } else {
-#pragma unroll
-            for (int u = 0; u < N; ++u) {
-                float zr = 0.f, zi = 0.f;
-#pragma unroll
-                for (int k = 0; k < H; ++k) {
-                    zr = fmaf(ar[k], tw.c[k][u], zr);
-                    zi = fmaf(ai[k], tw.c[k][u], zi);
-                    if (k != 0 && 2 * k != N) {
-                        zr = fmaf(br[k], tw.s[k][u], zr);
-                        zi = fmaf(bi[k], tw.s[k][u], zi);
-                    }
+                zr = fmaf(ar[k], tw.c[k][u], zr);
+                zi = fmaf(ai[k], tw.c[k][u], zi);
+                if (k != 0 && 2 * k != N) {
+                    zr = fmaf(br[k], tw.s[k][u], zr);
+                    zi = fmaf(bi[k], tw.s[k][u], zi);
                 }
-                float2* w = s_win + (yi + u) * NT + tid;
-                float2 acc = *w;
-                acc.x += zr;
-                acc.y += zi;
-                *w = acc;
             }
-        }
-    }
-    if constexpr (SL) {
-        // the full sum P_{YC-1}: positions YC - 1 .. n - 1 take z(P_{YC-1}, p); positions n + i add z(P_{YC-1}, i)
-#pragma unroll
-        for (int p = 0; p < N; ++p) {
-            float zr, zi;
-            z_at(p, zr, zi);
-            if (p < YC - 1) {
-                float2* w = s_win + (N + p) * NT + tid;
-                float2 acc = *w;
-                acc.x += zr;
-                acc.y += zi;
-                *w = acc;
-            } else {
-                s_win[p * NT + tid] = make_float2(zr, zi);
-            }
+            float2* w = s_win + (yi + u) * NT + tid;
+            float2 acc = *w;
+            acc.x += zr;
+            acc.y += zi;
+            *w = acc;
         }
     }
     if (!EN) {
         // the small bins go to the listed-bin pass when a list is given and they fit in it
         unsigned* s_wbits = reinterpret_cast<unsigned*>(smem_raw + G::WB_OFF);
-        const size_t cta = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-        const size_t ncta = (size_t)gridDim.x * gridDim.y * gridDim.z;
-        const bool listed = lists && list_small_bins<NT, YC>(s_small, s_wbits,
+        const bool listed = !DENSE && lists && list_small_bins<NT, YC>(s_small, s_wbits,
                                                              lists + list_cta_offset(ncta) + cta * kListStride,
-                                                             lists + 4, lists, (long long)cta);
+                                                             lists + 4, lists, cta);
         if (!listed)
             resolve_small_bins<N, NT, YC, BY, H, ROWS>(V, X, Y, bnd, y_start, taper, s_small, s_src, s_win, s_ge,
                                                        s_l1, wtab, tw, ex, s_wbits);
@@ -800,8 +629,6 @@ k5_spectra_adjoint_f32(const float* __restrict__ V, const float* __restrict__ gE
     __syncthreads();
 
     // ---- step 5: adjoint of stage 1 (t), real part -> scratch block [u_t][u_x][y] -------------
-    const size_t cta = ((size_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
-    float* blk = blocks + cta * G::BLOCK_FLOATS;
     for (int it = tid; it < N * YH; it += NT) {
         const int ux = it / YH, y = it % YH;
         float2 g[H];
@@ -815,62 +642,84 @@ k5_spectra_adjoint_f32(const float* __restrict__ V, const float* __restrict__ gE
                 z = fmaf(g[k].x, tw.c[k][u], z);
                 if (k != 0 && 2 * k != N) z = fmaf(-g[k].y, tw.s[k][u], z);
             }
-            blk[(size_t)u * G::SLICE + ux * YH + y] = z;
+            if (!DENSE) blk[(size_t)u * G::SLICE + ux * YH + y] = z;
+            else if (y < dg.YH) blk[(size_t)u * dg.slice + ux * dg.YH + y] += z;
         }
     }
 }
 
-template <int N> constexpr bool kAdjointSliding = N >= 8;
+// A CTA per brick (one x0).  The rect cube at n = 8, 16 takes the sliding form (k_spectra_bwd_f32_slide.cu).
+template <int N, bool EN>
+__global__ void __launch_bounds__(BGeo<N>::NT, BCfg<N>::MINB)
+k5_spectra_adjoint_f32(const float* __restrict__ V, const float* __restrict__ gE, float* __restrict__ blocks,
+                       int T, int X, int Y, int bnd, int t_begin, int t_step, const float* __restrict__ wtab,
+                       int taper, const __grid_constant__ Tw<N> tw, const __grid_constant__ Exact2f<N> ex,
+                       const __grid_constant__ VanishTab vt, int* __restrict__ lists) {
+    const long long cta = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    // t_step s > 1: the lattice planes of stride-s windows
+    adjoint_brick<N, EN, false>(V, gE, blocks + cta * BGeo<N>::BLOCK_FLOATS, T, X, Y, bnd,
+                                t_begin + blockIdx.z * t_step, blockIdx.y, blockIdx.x * BGeo<N>::BY, wtab, taper, tw,
+                                ex, vt, lists, cta, (long long)gridDim.x * gridDim.y * gridDim.z,
+                                SpectraAdjointGeometry{});
+}
+
+// The bricks the sliding form leaves (dense[brick] set: more small bins than it lists): the blocks walk over the marks,
+// a marked brick's x0 one after the other into its block.
+template <int N>
+__global__ void __launch_bounds__(BGeo<N>::NT, BCfg<N>::MINB)
+k5_dense_f32(const float* __restrict__ V, const float* __restrict__ gE, float* __restrict__ blocks, int T, int X, int Y,
+             int bnd, int t_begin, int t_step, int t_count, const float* __restrict__ wtab,
+             const __grid_constant__ Tw<N> tw, const __grid_constant__ Exact2f<N> ex,
+             const __grid_constant__ VanishTab vt, const SpectraAdjointGeometry dg, const int* __restrict__ dense) {
+    const int nseg = (Y + dg.BY - 1) / dg.BY, nxs = (X + dg.BX - 1) / dg.BX;
+    const long long total = (long long)nseg * nxs * t_count;
+    for (long long b = blockIdx.x; b < total; b += gridDim.x) {
+        if (!dense[b]) continue;   // block-uniform
+        const int sg = (int)(b % nseg), xs = (int)(b / nseg % nxs), t0 = t_begin + (int)(b / ((long long)nseg * nxs)) * t_step;
+        float* blk = blocks + b * dg.block_floats;
+        for (int i = threadIdx.x; i < dg.block_floats; i += BGeo<N>::NT) blk[i] = 0.f;
+        for (int x0 = xs * dg.BX; x0 < min(X, xs * dg.BX + dg.BX); ++x0) {
+            __syncthreads();   // the block is zeroed; the previous x0 is done with it and with shared memory
+            adjoint_brick<N, false, true>(V, gE, blk + (size_t)(x0 - xs * dg.BX) * dg.YH, T, X, Y, bnd, t0, x0,
+                                          sg * dg.BY, wtab, 0, tw, ex, vt, nullptr, 0, 1, dg);
+        }
+    }
+}
+
+template <int N> constexpr bool kHasSliding = N >= 8;   // the rect cube takes k_spectra_bwd_f32_slide.cu
 
 template <int N>
 cudaError_t prepare_n() {
     constexpr int smem = (int)BGeo<N>::SMEM;
-    cudaError_t e = cudaFuncSetAttribute(k5_spectra_adjoint_f32<N, false, false>,
+    cudaError_t e = cudaFuncSetAttribute(k5_spectra_adjoint_f32<N, false>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k5_spectra_adjoint_f32<N, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if constexpr (kAdjointSliding<N>) {
+        e = cudaFuncSetAttribute(k5_spectra_adjoint_f32<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if constexpr (kHasSliding<N>) {
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k5_spectra_adjoint_f32<N, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     smem);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k5_spectra_adjoint_f32<N, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     smem);
+            e = cudaFuncSetAttribute(k5_dense_f32<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     }
     return e;
 }
 
-// The float-float constants of the exact recompute of small bins: cos, sin (2 pi m / n) and the taper
-// (rect, or the periodic Hann window 1/2 - cos(2 pi u / n) / 2), from the host's double-precision libm,
-// each split into an FP32 head and the FP32 rounding of the remainder.
 template <int N>
-Exact2f<N> make_exact2f(int taper) {
-    Exact2f<N> e;
-    auto split = [](double v, float& hi, float& lo) {
-        hi = (float)v;
-        lo = (float)(v - (double)hi);
-    };
-    for (int m = 0; m < N; ++m) {
-        const double a = 2.0 * 3.14159265358979323846 * m / N;
-        split(cos(a), e.ch[m], e.cl[m]);
-        split(sin(a), e.sh[m], e.sl[m]);
-        split(taper ? 0.5 - 0.5 * cos(a) : 1.0, e.hh[m], e.hl[m]);
-    }
-    return e;
-}
-
-template <int N, bool SL>
-void launch_sl(const TwiddleTable& t, const float* wtab, dim3 grid, const float* V, const float* gE, float* blocks,
-               int T, int X, int Y, int bnd, int feat, int t_begin, int t_step, int taper, int* lists,
-               cudaStream_t s) {
+cudaError_t launch_n(const TwiddleTable& t, const float* wtab, const float* V, const float* gE, float* blocks, int T,
+                     int X, int Y, int bnd, int feat, int t_begin, int t_step, int t_count, int taper, int* lists,
+                     cudaStream_t s) {
     using G = BGeo<N>;
+    dim3 grid((Y + G::BY - 1) / G::BY, X, t_count);
+    note_launches(1);
     if (feat == 1) {
-        k5_spectra_adjoint_f32<N, true, SL><<<grid, G::NT, G::SMEM, s>>>(
+        k5_spectra_adjoint_f32<N, true><<<grid, G::NT, G::SMEM, s>>>(
             V, gE, blocks, T, X, Y, bnd, t_begin, t_step, wtab, taper, f32::make_tw<N>(t), make_exact2f<N>(taper),
             VanishTab{}, nullptr);
-        return;
+        return cudaGetLastError();
     }
-    k5_spectra_adjoint_f32<N, false, SL><<<grid, G::NT, G::SMEM, s>>>(
+    if (lists) {   // the work-list counter starts at zero
+        const cudaError_t e = cudaMemsetAsync(lists, 0, sizeof(int), s);
+        if (e != cudaSuccess) return e;
+    }
+    k5_spectra_adjoint_f32<N, false><<<grid, G::NT, G::SMEM, s>>>(
         V, gE, blocks, T, X, Y, bnd, t_begin, t_step, wtab, taper, f32::make_tw<N>(t), make_exact2f<N>(taper),
         make_vanish_tab(N, T, X, Y, bnd, taper), lists);
     if (lists) {
@@ -880,26 +729,20 @@ void launch_sl(const TwiddleTable& t, const float* wtab, dim3 grid, const float*
         k5_listed_apply_f32<N><<<(unsigned)((ncta + 7) / 8), 256, 0, s>>>(blocks, lists, ncta, f32::make_tw<N>(t));
         note_launches(2);
     }
+    return cudaGetLastError();
 }
 
 template <int N>
-cudaError_t launch_n(const TwiddleTable& t, const float* wtab, const float* V, const float* gE, float* blocks, int T,
-                     int X, int Y, int bnd, int feat, int t_begin, int t_step, int t_count, int taper, int* lists,
-                     cudaStream_t s) {
+cudaError_t launch_dense(const TwiddleTable& t, const float* wtab, const float* V, const float* gE, float* blocks,
+                         int T, int X, int Y, int bnd, int t_begin, int t_step, int t_count, const int* dense,
+                         cudaStream_t s) {
     using G = BGeo<N>;
-    dim3 grid((Y + G::BY - 1) / G::BY, X, t_count);
-    if (lists && feat != 1) {   // the work-list counter starts at zero
-        const cudaError_t e = cudaMemsetAsync(lists, 0, sizeof(int), s);
-        if (e != cudaSuccess) return e;
-    }
-    if constexpr (kAdjointSliding<N>) {
-        if (taper == 0)
-            launch_sl<N, true>(t, wtab, grid, V, gE, blocks, T, X, Y, bnd, feat, t_begin, t_step, taper, lists, s);
-        else
-            launch_sl<N, false>(t, wtab, grid, V, gE, blocks, T, X, Y, bnd, feat, t_begin, t_step, taper, lists, s);
-    } else {
-        launch_sl<N, false>(t, wtab, grid, V, gE, blocks, T, X, Y, bnd, feat, t_begin, t_step, taper, lists, s);
-    }
+    const SpectraAdjointGeometry g = spectra_adjoint_f32_slide_geometry(N);
+    const long long total = (long long)((Y + g.BY - 1) / g.BY) * ((X + g.BX - 1) / g.BX) * t_count;
+    const int grid = (int)(total < 2 * device_sms() ? total : 2 * device_sms());
+    k5_dense_f32<N><<<grid, G::NT, G::SMEM, s>>>(V, gE, blocks, T, X, Y, bnd, t_begin, t_step, t_count, wtab,
+                                                 f32::make_tw<N>(t), make_exact2f<N>(0),
+                                                 make_vanish_tab(N, T, X, Y, bnd, 0), g, dense);
     note_launches(1);
     return cudaGetLastError();
 }
@@ -924,6 +767,15 @@ SpectraAdjointGeometry spectra_adjoint_f32_geometry(int n) {
         case 16: return {BGeo<16>::BY, BGeo<16>::YH, 1, 16, BGeo<16>::BLOCK_FLOATS, BGeo<16>::SLICE};
         default: return {0, 0, 0, 0, 0, 0};
     }
+}
+
+cudaError_t spectra_adjoint_f32_dense_launch(int n, const TwiddleTable& tw, const float* wtab, const float* V,
+                                             const float* gE, float* blocks, int T, int X, int Y, int bnd,
+                                             int t_begin, int t_step, int t_count, const int* dense, cudaStream_t s) {
+    if (t_step < 1) return cudaErrorInvalidValue;
+    if (n == 8) return launch_dense<8>(tw, wtab, V, gE, blocks, T, X, Y, bnd, t_begin, t_step, t_count, dense, s);
+    if (n == 16) return launch_dense<16>(tw, wtab, V, gE, blocks, T, X, Y, bnd, t_begin, t_step, t_count, dense, s);
+    return cudaErrorInvalidValue;
 }
 
 size_t spectra_adjoint_f32_list_bytes(int n, int X, int Y, int t_count) {

@@ -29,7 +29,7 @@ struct sal_handle {
     void* tc_tables = nullptr;  // constant tensor-core operands of K1 (BF16/FP16 forms)
     void* adj_tables = nullptr; // constant tensor-core operands of K5 (FP16)
     float* f32_wt = nullptr;    // Eq. 1 weight table of the FP32 K1 / K5 (n <= 16)
-    float* slide_wt = nullptr;  // Eq. 1 weight table of the sliding FP32 K1 (set where that form applies)
+    float* slide_wt = nullptr;  // Eq. 1 weight table of the sliding FP32 K1 (stride 1) and K5 (n <= 16): rect cubes
     float* sp_tab = nullptr;    // spatial-domain reading: the Eq. 1 ratio table
     float* vpad = nullptr;      // V with rows padded to ypad floats (tensor-core forms, Y not a multiple of 4)
     int ypad = 0;
@@ -41,6 +41,7 @@ struct sal_handle {
     float* gext = nullptr;   // the blocks summed along t, per extended plane of the slab
     float* gEl = nullptr;    // stride > 1: the feature gradient gathered onto the lattice voxels (zero elsewhere)
     int slab_t = 0;
+    bool adj_slide = false;  // the FP32 adjoint's sliding form (rect cube, n = 8, 16), set with the backward scratch
     volatile int* err_host = nullptr;  // mapped host word set by bounded device waits that gave up
     int* err_dev = nullptr;
     size_t bytes = 0;
@@ -136,7 +137,7 @@ cudaError_t launch_k1(sal_handle* h, const float* V, float* E, cudaStream_t st) 
     cudaError_t e;
     if (h->feature == 2) {
         e = sal::spatial_f32_launch(h->n, h->sp_tab, V, E, h->T, h->X, h->Y, h->boundary, h->taper, st);
-    } else if (h->slide_wt) {
+    } else if (h->slide_wt && s == 1) {
         e = sal::spectra_f32_slide_launch(h->n, h->slide_wt, V, out, h->T, h->X, h->Y, h->boundary, h->feature, st);
     } else if (h->n == 32) {
         e = h->prec == SAL_FP32
@@ -330,11 +331,11 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
         if (e == cudaSuccess && h->prec != SAL_FP32) e = sal::spectra_tc_prepare(h->n, h->prec == SAL_BF16 ? 1 : 0);
         if (e == cudaSuccess && h->prec != SAL_FP32) e = sal::spectra_adjoint_tc_prepare(h->n, 0);
     }
-    // the rect cube at stride 1 and n >= 8: the sliding form of the FP32 K1 (a tapered window does not slide, and on a
-    // lattice there is no run of neighbours to slide over)
-    const bool slide = h->prec == SAL_FP32 && h->feature != 2 && h->taper == 0 && h->stride == 1 &&
-                       sal::f32_slide_supported(h->n);
+    // the rect cube at n >= 8: the sliding forms of the FP32 K1 (stride 1) and K5 (a tapered window does not slide, and
+    // the forward on a lattice has no run of neighbours to slide over)
+    const bool slide = h->prec == SAL_FP32 && h->feature != 2 && h->taper == 0 && sal::f32_slide_supported(h->n);
     if (e == cudaSuccess && slide) e = sal::spectra_f32_slide_prepare(h->n);
+    if (e == cudaSuccess && slide && h->n != 32) e = sal::spectra_adjoint_f32_slide_prepare(h->n);
     if (e == cudaSuccess && h->feature == 2) e = sal::spatial_f32_prepare();
     if (e == cudaSuccess) e = sal::dcs_prepare();
     if (e == cudaSuccess) e = sal::dcs_adjoint_prepare();
@@ -541,27 +542,40 @@ constexpr size_t kBlocksCap = (size_t)2 << 30;  // brick-block scratch of the sp
 // Brick geometry of the spectral adjoint in the handle's precision.
 sal::SpectraAdjointGeometry adjoint_geometry(const sal_handle* h) {
     if (h->feature == 2) return sal::spatial_adjoint_f32_geometry(h->n);
+    if (h->adj_slide) return sal::spectra_adjoint_f32_slide_geometry(h->n);
     return h->prec == SAL_FP32 ? sal::spectra_adjoint_f32_geometry(h->n) : sal::spectra_adjoint_tc_geometry(h->n);
 }
 
 sal_status ensure_backward_scratch(sal_handle* h) {
     if (h->n == 32) return fail(h, SAL_ERR_UNSUPPORTED, "the backward is built for n in {2,4,8,16}");
     if (h->gE) return SAL_OK;
-    const sal::SpectraAdjointGeometry g = adjoint_geometry(h);
-    const int nseg = (h->Y + g.BY - 1) / g.BY;
-    const size_t per_t = (size_t)((h->X + g.BX - 1) / g.BX) * nseg * g.block_floats * sizeof(float);
-    // the overlap-add's scratch: one brick-summed plane per extended plane of the slab (s (slab - 1) + n,
-    // s the stride: the bricks of a slab sit on the lattice planes)
     const int sc = h->stride;
-    const size_t per_ext = sal::gather_ext_floats(h->n, g, h->X, h->Y, 1, 1) / h->n * sizeof(float);
-    const size_t ext_fixed = (size_t)(h->n - sc) * per_ext;
+    h->adj_slide = h->prec == SAL_FP32 && h->feature != 2 && h->taper == 0 && (h->n == 8 || h->n == 16);
+    sal::SpectraAdjointGeometry g;
+    size_t per_t, per_ext, ext_fixed;
+    auto sizes = [&]() {
+        g = adjoint_geometry(h);
+        const int nseg = (h->Y + g.BY - 1) / g.BY;
+        per_t = (size_t)((h->X + g.BX - 1) / g.BX) * nseg * g.block_floats * sizeof(float);
+        // the overlap-add's scratch: one brick-summed plane per extended plane of the slab (s (slab - 1) + n,
+        // s the stride: the bricks of a slab sit on the lattice planes)
+        per_ext = sal::gather_ext_floats(h->n, g, h->X, h->Y, 1, 1) / h->n * sizeof(float);
+        ext_fixed = (size_t)(h->n - sc) * per_ext;
+    };
+    sizes();
     const int planes = (h->T + sc - 1) / sc;   // lattice planes (every plane at stride 1)
     size_t cap = kBlocksCap;
     const size_t plane3 = (size_t)3 * h->N * sizeof(float);
     const size_t lat3 = sc > 1 ? plane3 : 0;
     const size_t bpart = (size_t)sal::kRedBlocks * 64 * sizeof(double);
     if (h->budget) {
-        const size_t used = h->bytes + plane3 + lat3 + bpart + ext_fixed;
+        const size_t fixed = h->bytes + plane3 + lat3 + bpart;
+        if (h->adj_slide && fixed + ext_fixed + per_t + sc * per_ext > h->budget) {
+            // volumes of a few x positions: the sliding form's wider bricks may not fit where the others do
+            h->adj_slide = false;
+            sizes();
+        }
+        const size_t used = fixed + ext_fixed;
         if (used + per_t + sc * per_ext > h->budget)
             return fail(h, SAL_ERR_OOM, "backward scratch exceeds hbm_budget_bytes");
         cap = std::min(cap, h->budget - used);
@@ -612,7 +626,8 @@ sal_status spectral_adjoint(sal_handle* h, const float* V, const float* gE, floa
     }
     // the FP32 adjoint lists its small bins in the overlap-add's plane buffer, free until the gather runs
     const size_t ext_bytes = sal::gather_ext_floats(h->n, g, h->X, h->Y, h->slab_t, sc) * sizeof(float);
-    int* lists = h->prec == SAL_FP32 && h->feature == 0 &&
+    // (the sliding form: a mark per brick)
+    int* lists = h->prec == SAL_FP32 && h->feature == 0 && !h->adj_slide &&
                          sal::spectra_adjoint_f32_list_bytes(h->n, h->X, h->Y, h->slab_t) <= ext_bytes
                      ? reinterpret_cast<int*>(h->gext)
                      : nullptr;
@@ -621,6 +636,10 @@ sal_status spectral_adjoint(sal_handle* h, const float* V, const float* gE, floa
         e = h->feature == 2
                 ? sal::spatial_adjoint_f32_launch(h->n, h->sp_tab, V, gE, h->blocks, h->T, h->X, h->Y, h->boundary, t_begin, cnt,
                                                   h->taper, st)
+            : h->adj_slide
+                ? sal::spectra_adjoint_f32_slide_launch(h->n, h->slide_wt, V, gE, h->blocks, h->T, h->X, h->Y, h->boundary,
+                                                        h->feature, t_begin, sc, cnt, reinterpret_cast<int*>(h->gext),
+                                                        st)
             : h->prec == SAL_FP32
                 ? sal::spectra_adjoint_f32_launch(h->n, h->tw, h->f32_wt, V, gE, h->blocks, h->T, h->X, h->Y,
                                                   h->boundary, h->feature, t_begin, sc, cnt, h->taper, lists, st)
@@ -629,6 +648,10 @@ sal_status spectral_adjoint(sal_handle* h, const float* V, const float* gE, floa
                 : sal::spectra_adjoint_tc_launch(h->n, 0, h->tw, h->adj_tables, V, gE, h->blocks, h->T, h->X, h->Y,
                                                  h->boundary, h->feature, t_begin, sc, cnt, vt, h->ypad, h->err_dev,
                                                  st);
+        if (e == cudaSuccess && h->adj_slide && h->feature == 0)
+            e = sal::spectra_adjoint_f32_dense_launch(h->n, h->tw, h->f32_wt, V, gE, h->blocks, h->T, h->X, h->Y,
+                                                      h->boundary, t_begin, sc, cnt,
+                                                      reinterpret_cast<const int*>(h->gext), st);
         if (e != cudaSuccess) return cuda_fail(h, e, "spectral adjoint");
         if ((e = sal::gather_add_launch(h->blocks, h->gext, gV, h->T, h->X, h->Y, h->boundary, h->n, g, t_begin, cnt,
                                         sc, slabs, st)) != cudaSuccess)

@@ -156,6 +156,17 @@ size_t spectra_adjoint_f32_list_bytes(int n, int X, int Y, int t_count);
 cudaError_t spectra_adjoint_f32_launch(int n, const TwiddleTable& tw, const float* wtab, const float* V,
                                        const float* gE, float* blocks, int T, int X, int Y, int bnd, int feat,
                                        int t_begin, int t_step, int t_count, int taper, int* lists, cudaStream_t s);
+// The sliding form of the FP32 adjoint (rect cube, n = 8, 16): bricks of its own geometry.  wtab: the weight table of
+// the sliding forward (f32_slide_table_fill).  dense [bricks of the launch] (device): bricks it leaves, with more
+// small bins than it lists; spectra_adjoint_f32_dense_launch then computes those blocks (abs(F) reading only).
+cudaError_t spectra_adjoint_f32_slide_prepare(int n);
+SpectraAdjointGeometry spectra_adjoint_f32_slide_geometry(int n);
+cudaError_t spectra_adjoint_f32_slide_launch(int n, const float* wtab, const float* V, const float* gE, float* blocks,
+                                             int T, int X, int Y, int bnd, int feat, int t_begin, int t_step,
+                                             int t_count, int* dense, cudaStream_t s);
+cudaError_t spectra_adjoint_f32_dense_launch(int n, const TwiddleTable& tw, const float* wtab, const float* V,
+                                             const float* gE, float* blocks, int T, int X, int Y, int bnd,
+                                             int t_begin, int t_step, int t_count, const int* dense, cudaStream_t s);
 // K5 on the tensor cores (FP16 operands: fmt must be 0); its constant operands are built once per handle
 cudaError_t spectra_adjoint_tc_prepare(int n, int fmt);
 size_t spectra_adjoint_tc_tables_bytes(int n);

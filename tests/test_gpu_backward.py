@@ -148,6 +148,48 @@ def test_spectral_adjoint_taper_and_long_rows(sal, n, shape, taper, prec, tol):
     assert rel_l2(got, ref) <= tol, rel_l2(got, ref)
 
 
+# the sliding adjoint's bricks (n = 8: 16 x0 by 16 y0; 16: 12 by 16, two to a CTA) past their edges, an odd brick over,
+# cubes larger than the volume, every border extension, lattice planes
+@pytest.mark.parametrize("feature", ["abs", "energy"])
+@pytest.mark.parametrize("n,shape,boundary,stride", [
+    (8, (3, 17, 17), "symmetric", 1), (8, (2, 33, 40), "zero", 1), (8, (9, 5, 3), "periodic", 1),
+    (8, (7, 18, 33), "symmetric", 3), (16, (3, 13, 17), "zero", 1), (16, (2, 25, 33), "symmetric", 1),
+    (16, (17, 3, 5), "periodic", 1), (16, (5, 12, 19), "periodic", 2), (16, (1, 1, 16), "zero", 1),
+])
+def test_sliding_adjoint_bricks_match_oracle(sal, n, shape, boundary, stride, feature):
+    r = np.random.RandomState(n + sum(shape))
+    V, gE = r.randn(*shape).astype(np.float32) + 0.3, r.randn(3, *shape).astype(np.float32)
+    eng = sal.Saliency(shape, sal.Params(n=n, boundary=boundary, stride=stride, feature=feature))
+    try:
+        gV = torch.empty(shape, dtype=torch.float32, device="cuda")
+        sal.sal_local_spectra_project_backward(eng.h, _cuda(V), _cuda(gE), gV)
+        torch.cuda.synchronize()
+        got = gV.cpu().numpy()
+    finally:
+        eng.close()
+    want = oracle.features_adjoint(V, gE, n, boundary=boundary, feature=feature, stride=stride)
+    assert rel_l2(got, want) <= RTOL
+
+
+def test_adjoint_within_a_budget_the_sliding_form_exceeds(sal):
+    """One x position: the sliding form's bricks take more scratch than the direct form's, which then runs."""
+    shape, n = (6, 1, 40), 16
+    V, gE = synth.random_volume(shape, seed=1), synth.random_volume((3,) + shape, seed=2)
+    base = sal.Saliency(shape, sal.Params(n=n))
+    created = sal.sal_workspace_size(base.h)
+    base.close()
+    per_ext = 3 * 496 * 4   # three y segments of 16 x 31 floats; a block holds n of them
+    budget = created + 3 * int(np.prod(shape)) * 4 + 1216 * 64 * 8 + (n - 1) * per_ext + n * per_ext + per_ext
+    eng = sal.Saliency(shape, sal.Params(n=n, hbm_budget_bytes=budget))
+    try:
+        gV = torch.empty(shape, dtype=torch.float32, device="cuda")
+        sal.sal_local_spectra_project_backward(eng.h, _cuda(V), _cuda(gE), gV)
+        torch.cuda.synchronize()
+        assert rel_l2(gV.cpu().numpy(), oracle.features_adjoint(V, gE, n)) <= RTOL
+    finally:
+        eng.close()
+
+
 @pytest.mark.parametrize("boundary,shape", [("symmetric", (9, 8, 35)), ("periodic", (9, 8, 35)), ("zero", (9, 8, 35)),
                                             ("symmetric", (20, 24, 70)), ("periodic", (20, 24, 70)),
                                             ("zero", (19, 27, 66))])
