@@ -142,8 +142,8 @@ cudaError_t launch_k1(sal_handle* h, const float* V, float* E, cudaStream_t st) 
     } else if (h->n == 32) {
         e = h->prec == SAL_FP32
                 ? sal::spectra_f32_n32_launch(h->tw, V, out, h->T, h->X, h->Y, h->boundary, h->feature, s, st)
-                : sal::spectra_tc32_launch(h->prec == SAL_BF16 ? 1 : 0, h->tw, V, out, h->T, h->X, h->Y, h->boundary,
-                                           h->feature, s, h->err_dev, st);
+                : sal::spectra_tc32_launch(h->prec == SAL_BF16 ? 1 : 0, h->tw, h->tc_tables, h->S3, V, out, h->T, h->X,
+                                           h->Y, h->boundary, h->feature, s, h->err_dev, st);
     } else if (h->prec == SAL_FP32) {
         e = sal::spectra_f32_launch(h->n, h->tw, h->f32_wt, V, out, h->T, h->X, h->Y, h->boundary, h->feature, s, st);
     } else {
@@ -345,7 +345,8 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
     const size_t small = (size_t)sal::kRedBlocks * 8 * sizeof(float) + (size_t)sal::kRedBlocks * 16 * sizeof(double)
                          + 32 * sizeof(float) + 16 * sizeof(double) + 256;
     const bool tc_fwd = h->prec != SAL_FP32 && sal::spectra_tc_supported(h->n);
-    const size_t tab_bytes = tc_fwd ? sal::spectra_tc_tables_bytes(h->n) : 0;
+    const bool tc32 = h->prec != SAL_FP32 && h->n == 32;
+    const size_t tab_bytes = tc_fwd ? sal::spectra_tc_tables_bytes(h->n) : tc32 ? sal::spectra_tc32_tables_bytes() : 0;
     const size_t adj_bytes = tc_fwd ? sal::spectra_adjoint_tc_tables_bytes(h->n) : 0;
     const bool f32_tab = h->prec == SAL_FP32 && sal::spectra_f32_supported(h->n) && h->feature != 2;
     const size_t wt_bytes = f32_tab ? sal::f32_weight_table_floats(h->n) * sizeof(float) : 0;
@@ -421,6 +422,20 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
                                               0)) != cudaSuccess ||
             (e = sal::spectra_adjoint_tc_tables_build(h->n, h->tw, h->feature, h->adj_tables, 0)) != cudaSuccess ||
             (e = cudaStreamSynchronize(0)) != cudaSuccess) {
+            free_scratch(h);
+            delete h;
+            return cuda_fail(nullptr, e, "tensor-core tables");
+        }
+    }
+    if (tc32) {
+        if ((e = cudaMalloc(&h->tc_tables, tab_bytes)) != cudaSuccess) {
+            free_scratch(h);
+            delete h;
+            cudaGetLastError();
+            return fail(nullptr, SAL_ERR_OOM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+        }
+        if ((e = sal::spectra_tc32_tables_build(h->prec == SAL_BF16 ? 1 : 0, h->tw, h->feature, h->tc_tables, 0)) !=
+            cudaSuccess) {
             free_scratch(h);
             delete h;
             return cuda_fail(nullptr, e, "tensor-core tables");

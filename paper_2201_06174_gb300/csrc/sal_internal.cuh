@@ -100,8 +100,14 @@ cudaError_t spectra_f32_n32_prepare();
 cudaError_t spectra_f32_n32_launch(const TwiddleTable& tw, const float* V, float* E, int T, int X, int Y, int bnd,
                                    int feat, int stride, cudaStream_t s);
 cudaError_t spectra_tc32_prepare(int fmt);
-cudaError_t spectra_tc32_launch(int fmt, const TwiddleTable& tw, const float* V, float* E, int T, int X, int Y,
-                                int bnd, int feat, int stride, int* err, cudaStream_t s);
+// tables: its constant operands and Eq. 1 weights, built once per handle (synchronises the stream)
+size_t spectra_tc32_tables_bytes();
+cudaError_t spectra_tc32_tables_build(int fmt, const TwiddleTable& tw, int feat, void* tables, cudaStream_t s);
+// pmax: scratch of spectra_tc32_max_bytes (the bricks' plane maxima)
+size_t spectra_tc32_max_bytes(int T, int X, int Y);
+cudaError_t spectra_tc32_launch(int fmt, const TwiddleTable& tw, const void* tables, float* pmax, const float* V,
+                                float* E, int T, int X, int Y, int bnd, int feat, int stride, int* err,
+                                cudaStream_t s);
 
 // K1 on the tensor cores (BF16 fmt = 1, FP16 fmt = 0); err: device-visible error word.  The constant
 // operands (twiddles in the operand layouts, Eq. 1 weights) are built once per handle into `tables`.

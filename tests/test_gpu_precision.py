@@ -193,6 +193,20 @@ def test_window32_forward_matches_oracle(sal, prec, tol):
         assert np.abs(g["S"] - ref["S"]).max() <= 2e-2
 
 
+# bricks of 4 x0 by 16 y0 past their edges, cubes larger than the volume, planes past its ends, both operand types
+@pytest.mark.parametrize("prec", ["bf16", "fp16"])
+@pytest.mark.parametrize("shape,boundary,taper,feature", [
+    ((2, 5, 17), "zero", "rect", "abs"), ((3, 4, 16), "periodic", "hann", "abs"), ((40, 3, 33), "symmetric", "rect", "abs"),
+    ((3, 9, 5), "symmetric", "rect", "energy"), ((1, 1, 1), "zero", "rect", "abs"),
+])
+def test_window32_tensor_core_bricks(sal, shape, boundary, taper, feature, prec):
+    V = np.random.RandomState(sum(shape)).randn(*shape).astype(np.float32)
+    g = _run(sal, V, sal.Params(n=32, prec=prec, boundary=boundary, taper=taper, feature=feature))
+    E = oracle.features(V, 32, boundary=boundary, taper=taper, feature=feature)
+    for m in range(3):
+        assert rel_l2(g["E"][m], E[m]) <= 1e-2, (m, rel_l2(g["E"][m], E[m]))
+
+
 @pytest.mark.parametrize("shape,taper", [((3, 4, 40), "rect"), ((3, 5, 19), "hann")])
 def test_window32_fp32_sliding_and_taper(sal, shape, taper):
     """FP32, 32^3 window: rows of several y bricks (ragged last one) through the sliding form, and the Hann
