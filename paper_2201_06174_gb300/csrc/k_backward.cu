@@ -11,7 +11,7 @@
 // Every output is formed by gathering, so no atomics are used and results are deterministic.
 #include <cfloat>
 
-#include "sal_internal.cuh"
+#include "reduce_tail.cuh"
 
 namespace sal {
 namespace {
@@ -19,7 +19,10 @@ namespace {
 constexpr int kThreads = 256;
 constexpr int kYChunk = 128;   // voxels of a row per warp work item of the stencil kernels
 constexpr size_t kTileSmemMax = 96 * 1024;   // plane ring of the tiled center-surround adjoint
-enum : int { N_LO = 0, N_INV = 3, N_W = 6, N_LOC = 9, N_INVC = 10 };
+using tail::N_INV;
+using tail::N_INVC;
+using tail::N_LO;
+using tail::N_W;
 
 __device__ __forceinline__ int floordiv(int a, int b) {  // b > 0
     int q = a / b;
@@ -84,10 +87,11 @@ __device__ __forceinline__ int pre_range(int q, int N, int mode, int lo, int hi,
     return c;
 }
 
-// FP64 partials of sum_p gS[p] (S_m[p] - lo_m), m = 0..2.
+// gW and the per-map coefficients coef_m = W_m invC inv_m from FP64 sums of gS[p] (S_m[p] - lo_m), m = 0..2: a partial per
+// block, reduced by the last block.
 __global__ void __launch_bounds__(kThreads)
-kb_weights_partial(const float* __restrict__ S3, const float* __restrict__ gS, long long NV,
-                   const float* __restrict__ norm, double* __restrict__ part) {
+kb_weights(const float* __restrict__ S3, const float* __restrict__ gS, long long NV, const float* __restrict__ norm,
+           double* __restrict__ part, unsigned* counter, float* __restrict__ coef, float* __restrict__ gW) {
     const float lo0 = norm[N_LO], lo1 = norm[N_LO + 1], lo2 = norm[N_LO + 2];
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
     for (long long p = (long long)blockIdx.x * kThreads + threadIdx.x; p < NV; p += (long long)gridDim.x * kThreads) {
@@ -97,39 +101,31 @@ kb_weights_partial(const float* __restrict__ S3, const float* __restrict__ gS, l
         a2 += g * (double)(__ldg(S3 + 2 * NV + p) - lo2);
     }
     __shared__ double red[3][kThreads];
+    auto tree = [&]() {
+        __syncthreads();
+        for (int s = kThreads / 2; s > 0; s >>= 1) {
+            if (threadIdx.x < s)
+                for (int c = 0; c < 3; ++c) red[c][threadIdx.x] += red[c][threadIdx.x + s];
+            __syncthreads();
+        }
+    };
     red[0][threadIdx.x] = a0;
     red[1][threadIdx.x] = a1;
     red[2][threadIdx.x] = a2;
-    __syncthreads();
-    for (int s = kThreads / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s)
-            for (int c = 0; c < 3; ++c) red[c][threadIdx.x] += red[c][threadIdx.x + s];
-        __syncthreads();
-    }
+    tree();
     if (threadIdx.x < 3) part[blockIdx.x * 64 + threadIdx.x] = red[threadIdx.x][0];
-}
-
-// gW and the per-map coefficients coef_m = W_m invC inv_m.  One block.
-__global__ void __launch_bounds__(kThreads)
-kb_weights_finalize(const double* __restrict__ part, int nparts, const float* __restrict__ norm,
-                    float* __restrict__ coef, float* __restrict__ gW) {
-    __shared__ double s[3][kThreads];
+    if (!tail::last_block(counter, tail::C_WEIGHTS)) return;
     for (int c = 0; c < 3; ++c) {
         double a = 0.0;
-        for (int i = threadIdx.x; i < nparts; i += kThreads) a += part[i * 64 + c];
-        s[c][threadIdx.x] = a;
+        for (int i = threadIdx.x; i < (int)gridDim.x; i += kThreads) a += __ldcg(part + i * 64 + c);
+        red[c][threadIdx.x] = a;
     }
-    __syncthreads();
-    for (int st = kThreads / 2; st > 0; st >>= 1) {
-        if (threadIdx.x < st)
-            for (int c = 0; c < 3; ++c) s[c][threadIdx.x] += s[c][threadIdx.x + st];
-        __syncthreads();
-    }
+    tree();
     if (threadIdx.x < 3) {
         const int m = threadIdx.x;
         const double invC = norm[N_INVC], inv = norm[N_INV + m];
         coef[m] = (float)((double)norm[N_W + m] * invC * inv);
-        if (gW) gW[m] = (float)(invC * inv * s[m][0]);
+        if (gW) gW[m] = (float)(invC * inv * red[m][0]);
     }
 }
 
@@ -205,8 +201,8 @@ k4_dcs_adjoint(const float* __restrict__ E, const float* __restrict__ gS, long l
             }
             if (row_inner && y >= hy && y < Y - hy) {
                 // the neighbour is q + o and the only preimage of q under offset o is q - o
-#pragma unroll 2
-                for (int o = 0; o < Q; ++o) {
+#pragma unroll 3
+                for (int o = 0; o < Q; ++o) {   // 27 loads in flight
                     const long long d = s_lin[o];
                     const float w = s_w[o];
 #pragma unroll
@@ -579,14 +575,17 @@ k4_gw_partial(const float* __restrict__ E, const float* __restrict__ gS, long lo
 }
 
 // galpha_d = sum_{o in d} g_o gw_o, gw_o = -(1/Q) sum_blocks part[block][o].  One block; one warp per
-// offset sums its partials in a fixed order (strided lanes, then a shuffle tree).
-__global__ void __launch_bounds__(kThreads)
+// offset sums its partials in a fixed order (strided lanes, then a shuffle tree); 32 warps, so that the offsets of the
+// usual windows are summed side by side (8 warps took 15 us for 18 offsets of a 48^3 volume).
+constexpr int kGalphaThreads = 1024;
+__global__ void __launch_bounds__(kGalphaThreads)
 k4_galpha_finalize(const double* __restrict__ part, int nparts, const __grid_constant__ Stencil st,
                    float* __restrict__ galpha) {
     __shared__ double gw[kMaxOffsets];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    for (int o = wid; o < st.Q; o += kThreads / 32) {
+    for (int o = wid; o < st.Q; o += kGalphaThreads / 32) {
         double a = 0.0;
+#pragma unroll 8
         for (int i = lane; i < nparts; i += 32) a += part[i * 64 + o];
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) a += __shfl_xor_sync(0xffffffffu, a, d);
@@ -740,10 +739,8 @@ cudaError_t expand_gradient_launch(const float* gS, const float* coef, float* gS
 
 cudaError_t backward_weights_launch(const float* S3, const float* gS, long long N, const Reduce& r, double* part,
                                     float* coef, float* gW, cudaStream_t s) {
-    const int nb = red_blocks(N);
-    kb_weights_partial<<<nb, kThreads, 0, s>>>(S3, gS, N, r.norm, part);
-    kb_weights_finalize<<<1, kThreads, 0, s>>>(part, nb, r.norm, coef, gW);
-    note_launches(2);
+    kb_weights<<<red_blocks(N), kThreads, 0, s>>>(S3, gS, N, r.norm, part, r.counter, coef, gW);
+    note_launches(1);
     return cudaGetLastError();
 }
 
@@ -795,7 +792,7 @@ cudaError_t dcs_adjoint_galpha_launch(const float* E, const float* gS, long long
     }
     k4_dcs_adjoint_tiled<true><<<(int)nblk, kThreads, smem, s>>>(E, gS, gms, coef, gE, T, X, Y, bnd, st, tile_part);
     k4_gw_tiles_sum<<<st.Q, kThreads, 0, s>>>(tile_part, nblk, st.Q, part);
-    k4_galpha_finalize<<<1, kThreads, 0, s>>>(part, 1, st, galpha);
+    k4_galpha_finalize<<<1, kGalphaThreads, 0, s>>>(part, 1, st, galpha);
     note_launches(3);
     return cudaGetLastError();
 }
@@ -805,7 +802,7 @@ cudaError_t dcs_galpha_launch(const float* E, const float* gS, long long gms, co
     const long long NV = (long long)T * X * Y;
     const int nb = red_blocks(NV);
     k4_gw_partial<<<nb, kThreads, 0, s>>>(E, gS, gms, coef, T, X, Y, bnd, st, part);
-    k4_galpha_finalize<<<1, kThreads, 0, s>>>(part, nb, st, galpha);
+    k4_galpha_finalize<<<1, kGalphaThreads, 0, s>>>(part, nb, st, galpha);
     note_launches(2);
     return cudaGetLastError();
 }

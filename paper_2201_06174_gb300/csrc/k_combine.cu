@@ -5,25 +5,27 @@
 //          G and b accumulated in FP64 (per-thread, then per-block trees, then a fixed-order
 //          sum of the block partials) and solved on the device by one thread;
 //   S    = minmax(sum_m W_m S^_m).
-// All passes are grid-stride, HBM-bound and deterministic (no floating-point atomics).
+// All passes are grid-stride, HBM-bound and deterministic (no floating-point atomics).  The reductions of a handle's
+// calls are finished by the last block of the launch that leaves the partials (reduce_tail.cuh); the allocation-free entry
+// point, whose scratch every caller shares, keeps the separate one-block launches and no state between calls.
 #include <cfloat>
 #include <cmath>
 #include <mutex>
 #include <string>
 
-#include "sal_internal.cuh"
+#include "reduce_tail.cuh"
 
 namespace sal {
 namespace {
 
-constexpr int kThreads = 256;
+constexpr int kThreads = tail::kTailThreads;
 
-enum : int { N_LO = 0, N_INV = 3, N_W = 6, N_LOC = 9, N_INVC = 10 };
-
-__device__ __forceinline__ float flat_inv(float lo, float hi) {
-    const float span = hi - lo;
-    return (span > 1e-30f * fmaxf(1.f, fabsf(hi))) ? 1.f / span : 0.f;
-}
+using tail::flat_inv;
+using tail::N_INV;
+using tail::N_INVC;
+using tail::N_LO;
+using tail::N_LOC;
+using tail::N_W;
 
 // Reduces per-block min/max partials (layout [part][8]: min at c, max at 3+c) of `nmaps`
 // maps; writes lo and 1/(hi-lo) (0 for a flat map).  One block.
@@ -56,10 +58,57 @@ k3_minmax_finalize(const float* __restrict__ mm_part, int nparts, int nmaps, flo
         }
 }
 
+// The template fit by one block: W from the Gram partials (strided threads, then a tree), into norm and W_out.
+__device__ void fit_weights(const double* g_part, int nparts, double delta, float* norm, float* W_out, double* wsum) {
+    __shared__ double s[9][kThreads];
+    for (int c = 0; c < 9; ++c) {
+        double a = 0.0;
+        for (int i = threadIdx.x; i < nparts; i += kThreads) a += __ldcg(g_part + i * 16 + c);
+        s[c][threadIdx.x] = a;
+    }
+    __syncthreads();
+    for (int st = kThreads / 2; st > 0; st >>= 1) {
+        if (threadIdx.x < st)
+            for (int c = 0; c < 9; ++c) s[c][threadIdx.x] += s[c][threadIdx.x + st];
+        __syncthreads();
+    }
+    if (threadIdx.x != 0) return;
+    double W[3];
+    double A[3][4] = {{s[0][0] + delta, s[1][0], s[2][0], s[6][0]},
+                      {s[1][0], s[3][0] + delta, s[4][0], s[7][0]},
+                      {s[2][0], s[4][0], s[5][0] + delta, s[8][0]}};
+    for (int c = 0; c < 9; ++c) wsum[c] = s[c][0];
+    // Gaussian elimination with partial pivoting.
+    for (int c = 0; c < 3; ++c) {
+        int piv = c;
+        for (int r = c + 1; r < 3; ++r)
+            if (fabs(A[r][c]) > fabs(A[piv][c])) piv = r;
+        if (piv != c)
+            for (int k = 0; k < 4; ++k) {
+                double tmp = A[c][k]; A[c][k] = A[piv][k]; A[piv][k] = tmp;
+            }
+        const double d = A[c][c];
+        for (int r = c + 1; r < 3; ++r) {
+            const double f = d != 0.0 ? A[r][c] / d : 0.0;
+            for (int k = c; k < 4; ++k) A[r][k] -= f * A[c][k];
+        }
+    }
+    for (int c = 2; c >= 0; --c) {
+        double v = A[c][3];
+        for (int k = c + 1; k < 3; ++k) v -= A[c][k] * W[k];
+        W[c] = A[c][c] != 0.0 ? v / A[c][c] : 0.0;
+    }
+    for (int m = 0; m < 3; ++m) {
+        norm[N_W + m] = (float)W[m];
+        if (W_out) W_out[m] = (float)W[m];
+    }
+}
+
 // FP64 partial Gram matrix and right-hand side of the template fit.
 __global__ void __launch_bounds__(kThreads)
-k3_gram(const float* __restrict__ S3, const float* __restrict__ D, long long NV, const float* __restrict__ norm,
-        double* __restrict__ g_part) {
+k3_gram(const float* __restrict__ S3, const float* __restrict__ D, long long NV, float* __restrict__ norm,
+        double* __restrict__ g_part, unsigned* counter, double delta, float* __restrict__ W_out,
+        double* __restrict__ wsum) {
     const float lo0 = norm[N_LO], lo1 = norm[N_LO + 1], lo2 = norm[N_LO + 2];
     const float iv0 = norm[N_INV], iv1 = norm[N_INV + 1], iv2 = norm[N_INV + 2];
     double acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
@@ -81,67 +130,25 @@ k3_gram(const float* __restrict__ S3, const float* __restrict__ D, long long NV,
         __syncthreads();
     }
     if (threadIdx.x < 9) g_part[blockIdx.x * 16 + threadIdx.x] = red[threadIdx.x][0];
+    if (counter && tail::last_block(counter, tail::C_GRAM)) fit_weights(g_part, gridDim.x, delta, norm, W_out, wsum);
 }
 
 // Chooses the weights: mode 0 equal, 1 given (W_in), 2 least squares from the Gram partials.
 __global__ void __launch_bounds__(kThreads)
 k3_weights(const double* __restrict__ g_part, int nparts, const float* __restrict__ W_in, int mode, double delta,
            float* __restrict__ norm, float* __restrict__ W_out, double* __restrict__ wsum) {
-    __shared__ double s[9][kThreads];
     if (mode == 2) {
-        for (int c = 0; c < 9; ++c) {
-            double a = 0.0;
-            for (int i = threadIdx.x; i < nparts; i += kThreads) a += g_part[i * 16 + c];
-            s[c][threadIdx.x] = a;
-        }
-        __syncthreads();
-        for (int st = kThreads / 2; st > 0; st >>= 1) {
-            if (threadIdx.x < st)
-                for (int c = 0; c < 9; ++c) s[c][threadIdx.x] += s[c][threadIdx.x + st];
-            __syncthreads();
-        }
-    }
-    if (threadIdx.x != 0) return;
-    double W[3];
-    if (mode == 0) {
-        W[0] = W[1] = W[2] = 1.0 / 3.0;
-    } else if (mode == 1) {
-        for (int m = 0; m < 3; ++m) W[m] = (double)W_in[m];
-    } else {
-        double A[3][4] = {{s[0][0] + delta, s[1][0], s[2][0], s[6][0]},
-                          {s[1][0], s[3][0] + delta, s[4][0], s[7][0]},
-                          {s[2][0], s[4][0], s[5][0] + delta, s[8][0]}};
-        for (int c = 0; c < 9; ++c) wsum[c] = s[c][0];
-        // Gaussian elimination with partial pivoting.
-        for (int c = 0; c < 3; ++c) {
-            int piv = c;
-            for (int r = c + 1; r < 3; ++r)
-                if (fabs(A[r][c]) > fabs(A[piv][c])) piv = r;
-            if (piv != c)
-                for (int k = 0; k < 4; ++k) {
-                    double tmp = A[c][k]; A[c][k] = A[piv][k]; A[piv][k] = tmp;
-                }
-            const double d = A[c][c];
-            for (int r = c + 1; r < 3; ++r) {
-                const double f = d != 0.0 ? A[r][c] / d : 0.0;
-                for (int k = c; k < 4; ++k) A[r][k] -= f * A[c][k];
-            }
-        }
-        for (int c = 2; c >= 0; --c) {
-            double v = A[c][3];
-            for (int k = c + 1; k < 3; ++k) v -= A[c][k] * W[k];
-            W[c] = A[c][c] != 0.0 ? v / A[c][c] : 0.0;
-        }
-    }
-    for (int m = 0; m < 3; ++m) {
-        norm[N_W + m] = (float)W[m];
-        if (W_out) W_out[m] = (float)W[m];
+        fit_weights(g_part, nparts, delta, norm, W_out, wsum);
+    } else if (threadIdx.x < 3) {
+        const float w = mode == 0 ? (float)(1.0 / 3.0) : W_in[threadIdx.x];
+        norm[N_W + threadIdx.x] = w;
+        if (W_out) W_out[threadIdx.x] = w;
     }
 }
 
 __global__ void __launch_bounds__(kThreads)
-k3_combine(const float* __restrict__ S3, long long NV, const float* __restrict__ norm, float* __restrict__ S,
-           float* __restrict__ mm_part) {
+k3_combine(const float* __restrict__ S3, long long NV, float* __restrict__ norm, float* __restrict__ S,
+           float* __restrict__ mm_part, unsigned* counter) {   // S null: only the bounds of the combination
     const float lo0 = norm[N_LO], lo1 = norm[N_LO + 1], lo2 = norm[N_LO + 2];
     const float a0 = norm[N_INV] * norm[N_W], a1 = norm[N_INV + 1] * norm[N_W + 1], a2 = norm[N_INV + 2] * norm[N_W + 2];
     float mn = FLT_MAX, mx = -FLT_MAX;
@@ -149,7 +156,7 @@ k3_combine(const float* __restrict__ S3, long long NV, const float* __restrict__
         float c = (__ldg(S3 + p) - lo0) * a0;
         c = fmaf(__ldg(S3 + NV + p) - lo1, a1, c);
         c = fmaf(__ldg(S3 + 2 * NV + p) - lo2, a2, c);
-        S[p] = c;
+        if (S) S[p] = c;
         mn = fminf(mn, c);
         mx = fmaxf(mx, c);
     }
@@ -168,11 +175,12 @@ k3_combine(const float* __restrict__ S3, long long NV, const float* __restrict__
         mm_part[blockIdx.x * 8] = smin[0];
         mm_part[blockIdx.x * 8 + 3] = smax[0];
     }
+    if (counter && tail::last_block(counter, tail::C_COMBINE)) tail::minmax<1>(mm_part, gridDim.x, norm + N_LOC, norm + N_INVC);
 }
 
 // Per-block min/max partials of the three S_m planes (used when S3 did not come from K2).
 __global__ void __launch_bounds__(kThreads)
-k3_minmax3(const float* __restrict__ S3, long long NV, float* __restrict__ mm_part) {
+k3_minmax3(const float* __restrict__ S3, long long NV, float* __restrict__ mm_part, const MapTail tl) {
     float mn[3] = {FLT_MAX, FLT_MAX, FLT_MAX}, mx[3] = {-FLT_MAX, -FLT_MAX, -FLT_MAX};
     for (long long p = (long long)blockIdx.x * kThreads + threadIdx.x; p < NV; p += (long long)gridDim.x * kThreads)
 #pragma unroll
@@ -199,6 +207,7 @@ k3_minmax3(const float* __restrict__ S3, long long NV, float* __restrict__ mm_pa
         mm_part[blockIdx.x * 8 + threadIdx.x] = smin[threadIdx.x][0];
         mm_part[blockIdx.x * 8 + 3 + threadIdx.x] = smax[threadIdx.x][0];
     }
+    if (tl.counter && tail::last_block(tl.counter, tail::C_MAPS)) tail::bounds_and_weights(mm_part, tl);
 }
 
 __global__ void __launch_bounds__(kThreads)
@@ -215,27 +224,27 @@ int red_blocks(long long NV) {
     return (int)(b < kRedBlocks ? b : kRedBlocks);
 }
 
+MapTail map_tail(const Reduce& r, const float* D, const float* W_in, float* W_out) {
+    return MapTail{r.counter, r.norm, D ? 2 : (W_in ? 1 : 0), W_in, W_out};
+}
+
 cudaError_t minmax_bounds_launch(const float* S3, long long N, const Reduce& r, cudaStream_t s) {
-    const int nb = red_blocks(N);
-    k3_minmax3<<<nb, kThreads, 0, s>>>(S3, N, r.mm_part);
-    k3_minmax_finalize<<<1, kThreads, 0, s>>>(r.mm_part, nb, 3, r.norm + N_LO, r.norm + N_INV);
-    note_launches(2);
+    MapTail t = map_tail(r, nullptr, nullptr, nullptr);
+    t.mode = 2;   // no weights
+    k3_minmax3<<<red_blocks(N), kThreads, 0, s>>>(S3, N, r.mm_part, t);
+    note_launches(1);
     return cudaGetLastError();
 }
 
 cudaError_t combine_launch(const float* S3, const float* D, const float* W_in, float* W_out, float* S,
-                           long long N, double delta, bool s3_partials_ready, const Reduce& r, cudaStream_t s) {
+                           long long N, double delta, bool bounds_ready, const Reduce& r, cudaStream_t s) {
     const int nb = red_blocks(N);
-    // min/max partials of S3: written by K2 (same block count) when it produced S3
-    if (!s3_partials_ready) k3_minmax3<<<nb, kThreads, 0, s>>>(S3, N, r.mm_part);
-    k3_minmax_finalize<<<1, kThreads, 0, s>>>(r.mm_part, nb, 3, r.norm + N_LO, r.norm + N_INV);
-    int mode = D ? 2 : (W_in ? 1 : 0);
-    if (mode == 2) k3_gram<<<nb, kThreads, 0, s>>>(S3, D, N, r.norm, r.g_part);
-    k3_weights<<<1, kThreads, 0, s>>>(r.g_part, nb, W_in, mode, delta, r.norm, W_out, r.wsum);
-    k3_combine<<<nb, kThreads, 0, s>>>(S3, N, r.norm, S, r.mm_part);
-    k3_minmax_finalize<<<1, kThreads, 0, s>>>(r.mm_part, nb, 1, r.norm + N_LOC, r.norm + N_INVC);
-    k3_normalize<<<nb, kThreads, 0, s>>>(S, N, r.norm);
-    note_launches(5 + (s3_partials_ready ? 0 : 1) + (mode == 2 ? 1 : 0));
+    // bounds of S3: left by K2's last block when it produced S3
+    if (!bounds_ready) k3_minmax3<<<nb, kThreads, 0, s>>>(S3, N, r.mm_part, map_tail(r, D, W_in, W_out));
+    if (D) k3_gram<<<nb, kThreads, 0, s>>>(S3, D, N, r.norm, r.g_part, r.counter, delta, W_out, r.wsum);
+    k3_combine<<<nb, kThreads, 0, s>>>(S3, N, r.norm, S, r.mm_part, r.counter);
+    if (S) k3_normalize<<<nb, kThreads, 0, s>>>(S, N, r.norm);
+    note_launches(1 + (S ? 1 : 0) + (bounds_ready ? 0 : 1) + (D ? 1 : 0));
     return cudaGetLastError();
 }
 
@@ -344,12 +353,12 @@ extern "C" sal_status sal_combine_noalloc(int T, int X, int Y, const float* S3, 
     // of a previous call need no clearing.
     const int nb = (int)((N + kNoAllocVoxPerBlock - 1) / kNoAllocVoxPerBlock);
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    sal::k3_minmax3<<<nb, sal::kThreads, 0, s>>>(S3, N, r.mm_part);
+    sal::k3_minmax3<<<nb, sal::kThreads, 0, s>>>(S3, N, r.mm_part, sal::MapTail{});
     sal::k3_minmax_finalize<<<1, sal::kThreads, 0, s>>>(r.mm_part, nb, 3, r.norm + sal::N_LO, r.norm + sal::N_INV);
     const int mode = D ? 2 : (W_in ? 1 : 0);
-    if (mode == 2) sal::k3_gram<<<nb, sal::kThreads, 0, s>>>(S3, D, N, r.norm, r.g_part);
+    if (mode == 2) sal::k3_gram<<<nb, sal::kThreads, 0, s>>>(S3, D, N, r.norm, r.g_part, nullptr, 0.0, nullptr, nullptr);
     sal::k3_weights<<<1, sal::kThreads, 0, s>>>(r.g_part, nb, W_in, mode, ls_delta, r.norm, W_out, r.wsum);
-    sal::k3_combine<<<nb, sal::kThreads, 0, s>>>(S3, N, r.norm, S, r.mm_part);
+    sal::k3_combine<<<nb, sal::kThreads, 0, s>>>(S3, N, r.norm, S, r.mm_part, nullptr);
     sal::k3_minmax_finalize<<<1, sal::kThreads, 0, s>>>(r.mm_part, nb, 1, r.norm + sal::N_LOC, r.norm + sal::N_INVC);
     sal::k3_normalize<<<nb, sal::kThreads, 0, s>>>(S, N, r.norm);
     sal::note_launches(6 + (mode == 2 ? 1 : 0));

@@ -11,12 +11,13 @@
 #include <algorithm>
 #include <cfloat>
 
-#include "sal_internal.cuh"
+#include "reduce_tail.cuh"
 
 namespace sal {
 namespace {
 
 constexpr int kThreads = 256;
+static_assert(kThreads == tail::kTailThreads, "the tails' block");
 constexpr int kYChunk = 128;   // voxels of a row per warp work item
 
 __device__ __forceinline__ float warp_min(float v) {
@@ -32,7 +33,7 @@ __device__ __forceinline__ float warp_max(float v) {
 
 __global__ void __launch_bounds__(kThreads)
 k2_dcs(const float* __restrict__ E, float* __restrict__ S3, int T, int X, int Y, int bnd,
-       const __grid_constant__ Stencil st, float* __restrict__ mm_part) {
+       const __grid_constant__ Stencil st, float* __restrict__ mm_part, const MapTail tl) {
     constexpr int kWarps = kThreads / 32;
     const long long NV = (long long)T * X * Y;
     // linear offset of each neighbour: the whole comparison of a voxel at least the halo away from every
@@ -62,8 +63,8 @@ k2_dcs(const float* __restrict__ E, float* __restrict__ S3, int T, int X, int Y,
 #pragma unroll
             for (int m = 0; m < 3; ++m) ec[m] = __ldg(E + m * NV + p);
             if (row_inner && y >= hy && y < Y - hy) {
-#pragma unroll 2
-                for (int o = 0; o < Q; ++o) {
+#pragma unroll 6
+                for (int o = 0; o < Q; ++o) {   // 18 loads in flight
                     const float* e = E + p + s_lin[o];
                     const float w = s_w[o];
 #pragma unroll
@@ -76,6 +77,7 @@ k2_dcs(const float* __restrict__ E, float* __restrict__ S3, int T, int X, int Y,
                     }
                 }
             } else {
+#pragma unroll 3
                 for (int o = 0; o < Q; ++o) {
                     const int tt = ext_index(t + st.off[o][0], T, bnd);
                     const int xx = ext_index(x + st.off[o][1], X, bnd);
@@ -118,6 +120,7 @@ k2_dcs(const float* __restrict__ E, float* __restrict__ S3, int T, int X, int Y,
         for (int w = 1; w < kThreads / 32; ++w) v = c < 3 ? fminf(v, red[w][c]) : fmaxf(v, red[w][c]);
         mm_part[blockIdx.x * 8 + c] = v;
     }
+    if (tl.counter && tail::last_block(tl.counter, tail::C_MAPS)) tail::bounds_and_weights(mm_part, tl);
 }
 
 // K2, ring-staged: the same sums, with E read from global memory about once per tile.  A tile is 16 x 16
@@ -126,7 +129,7 @@ k2_dcs(const float* __restrict__ E, float* __restrict__ S3, int T, int X, int Y,
 // at the border or not, reads its neighbours ext(p + o) from the ring in the order of the offsets (the
 // result is that of k2_dcs bit for bit).  The next plane is fetched into registers while the current one
 // is computed.  Blocks are persistent over the tiles (as many as fit on the GPU at once); each keeps the
-// min/max of its outputs, and partial slots beyond the grid get neutral values (K3 reads a fixed count).
+// min/max of its outputs.
 constexpr int kTX = 16, kTY = 16, kTT = 16;
 constexpr int kPre = 2;   // plane elements per thread prefetched into registers (the rest loaded at store)
 static_assert(kTX * kTY == kThreads, "one column per thread");
@@ -137,7 +140,7 @@ __host__ __device__ inline size_t ring_bytes(int ht, int hx, int hy) {
 
 __global__ void __launch_bounds__(kThreads)
 k2_dcs_tiled(const float* __restrict__ E, float* __restrict__ S3, int T, int X, int Y, int bnd,
-             const __grid_constant__ Stencil st, float* __restrict__ mm_part, int nparts) {
+             const __grid_constant__ Stencil st, float* __restrict__ mm_part, const MapTail tl) {
     extern __shared__ float s_ring[];   // [2 h_t + 1][3][TXH][TYH]
     __shared__ float s_w[kMaxOffsets];
     __shared__ int s_d[kMaxOffsets][3];
@@ -258,10 +261,7 @@ k2_dcs_tiled(const float* __restrict__ E, float* __restrict__ S3, int T, int X, 
         for (int w = 1; w < kThreads / 32; ++w) v = c < 3 ? fminf(v, red[w][c]) : fmaxf(v, red[w][c]);
         mm_part[blockIdx.x * 8 + c] = v;
     }
-    // the slots of the partials no block of this grid fills: neutral (min +inf-like, max -inf-like)
-    if (blockIdx.x == 0)
-        for (int i = gridDim.x * 8 + threadIdx.x; i < nparts * 8; i += kThreads)
-            mm_part[i] = (i % 8) < 3 ? FLT_MAX : -FLT_MAX;
+    if (tl.counter && tail::last_block(tl.counter, tail::C_MAPS)) tail::bounds_and_weights(mm_part, tl);
 }
 
 constexpr size_t kRingMax = 96 * 1024;   // windows whose ring is larger take the row kernel
@@ -273,9 +273,9 @@ cudaError_t dcs_prepare() {
 }
 
 cudaError_t dcs_launch(const float* E, float* S3, int T, int X, int Y, int bnd, const Stencil& st,
-                       float* mm_part, cudaStream_t s) {
+                       float* mm_part, const MapTail& tl, cudaStream_t s) {
     const long long NV = (long long)T * X * Y;
-    const int nparts = red_blocks(NV);  // K3 reduces exactly this many min/max partials
+    const int nparts = red_blocks(NV);
     const size_t smem = ring_bytes(st.halo[0], st.halo[1], st.halo[2]);
     int per_sm = 0;
     if (smem <= kRingMax) {
@@ -288,11 +288,11 @@ cudaError_t dcs_launch(const float* E, float* S3, int T, int X, int Y, int bnd, 
     // SMs idle, and the row kernel, whose warps cover every row, is faster
     if (smem <= kRingMax && per_sm > 0 && ntiles >= wave) {
         long long grid = std::min<long long>(wave, nparts);
-        k2_dcs_tiled<<<(int)grid, kThreads, smem, s>>>(E, S3, T, X, Y, bnd, st, mm_part, nparts);
+        k2_dcs_tiled<<<(int)grid, kThreads, smem, s>>>(E, S3, T, X, Y, bnd, st, mm_part, tl);
         note_launches(1);
         return cudaGetLastError();
     }
-    k2_dcs<<<nparts, kThreads, 0, s>>>(E, S3, T, X, Y, bnd, st, mm_part);
+    k2_dcs<<<nparts, kThreads, 0, s>>>(E, S3, T, X, Y, bnd, st, mm_part, tl);
     note_launches(1);
     return cudaGetLastError();
 }

@@ -343,7 +343,7 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
 
     const size_t plane3 = (size_t)3 * h->N * sizeof(float);
     const size_t small = (size_t)sal::kRedBlocks * 8 * sizeof(float) + (size_t)sal::kRedBlocks * 16 * sizeof(double)
-                         + 32 * sizeof(float) + 16 * sizeof(double) + 256;
+                         + 32 * sizeof(float) + 16 * sizeof(double) + 256;   // (the block counters in the last)
     const bool tc_fwd = h->prec != SAL_FP32 && sal::spectra_tc_supported(h->n);
     const bool tc32 = h->prec != SAL_FP32 && h->n == 32;
     const size_t tab_bytes = tc_fwd ? sal::spectra_tc_tables_bytes(h->n) : tc32 ? sal::spectra_tc32_tables_bytes() : 0;
@@ -395,9 +395,10 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
     h->red.mm_part = reinterpret_cast<float*>(b);
     b += (size_t)sal::kRedBlocks * 8 * sizeof(float);
     h->red.norm = reinterpret_cast<float*>(b);
+    h->red.counter = reinterpret_cast<unsigned*>(b + 32 * sizeof(float));
     {
         // norm layout: [0..10] bounds and weights, [12..14] gradient coefficients, [16..18] ones
-        float init[32] = {0.f};
+        float init[36] = {0.f};   // and the four counters, 0
         init[16] = init[17] = init[18] = 1.f;
         if ((e = cudaMemcpy(h->red.norm, init, sizeof(init), cudaMemcpyHostToDevice)) != cudaSuccess) {
             free_scratch(h);
@@ -519,7 +520,7 @@ sal_status sal_center_surround(sal_handle* h, const float* E, float* S3, void* s
     sal_status s = check_handle(h);
     if (s != SAL_OK) return s;
     if (!E || !S3) return fail(h, SAL_ERR_INVALID_ARG, "E and S3 must not be NULL");
-    cudaError_t e = sal::dcs_launch(E, S3, h->T, h->X, h->Y, h->boundary, h->st, h->red.mm_part,
+    cudaError_t e = sal::dcs_launch(E, S3, h->T, h->X, h->Y, h->boundary, h->st, h->red.mm_part, sal::MapTail{},
                                     static_cast<cudaStream_t>(stream));
     return e == cudaSuccess ? SAL_OK : cuda_fail(h, e, "center_surround launch");
 }
@@ -544,7 +545,8 @@ sal_status sal_saliency(sal_handle* h, const float* V, const float* D, const flo
     float* S3 = S3_opt ? S3_opt : h->S3;
     cudaError_t e = launch_k1(h, V, E, st);
     if (e != cudaSuccess) return cuda_fail(h, e, "local_spectra_project launch");
-    e = sal::dcs_launch(E, S3, h->T, h->X, h->Y, h->boundary, h->st, h->red.mm_part, st);
+    e = sal::dcs_launch(E, S3, h->T, h->X, h->Y, h->boundary, h->st, h->red.mm_part,
+                        sal::map_tail(h->red, D, W_in, W_out), st);
     if (e != cudaSuccess) return cuda_fail(h, e, "center_surround launch");
     e = sal::combine_launch(S3, D, W_in, W_out, S, h->N, h->ls_delta, true, h->red, st);
     return e == cudaSuccess ? SAL_OK : cuda_fail(h, e, "combine launch");
@@ -687,10 +689,11 @@ sal_status sal_saliency_backward(sal_handle* h, const float* V, const float* W, 
     cudaError_t e;
     // forward recompute: features, raw maps, normalisation bounds for the given weights
     if ((e = launch_k1(h, V, h->E, st)) != cudaSuccess) return cuda_fail(h, e, "backward: local_spectra_project");
-    if ((e = sal::dcs_launch(h->E, h->S3, h->T, h->X, h->Y, h->boundary, h->st, h->red.mm_part, st)) != cudaSuccess)
+    if ((e = sal::dcs_launch(h->E, h->S3, h->T, h->X, h->Y, h->boundary, h->st, h->red.mm_part,
+                             sal::map_tail(h->red, nullptr, W, nullptr), st)) != cudaSuccess)
         return cuda_fail(h, e, "backward: center_surround");
-    // the combined map itself is not needed: gE's first plane holds it until K4 overwrites it
-    if ((e = sal::combine_launch(h->S3, nullptr, W, nullptr, h->gE, h->N, h->ls_delta, true, h->red, st)) !=
+    // the combined map itself is not needed, only its bounds
+    if ((e = sal::combine_launch(h->S3, nullptr, W, nullptr, nullptr, h->N, h->ls_delta, true, h->red, st)) !=
         cudaSuccess)
         return cuda_fail(h, e, "backward: combine");
     float* coef = h->red.norm + 12;
@@ -778,8 +781,8 @@ sal_status sal_combine_backward(sal_handle* h, const float* S3, const float* W, 
     if ((s = ensure_backward_scratch(h)) != SAL_OK) return s;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     cudaError_t e;
-    // bounds of the forward combination; its map goes to gS3's first plane until overwritten
-    if ((e = sal::combine_launch(S3, nullptr, W, nullptr, gS3, h->N, h->ls_delta, false, h->red, st)) != cudaSuccess)
+    // bounds of the forward combination
+    if ((e = sal::combine_launch(S3, nullptr, W, nullptr, nullptr, h->N, h->ls_delta, false, h->red, st)) != cudaSuccess)
         return cuda_fail(h, e, "combine_backward: bounds");
     float* coef = h->red.norm + 12;
     if ((e = sal::backward_weights_launch(S3, gS, h->N, h->red, h->bpart, coef, gW, st)) != cudaSuccess)

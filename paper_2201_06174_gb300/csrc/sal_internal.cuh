@@ -59,6 +59,17 @@ struct Reduce {
     double* g_part;     // [kRedBlocks][16] per-block FP64 partial sums
     float* norm;        // [16]: lo[3], inv[3], W[3], loC, invC, flags
     double* wsum;       // [16]: reduced FP64 sums (Gram, gradient of W)
+    unsigned* counter;  // [4]: blocks of a launch that are done, by kernel (reduce_tail.cuh); null: no fused tails
+};
+
+// What the last block of a launch that leaves min/max partials of the three maps finishes: their bounds, and the weights
+// of mode 0 (equal) or 1 (given).  counter null: nothing.
+struct MapTail {
+    unsigned* counter;
+    float* norm;
+    int mode;
+    const float* W_in;
+    float* W_out;
 };
 
 // ---- K1: local spectra + projection + features ----------------------------------------------
@@ -134,12 +145,15 @@ cudaError_t adapt_launch(const float* S3, const float* D, int T, int X, int Y, i
 // Once per device: the shared-memory size limit of the ring-staged K2 (windows whose ring fits 96 KB).
 cudaError_t dcs_prepare();
 cudaError_t dcs_launch(const float* E, float* S3, int T, int X, int Y, int bnd, const Stencil& st,
-                       float* mm_part, cudaStream_t s);
+                       float* mm_part, const MapTail& tail, cudaStream_t s);
 
 // ---- K3: normalisation + combination ----------------------------------------------------------
 int red_blocks(long long NV);  // grid of the grid-stride reduction kernels (<= kRedBlocks)
+MapTail map_tail(const Reduce& r, const float* D, const float* W_in, float* W_out);
+// The combination, its bounds left in r.norm.  bounds_ready: the launch that produced S3 had the map_tail of the same D,
+// W_in and W_out; S null: only the bounds are wanted.
 cudaError_t combine_launch(const float* S3, const float* D, const float* W_in, float* W_out, float* S,
-                           long long N, double delta, bool s3_partials_ready, const Reduce& r, cudaStream_t s);
+                           long long N, double delta, bool bounds_ready, const Reduce& r, cudaStream_t s);
 
 // ---- K4/K5 and the backward reductions ---------------------------------------------------------
 // Brick of the spectral adjoint: outputs x0 in [xs*BX, xs*BX+BX), y0 in [ys*BY, ys*BY+BY) at one t0;
