@@ -18,7 +18,8 @@ from . import sal as _sal
 class SaliencyFunction(torch.autograd.Function):
     @staticmethod
     def forward(ctx, V, W, alpha, engine):
-        engine.set_alpha(alpha.detach().cpu().numpy())
+        ctx.host_alpha = alpha.detach().cpu().numpy().copy()   # the backward sets it again without another device read
+        engine.set_alpha(ctx.host_alpha)
         S = torch.empty(engine.shape, dtype=torch.float32, device=engine.device)
         E = torch.empty((3,) + tuple(engine.shape), dtype=torch.float32, device=engine.device)
         S3 = torch.empty_like(E)
@@ -31,13 +32,15 @@ class SaliencyFunction(torch.autograd.Function):
     def backward(ctx, gS):
         V, W, alpha, E, S3 = ctx.saved_tensors
         eng = ctx.engine
-        eng.set_alpha(alpha.detach().cpu().numpy())
+        eng.set_alpha(ctx.host_alpha)
         gW = torch.empty(3, dtype=torch.float32, device=V.device)
-        galpha = torch.empty_like(alpha)
+        galpha = torch.empty_like(alpha) if ctx.needs_input_grad[2] else None
         gS3 = torch.empty_like(S3)
         _sal.sal_combine_backward(eng.h, S3, W.contiguous(), gS.contiguous(), gS3, gW)
-        gE = torch.empty_like(E)
-        _sal.sal_center_surround_backward(eng.h, E, gS3, gE, galpha)
+        # the features' gradient is only wanted on its way to the volume's
+        gE = torch.empty_like(E) if ctx.needs_input_grad[0] else None
+        if gE is not None or galpha is not None:
+            _sal.sal_center_surround_backward(eng.h, E, gS3, gE, galpha)
         gV = None
         if ctx.needs_input_grad[0]:
             gV = torch.empty_like(V)

@@ -415,3 +415,28 @@ def test_autograd_matches_abi_and_descends(sal):
         assert float(loss1) < float(loss0)
     finally:
         eng.close()
+
+
+@pytest.mark.parametrize("wanted", [(True, False, False), (False, True, False), (False, False, True), (True, False, True)])
+def test_autograd_of_some_inputs_matches_that_of_all(wanted):
+    """What a caller does not differentiate by is not computed, and the rest is the same: the FP64 sums of the alpha
+    gradient are taken in another order without the features' gradient, and rounded once to FP32."""
+    import torch
+    from paper_2201_06174_gb300 import autograd as sal_autograd, sal as capi
+    shape = (11, 9, 14)
+    g = torch.Generator().manual_seed(3)
+    V, gS = (torch.randn(shape, generator=g).cuda() for _ in range(2))
+    W, alpha = torch.tensor([0.2, 0.5, 0.4]).cuda(), torch.tensor([1.0, 0.9, 1.1]).cuda()
+    eng = capi.Saliency(shape, capi.Params(n=8, directions=((1, 0, 0), (0, 1, 0), (1, 1, 0))))
+    try:
+        def grads(need):
+            x = [t.clone().requires_grad_(r) for t, r in zip((V, W, alpha), need)]
+            eng.set_alpha([3.0, 3.0, 3.0])   # not the one of this call
+            S = sal_autograd.saliency(*x, eng)
+            eng.set_alpha([2.0, 2.0, 2.0])   # nor in its backward
+            return torch.autograd.grad(S, [t for t, r in zip(x, need) if r], gS)
+        full = grads((True, True, True))
+        for got, want in zip(grads(wanted), [f for f, r in zip(full, wanted) if r]):
+            assert torch.allclose(got, want, rtol=2.0 ** -22, atol=0)
+    finally:
+        eng.close()
