@@ -8,6 +8,8 @@
 // run the epilogue.  Two 128-column accumulator buffers alternate; producer and consumers meet only on
 // mbarriers (buffer full: MMA commit; buffer empty and stage-3 A written: one arrival per consumer
 // warp), so the tensor core runs up to two passes ahead and no CTA-wide barrier sits in the k_t loop.
+// A pass's stage-3 products are one N = 128 MMA per part and 16 K rows instead of two N = 2 n ones per output: whole call
+// at n = 8 on 256 x 384 x 192, 5018 -> 4742 us (16 MMAs a pass became 2); at n = 16 on 128^3 2414 -> 2385 us (8 became 4).
 // Every wait is bounded; on timeout the CTA sets the error word, stops issuing and leaves after
 // releasing its tensor memory.
 #include "tc_spectra_common.cuh"
@@ -26,11 +28,15 @@ constexpr int kConsumers = 8;           // consumer warps: 2 per tensor-memory l
 constexpr int kThreads = 32 * (kConsumers + 1);   // + one producer warp
 constexpr uint32_t kTmemCols = 256;     // two 128-column accumulator buffers
 
-template <int N> struct TcGeo : tcs::FwdGeo<N> {
-    using F = tcs::FwdGeo<N>;
+template <int N> struct TcGeo : tcs::FwdGeo<N, true> {
+    using F = tcs::FwdGeo<N, true>;
     static constexpr size_t OFF_TAB = F::R0_B;
     static constexpr size_t OFF_A3 = OFF_TAB + F::TAB_B;
-    static constexpr size_t OFF_MISC = OFF_A3 + 2 * F::A3_B;
+    // the wide stage-3 windows of a group of 8 rows run past its kKRows rows into the next group (finite, times zero); those
+    // of the last group into a pad of zeros
+    static constexpr int OVER = kBY - F::OPP + F::K3 - tcs::kKRows;
+    static constexpr size_t PAD_B = OVER > 0 ? (size_t)OVER * 16 : 0;
+    static constexpr size_t OFF_MISC = OFF_A3 + 2 * F::A3_B + PAD_B;
     static constexpr size_t SMEM = OFF_MISC + 80 + 16 * 4;
     static_assert(F::NB1 * 16 <= (int)kTmemCols, "tensor memory");
     static_assert(F::PASSES * F::OPC * 2 == 8, "accumulator slots");
@@ -39,7 +45,7 @@ template <int N> struct TcGeo : tcs::FwdGeo<N> {
 
 template <int N, int FMT>
 __global__ void k1_tc_tables(const __grid_constant__ Tw<N> tw, unsigned char* __restrict__ out, int feat) {
-    tcs::build_fwd_tables<N, FMT>(tw, out, threadIdx.x, blockDim.x, feat);
+    tcs::build_fwd_tables<N, FMT, true>(tw, out, threadIdx.x, blockDim.x, feat);
 }
 
 // EN: the energy reading of the feature (|F|^2 per bin; the weight table then holds r_m^2)
@@ -90,14 +96,15 @@ k1_spectra_tc(const float* __restrict__ V, float* __restrict__ E, int T, int X, 
     if (tma && warp == 0)
         tcs::stage_issue<N>(smode, &tmap, V, X, Y, t0, xb, yb, smem + G::STG_OFF, tc::smem_u32(&s_mbar[7]), lane);
     // stage-3 A rows beyond the halo (read by the last windows, multiplied by zero twiddles) stay zero
-    for (int i = tid; i < (int)(2 * G::A3_B / 16); i += kThreads)
+    for (int i = tid; i < (int)((2 * G::A3_B + G::PAD_B) / 16); i += kThreads)
         reinterpret_cast<uint4*>(s_are)[i] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();   // mbarriers initialised before anyone waits on them
 
     // ---- the halo brick as the 16-bit stage-1 A operand ----------------------------------------------
+    bool nonfinite;
     const float scale = tcs::stage_brick<N, FMT, kThreads>(V, T, X, Y, bnd, t0, xb, yb, s_a1, s_red, tid, tma,
                                                            smem + G::STG_OFF, smode, tc::smem_u32(&s_mbar[7]), err,
-                                                           s_fail);
+                                                           s_fail, &nonfinite);
     tc::fence_async_smem();
     tc::fence_before_sync();
     __syncthreads();
@@ -117,11 +124,12 @@ k1_spectra_tc(const float* __restrict__ V, float* __restrict__ E, int T, int X, 
         {
             const uint32_t idesc1 = tc::idesc_f16(FMT, 128, 16, 1, 0);
             const uint32_t idesc2 = tc::idesc_f16(FMT, 128, G::N2, 0, 0);
-            const uint32_t idesc3 = tc::idesc_f16(FMT, 128, G::N3, 1, 0);
+            const uint32_t idesc3 = tc::idesc_f16(FMT, 128, G::N3, 1, 0);     // one output
+            const uint32_t idesc3w = tc::idesc_f16(FMT, 128, G::W3, 1, 0);    // a pass
             const uint32_t tab = tc::smem_u32(s_tab), b2base = tc::smem_u32(s_b2);
             const uint32_t are = tc::smem_u32(s_are), aim = tc::smem_u32(s_aim);
-            const uint64_t b3a = tc::desc_noswizzle(tab + (uint32_t)G::TAB_B3A, 128, 256);
-            const uint64_t b3b = tc::desc_noswizzle(tab + (uint32_t)G::TAB_B3B, 128, 256);
+            const uint64_t b3a = tc::desc_noswizzle(tab + (uint32_t)G::TAB_B3A, 128, G::SBO_B3);
+            const uint64_t b3b = tc::desc_noswizzle(tab + (uint32_t)G::TAB_B3B, 128, G::SBO_B3);
             // warp-uniform bounded wait; a give-up (here or in a consumer) stops all further issue
             auto pwait = [&](int b, uint32_t parity) -> bool {
                 bool ok = !*v_fail && tc::mbar_wait(tc::smem_u32(&s_mbar[b]), parity, kWaitLimit);
@@ -148,8 +156,19 @@ k1_spectra_tc(const float* __restrict__ V, float* __restrict__ E, int T, int X, 
             };
             auto issue_s3 = [&](int pass) {
                 const uint32_t col = (uint32_t)(128 * (pass & 1));
-                if (tc::elect_one()) {
+                if (!nonfinite) {
+                    if (tc::elect_one()) {
 #pragma unroll
+                        for (int k = 0; k < 2 * (G::K3 / 16); ++k) {   // real part, then imaginary
+                            const uint32_t st = k % (G::K3 / 16) * 256;
+                            const bool im = k >= G::K3 / 16;
+                            tc::mma_f16(tmem + col, tc::desc_add(im ? aimd : ared, pass * G::OPP * 16 + st),
+                                        tc::desc_add(im ? b3b : b3a, st), idesc3w, k > 0 ? 1u : 0u);
+                        }
+                        tc::mma_commit(tc::smem_u32(&s_mbar[pass & 1]));
+                    }
+                } else if (tc::elect_one()) {
+#pragma unroll 1
                     for (int j = 0; j < G::OPP; ++j) {
                         const uint32_t y0 = pass * G::OPP + j;
                         tc::mma_f16(tmem + col + j * G::N3, tc::desc_add(ared, y0 * 16), b3a, idesc3, 0);

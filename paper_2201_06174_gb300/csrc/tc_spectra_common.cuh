@@ -17,6 +17,11 @@
 //            descriptor moved by 16 y0 bytes.
 //   stage 3 (y), per output y0:  D3[(x0, k_x)][(re|im, k_y)] = Are(y0) B3a + Aim(y0) B3b,
 //            B3a = [c | -s], B3b = [s | c] over all k_y: the accumulator holds Re F and Im F.
+//            Wide form (K1-TC): one MMA takes all outputs of a pass, N = 128, with B3a and B3b repeated for
+//            output j at K rows moved by j (zero elsewhere; K = 16, or 32 where n + outputs - 1 > 16): an MMA's
+//            cost is its issue up to N = 64 and hardly more at 128, and a pass takes 2 or 4 of them instead of
+//            16 or 8.  The zero rows read rows of other windows, so a brick with a NaN or an infinity keeps the
+//            narrow form, whose window is the 16 rows from its own first (output 0's block of the same B3).
 #pragma once
 
 #include <cuda.h>
@@ -38,7 +43,7 @@ constexpr int kXHP = 24;                // halo rows along x staged (>= P + n - 
 constexpr int kK2 = 2 * kXHP;           // stage-2 K: 24 cos taps + 24 sin taps
 constexpr uint32_t kWaitLimit = 1u << 22;
 
-template <int N> struct FwdGeo {
+template <int N, bool WIDE = false> struct FwdGeo {
     static constexpr int H = N / 2 + 1;
     static constexpr int P = 128 / N;          // x0 positions per CTA
     static constexpr int XH = P + N - 1;       // x extent of the halo
@@ -59,7 +64,10 @@ template <int N> struct FwdGeo {
     static constexpr size_t R0_B = ((A1_B > B2ALL_B ? A1_B : B2ALL_B) + 127) / 128 * 128;  // A1, then B2 tiles
     // forward constant operands: [A2 | B1 | B3a | B3b | Eq. 1 weight table]
     static constexpr size_t A2_B = (size_t)16 * SBO_K2;
-    static constexpr size_t B3_B = (size_t)N3 / 8 * 256;
+    static constexpr int W3 = WIDE ? 128 : N3;                         // stage-3 N of one MMA
+    static constexpr int K3 = WIDE && N + OPP - 1 > 16 ? 32 : 16;       // its K rows
+    static constexpr uint32_t SBO_B3 = K3 / 8 * 128;
+    static constexpr size_t B3_B = (size_t)W3 / 8 * SBO_B3;
     static constexpr size_t WT_B = ((size_t)H * H * H * 3 * 4 + 15) / 16 * 16;
     static constexpr size_t TAB_B1 = A2_B;
     static constexpr size_t TAB_B3A = TAB_B1 + 512;
@@ -126,9 +134,9 @@ template <int N> __device__ __forceinline__ float tws(const Tw<N>& tw, int k, in
 // stage-2 twiddles, K-major), B1 (stage-1 twiddles), B3a / B3b (stage-3 twiddles), the Eq. 1 weight
 // table [k_t][|k_x|][|k_y|][3] (r_m, or r_m^2 for the energy reading feat = 1, with the k_t multiplicity
 // and the 1/n^3 of the mean folded in).
-template <int N, int FMT>
+template <int N, int FMT, bool WIDE = false>
 __device__ void build_fwd_tables(const Tw<N>& tw, unsigned char* out, int tid, int nt, int feat) {
-    using G = FwdGeo<N>;
+    using G = FwdGeo<N, WIDE>;
     constexpr int H = G::H;
     unsigned char* a2 = out;
     unsigned char* b1 = out + G::TAB_B1;
@@ -144,12 +152,12 @@ __device__ void build_fwd_tables(const Tw<N>& tw, unsigned char* out, int tid, i
         *reinterpret_cast<uint16_t*>(b1 + (c / 8) * 256 + (u / 8) * 128 + (c % 8) * 16 + (u % 8) * 2) =
             Pack<FMT>::one(v);
     }
-    // B3a[ncol][u] = [c | -s], B3b[ncol][u] = [s | c] over k_y = ncol % n (K-major, K = u)
-    for (int i = tid; i < G::N3 * 16; i += nt) {
-        const int ncol = i / 16, u = i % 16, k = ncol % N;
-        const bool re = ncol < N;
+    // B3a[ncol][k] = [c | -s], B3b[ncol][k] = [s | c] over k_y = ncol % n at tap k - j of output j = ncol / 2n (K-major)
+    for (int i = tid; i < G::W3 * G::K3; i += nt) {
+        const int ncol = i / G::K3, kk = i % G::K3, k = ncol % N, u = kk - ncol / G::N3;
+        const bool re = ncol % G::N3 < N;
         const float c = twc<N>(tw, k, u), sn = tws<N>(tw, k, u);
-        const size_t off = (ncol / 8) * 256 + (u / 8) * 128 + (ncol % 8) * 16 + (u % 8) * 2;
+        const size_t off = (ncol / 8) * G::SBO_B3 + (kk / 8) * 128 + (ncol % 8) * 16 + (kk % 8) * 2;
         *reinterpret_cast<uint16_t*>(b3a + off) = Pack<FMT>::one(re ? c : -sn);
         *reinterpret_cast<uint16_t*>(b3b + off) = Pack<FMT>::one(re ? sn : c);
     }
@@ -256,11 +264,12 @@ __device__ void stage_issue(int smode, const CUtensorMap* tmap, const float* __r
 // Bricks staged by the TMA unit (tma_brick; stage_issue has issued their copies) read their samples from
 // s_stage once mbar completes (a bounded wait: on timeout the error word and *s_fail are set and the
 // brick is taken as zero); the others load them from V, applying the border extension.  Contains one
-// __syncthreads.
+// __syncthreads.  nonfinite (may be null): whether a sample of the halo, or one
+// scaled, is a NaN or an infinity.
 template <int N, int FMT, int NT>
 __device__ float stage_brick(const float* __restrict__ V, int T, int X, int Y, int bnd, int t0, int xb, int yb,
                              unsigned char* s_a1, float* s_red, int tid, bool tma, const unsigned char* s_stage,
-                             int smode, uint32_t mbar, int* err, int* s_fail) {
+                             int smode, uint32_t mbar, int* err, int* s_fail, bool* nonfinite = nullptr) {
     using G = FwdGeo<N>;
     constexpr int XH = G::XH, YH = G::YH, YG = G::YG, YP = G::YP;
     constexpr int PER = (G::STAGE_ITEMS + NT - 1) / NT;
@@ -279,6 +288,7 @@ __device__ float stage_brick(const float* __restrict__ V, int T, int X, int Y, i
                           ty + YP <= Y;
     float vals[PER][8];
     float vmax = 0.f;
+    bool bad = false;
 #pragma unroll
     for (int r = 0; r < PER; ++r) {
         const int item = tid + r * NT;
@@ -322,17 +332,23 @@ __device__ float stage_brick(const float* __restrict__ V, int T, int X, int Y, i
         for (int i = 0; i < 8; ++i) {
             if (y8 + i >= YH) vals[r][i] = 0.f;     // positions past the halo (their outputs are not used)
             vmax = fmaxf(vmax, fabsf(vals[r][i]));
+            if (nonfinite) bad |= !(fabsf(vals[r][i]) <= 3.402823466e38f);
         }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-    if (lane == 0) s_red[warp] = vmax;
+    if (nonfinite) bad = __any_sync(0xffffffffu, bad);
+    if (lane == 0) s_red[warp] = bad ? -vmax : vmax;   // the sign carries the flag
     __syncthreads();
     float bmax = 0.f;
 #pragma unroll
-    for (int w = 0; w < NT / 32; ++w) bmax = fmaxf(bmax, s_red[w]);
+    for (int w = 0; w < NT / 32; ++w) {
+        bmax = fmaxf(bmax, fabsf(s_red[w]));
+        if (nonfinite) bad |= signbit(s_red[w]);
+    }
     const float scale = bmax > 0.f ? bmax : 1.f;
     const float inv_scale = 1.f / scale;
+    if (nonfinite) *nonfinite = bad || !(inv_scale <= 3.402823466e38f);   // or a largest sample with no reciprocal
 #pragma unroll
     for (int r = 0; r < PER; ++r) {
         const int item = tid + r * NT;

@@ -234,3 +234,28 @@ def test_window32_backward_is_not_built(sal):
         assert ei.value.status == 2  # SAL_ERR_UNSUPPORTED
     finally:
         eng.close()
+
+
+@pytest.mark.parametrize("prec", ["bf16", "fp16"])
+@pytest.mark.parametrize("n", [8, 16])
+@pytest.mark.parametrize("y", [0, 33, 47, 69])
+def test_tensor_core_forward_keeps_a_nan_to_the_rows_of_its_windows(sal, n, y, prec):
+    """A NaN reaches the outputs of its brick of x positions whose 16-row operand along y holds it, and no others: those are
+    what the volume without it gives, up to the order of FP32 sums of up to 16^3 terms, 2 * 48 roundings of 2^-24."""
+    shape, x = (3, 20, 70), 9
+    V, _ = synth.volume(synth.small_spec(shape, seed=n + y, faults=1))
+    V[1, x, y] = 0.0
+    p = sal.Params(n=n, boundary="zero", prec=prec)
+    clean = _run(sal, V, p)["E"]
+    V[1, x, y] = np.nan
+    E = _run(sal, V, p)["E"]
+    y0, x0, P = np.arange(shape[2]), np.arange(shape[1]), 128 // n
+    rows = (y0 - n // 2 <= y) & (y < y0 - n // 2 + 16)
+    xb = x0 // P * P
+    cols = (xb - n // 2 <= x) & (x < xb - n // 2 + P + n - 1)
+    reach = np.broadcast_to(cols[:, None] & rows[None, :], shape)
+    true = np.broadcast_to(((x0 - n // 2 <= x) & (x < x0 + n // 2))[:, None] &
+                           ((y0 - n // 2 <= y) & (y < y0 + n // 2))[None, :], shape)
+    for m in range(3):
+        assert np.isnan(E[m][true]).all()
+        assert np.allclose(E[m][~reach], clean[m][~reach], rtol=96 * 2.0 ** -24, atol=0)
