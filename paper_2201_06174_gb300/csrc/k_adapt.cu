@@ -20,7 +20,7 @@
 //                      operations a step at 2 per clock and SM);
 //   k3_adapt_chain     a block per chain: the weights at the start of each group of 32 segments, and W_out;
 //   k3_adapt_errors    (only for err2) each segment's steps again from its own starting weights, all at once.
-// All in FP64; 96^3, NLMS with err2: 708.1 -> 0.35 ms a call.  Chains the regrouping could make less exact than
+// All in FP64; 96^3, NLMS with err2: 708.1 -> 0.25 ms a call.  Chains the regrouping could make less exact than
 // the step-by-step filter are marked and left to it (k3_adapt): maps that grow (an entry above kGrow: LMS or NLMS
 // with a step size beyond their stability limit, or values that are not finite), and RLS whose R is near singular (kPivot).
 #include <algorithm>
@@ -119,12 +119,14 @@ k3_adapt(const float* __restrict__ S3, const float* __restrict__ D, int T, int X
 }
 
 // ---- The regrouped form -------------------------------------------------------------------------
-constexpr int kSegY = 8;               // sections of a block: 8 consecutive y are one 32-byte sector of S3 and D
+constexpr int kSegY = 4;               // sections of a block: with 8 (a whole 32-byte sector of S3 and D) the 216 blocks of
+                                       // a 96^3 volume left half of the SMs with two and the others waiting
 constexpr int kSegS = 32;              // segments of each section in a block
 constexpr int kSegThreads = kSegY * kSegS;
 constexpr int kMinSeg = 16;            // steps of a segment at least: the maps' composition costs what ~1.5 steps cost
-constexpr int kChainThreads = 64;      // chunks of a chain's groups: half of the FP64 work of the chain kernel is the
-                                       // threads' own chunks, the serial rest is one application per thread
+constexpr int kChainThreads = 256;     // chunks of a chain's groups, in kChainRows rows: chunks, then rows, are composed
+constexpr int kChainRows = 16;         // side by side (the rows by lanes of one warp: a partly filled warp takes as much of
+                                       // the FP64 pipe as a full one), and only the rows' maps one after the other
 constexpr double kGrow = 16.0;         // largest entry of a map that counts as stable (a contraction's is at most 1)
 constexpr double kPivot = 1e-7;        // smallest Cholesky pivot of R over its trace
 
@@ -254,14 +256,31 @@ struct SegGeo {
     double mu, eps, delta;
 };
 
-// The normalised maps and the desired value of step r of section y, as k3_adapt stages them.
+// (double)f on the integer pipe for zeros and normal numbers: the FP64 pipe, which bounds these kernels, also converts.
+__device__ __forceinline__ double widen(float f) {
+    const unsigned b = __float_as_uint(f), e = (b >> 23) & 255u;
+    if (e - 1u >= 254u) return (b << 1) == 0u ? 0.0 : (double)f;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + 0x38000000u)), (int)(b << 29));
+}
+
+// 1 / d by Newton's iteration from the FP32 reciprocal (2^-22, then 2^-44, then FP64's rounding): 4 multiply-adds of the
+// FP64 pipe; outside FP32's range the division.
+__device__ __forceinline__ double reciprocal(double d) {
+    const float f = (float)d;
+    if (!(f >= 1e-30f && f <= 1e30f)) return 1.0 / d;
+    double y = widen(__fdividef(1.0f, f));
+    y = fma(y, fma(-d, y, 1.0), y);
+    return fma(y, fma(-d, y, 1.0), y);
+}
+
+// The normalised maps and the desired value of step r of section y (nlo = -lo iv).
 __device__ __forceinline__ void seg_load(const float* __restrict__ S3, const float* __restrict__ D, const SegGeo& g,
-                                         long long NV, const double (&lo)[3], const double (&iv)[3], int y, int t, int xi,
+                                         long long NV, const double (&nlo)[3], const double (&iv)[3], int y, int t, int xi,
                                          double (&x)[3], double& d) {
     const long long p = ((long long)t * g.X + xi) * g.Y + y;
 #pragma unroll
-    for (int m = 0; m < 3; ++m) x[m] = ((double)__ldg(S3 + m * NV + p) - lo[m]) * iv[m];
-    d = (double)__ldg(D + p);
+    for (int m = 0; m < 3; ++m) x[m] = fma(widen(__ldg(S3 + m * NV + p)), iv[m], nlo[m]);
+    d = widen(__ldg(D + p));
 }
 
 template <bool RLS>
@@ -273,7 +292,7 @@ k3_adapt_segments(const float* __restrict__ S3, const float* __restrict__ D, Seg
     const long long NV = (long long)g.T * g.X * g.Y;
     const int yl = threadIdx.x % kSegY, sl = threadIdx.x / kSegY;
     const int y = blockIdx.y * kSegY + yl, seg = blockIdx.x * kSegS + sl;
-    const double lo[3] = {norm[0], norm[1], norm[2]}, iv[3] = {norm[3], norm[4], norm[5]};
+    const double iv[3] = {norm[3], norm[4], norm[5]}, nlo[3] = {-(norm[0] * iv[0]), -(norm[1] * iv[1]), -(norm[2] * iv[2])};
     St s;
     s.identity();
     if (y < g.Y && seg < g.nseg) {
@@ -281,14 +300,15 @@ k3_adapt_segments(const float* __restrict__ S3, const float* __restrict__ D, Seg
         const int cnt = (int)(per - r0 < g.L ? per - r0 : g.L);
         int xi = (int)(r0 / g.T), t = (int)(r0 - (long long)xi * g.T);
         double x[3], d;
-        seg_load(S3, D, g, NV, lo, iv, y, t, xi, x, d);
+        seg_load(S3, D, g, NV, nlo, iv, y, t, xi, x, d);
         for (int i = 0; i < cnt; ++i) {
             if (++t == g.T) { t = 0; ++xi; }
             double xn[3] = {0.0, 0.0, 0.0}, dn = 0.0;
-            if (i + 1 < cnt) seg_load(S3, D, g, NV, lo, iv, y, t, xi, xn, dn);   // under this step's arithmetic
+            if (i + 1 < cnt) seg_load(S3, D, g, NV, nlo, iv, y, t, xi, xn, dn);   // under this step's arithmetic
             const double gain = RLS ? 0.0
-                                : g.method == ADAPT_NLMS ? g.mu / (g.eps + (x[0] * x[0] + x[1] * x[1] + x[2] * x[2]))
-                                                         : g.mu;
+                                : g.method == ADAPT_NLMS
+                                    ? g.mu * reciprocal(g.eps + (x[0] * x[0] + x[1] * x[1] + x[2] * x[2]))
+                                    : g.mu;
             s.step(x, d, gain);
             x[0] = xn[0]; x[1] = xn[1]; x[2] = xn[2];
             d = dn;
@@ -320,45 +340,68 @@ k3_adapt_segments(const float* __restrict__ S3, const float* __restrict__ D, Seg
     }
 }
 
-// One block per chain: its groups (section by section) in kChainThreads contiguous chunks, each composed by one
-// thread; thread 0 applies the chunks in order; each thread then walks its chunk's groups from its start.
+// One block per chain: its groups (section by section) in kChainThreads contiguous chunks, each composed by one thread; 16
+// lanes compose 16 chunks each; thread 0 applies these rows in order; the lanes then walk their chunks, and each thread its
+// groups, from their starts.
 template <bool RLS>
 __global__ void __launch_bounds__(kChainThreads)
 k3_adapt_chain(SegGeo g, const double* __restrict__ groups, double* __restrict__ starts, float* __restrict__ W_out,
                int* __restrict__ todo) {
     using St = SegState<RLS>;
     using Sa = Start<RLS>;
-    __shared__ double s_v[St::K][kChainThreads], s_st[Sa::K][kChainThreads];
+    constexpr int kPerRow = kChainThreads / kChainRows, kPitch = kPerRow + 1;   // rows one double apart in the banks
+    __shared__ double s_v[St::K][kChainRows * kPitch], s_r[St::K][kChainRows], s_st[Sa::K][kChainRows * kPitch];
     const int y0 = blockIdx.x * g.sec, y1 = min(g.Y, y0 + g.sec), tid = threadIdx.x;
+    const int slot = tid / kPerRow * kPitch + tid % kPerRow;
     const long long base = (long long)y0 * g.ngroup, total = (long long)(y1 - y0) * g.ngroup;
     const long long per = (total + kChainThreads - 1) / kChainThreads;
     const long long a = min(total, per * tid), b = min(total, a + per);
-    St s;
-    s.identity();
-    for (long long i = a; i < b; ++i) {
+    auto group = [&](long long i) {
         St l;
 #pragma unroll
         for (int k = 0; k < St::K; ++k) l.v[k] = __ldg(groups + (base + i) * St::K + k);
-        s.then(l);
+        return l;
+    };
+    auto get = [&](St& l, int i) {
+#pragma unroll
+        for (int k = 0; k < St::K; ++k) l.v[k] = s_v[k][i];
+    };
+    St s;
+    s.identity();
+    if (a < b) {
+        s = group(a);
+        for (long long i = a + 1; i < b; ++i) s.then(group(i));
     }
-    const int bad = __syncthreads_or(s.bad());
+#pragma unroll
+    for (int k = 0; k < St::K; ++k) s_v[k][slot] = s.v[k];
+    __syncthreads();
+    bool unsound = s.bad();
+    if (tid < kChainRows) {
+        get(s, tid * kPitch);
+        for (int i = 1; i < kPerRow; ++i) {
+            St l;
+            get(l, tid * kPitch + i);
+            s.then(l);
+        }
+        unsound = unsound || s.bad();
+#pragma unroll
+        for (int k = 0; k < St::K; ++k) s_r[k][tid] = s.v[k];
+    }
+    const int bad = __syncthreads_or(unsound);
     if (bad || todo[blockIdx.x]) {
         __syncthreads();
         if (tid == 0) todo[blockIdx.x] = 1;
         return;   // block-uniform: the step-by-step filter takes this chain
     }
-#pragma unroll
-    for (int k = 0; k < St::K; ++k) s_v[k][tid] = s.v[k];
-    __syncthreads();
+    Sa st;
     if (tid == 0) {
-        Sa st;
         st.first(g.delta);
-        for (int i = 0; i < kChainThreads; ++i) {
+        for (int i = 0; i < kChainRows; ++i) {
             St l;
 #pragma unroll
-            for (int k = 0; k < Sa::K; ++k) s_st[k][i] = st.v[k];
+            for (int k = 0; k < Sa::K; ++k) s_st[k][i * kPitch] = st.v[k];
 #pragma unroll
-            for (int k = 0; k < St::K; ++k) l.v[k] = s_v[k][i];
+            for (int k = 0; k < St::K; ++k) l.v[k] = s_r[k][i];
             st.advance(l);
         }
         double w[3], P[6];
@@ -369,18 +412,26 @@ k3_adapt_chain(SegGeo g, const double* __restrict__ groups, double* __restrict__
             todo[blockIdx.x] = 1;
         }
     }
-    __syncthreads();
     if (!starts) return;
-    Sa st;
+    __syncthreads();
+    if (tid < kChainRows) {
 #pragma unroll
-    for (int k = 0; k < Sa::K; ++k) st.v[k] = s_st[k][tid];
+        for (int k = 0; k < Sa::K; ++k) st.v[k] = s_st[k][tid * kPitch];
+        for (int i = 1; i < kPerRow; ++i) {
+            St l;
+            get(l, tid * kPitch + i - 1);
+            st.advance(l);
+#pragma unroll
+            for (int k = 0; k < Sa::K; ++k) s_st[k][tid * kPitch + i] = st.v[k];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < Sa::K; ++k) st.v[k] = s_st[k][slot];
     for (long long i = a; i < b; ++i) {
-        St l;
 #pragma unroll
         for (int k = 0; k < Sa::K; ++k) starts[(base + i) * Sa::K + k] = st.v[k];
-#pragma unroll
-        for (int k = 0; k < St::K; ++k) l.v[k] = __ldg(groups + (base + i) * St::K + k);
-        st.advance(l);
+        st.advance(group(i));
     }
 }
 
@@ -428,23 +479,23 @@ k3_adapt_errors(const float* __restrict__ S3, const float* __restrict__ D, SegGe
         todo[y / g.sec] = 1;
         return;
     }
-    const double lo[3] = {norm[0], norm[1], norm[2]}, iv[3] = {norm[3], norm[4], norm[5]};
+    const double iv[3] = {norm[3], norm[4], norm[5]}, nlo[3] = {-(norm[0] * iv[0]), -(norm[1] * iv[1]), -(norm[2] * iv[2])};
     const int cnt = (int)(per - r0 < g.L ? per - r0 : g.L);
     int xi = (int)(r0 / g.T), t = (int)(r0 - (long long)xi * g.T);
     float* out = err2 + (long long)y * per + r0;
     double x[3], d;
-    seg_load(S3, D, g, NV, lo, iv, y, t, xi, x, d);
+    seg_load(S3, D, g, NV, nlo, iv, y, t, xi, x, d);
     for (int i = 0; i < cnt; ++i) {
         if (++t == g.T) { t = 0; ++xi; }
         double xn[3] = {0.0, 0.0, 0.0}, dn = 0.0;
-        if (i + 1 < cnt) seg_load(S3, D, g, NV, lo, iv, y, t, xi, xn, dn);
+        if (i + 1 < cnt) seg_load(S3, D, g, NV, nlo, iv, y, t, xi, xn, dn);
         const double e = d - (w[0] * x[0] + w[1] * x[1] + w[2] * x[2]);
         out[i] = (float)(e * e);
         if (RLS) {
             const double p0 = P[0] * x[0] + P[1] * x[1] + P[2] * x[2];
             const double p1 = P[1] * x[0] + P[3] * x[1] + P[4] * x[2];
             const double p2 = P[2] * x[0] + P[4] * x[1] + P[5] * x[2];
-            const double inv = 1.0 / (1.0 + x[0] * p0 + x[1] * p1 + x[2] * p2);
+            const double inv = reciprocal(1.0 + x[0] * p0 + x[1] * p1 + x[2] * p2);
             const double k0 = p0 * inv, k1 = p1 * inv, k2 = p2 * inv;
             w[0] += k0 * e;
             w[1] += k1 * e;
@@ -453,7 +504,7 @@ k3_adapt_errors(const float* __restrict__ S3, const float* __restrict__ D, SegGe
             P[3] -= k1 * p1; P[4] -= k1 * p2; P[5] -= k2 * p2;
         } else {
             const double ge = g.method == ADAPT_NLMS
-                                  ? g.mu * e / (g.eps + (x[0] * x[0] + x[1] * x[1] + x[2] * x[2]))
+                                  ? g.mu * e * reciprocal(g.eps + (x[0] * x[0] + x[1] * x[1] + x[2] * x[2]))
                                   : g.mu * e;
 #pragma unroll
             for (int m = 0; m < 3; ++m) w[m] += ge * x[m];
