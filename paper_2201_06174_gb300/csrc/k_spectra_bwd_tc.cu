@@ -265,7 +265,7 @@ k5_spectra_adjoint_tc(const float* __restrict__ V, const float* __restrict__ gE,
             const bool adjoint = warp == kConsumers;
             const bool leader = lane == 0;
             const uint32_t idesc1 = tc::idesc_f16(kFmt, 128, 16, 1, 0);
-            const uint32_t idesc2 = tc::idesc_f16(kFmt, 128, G::N2, 0, 0);
+            const uint32_t idesc2 = tc::idesc_f16(kFmt, 128, G::N2, 0, 1);
             const uint32_t idesc3 = tc::idesc_f16(kFmt, 128, G::N3, 1, 0);
             const uint32_t idescy = tc::idesc_f16(kFmt, 128, 32, 0, 0);
             const uint32_t idescx = tc::idesc_f16(kFmt, 128, 64, 1, 1);
@@ -292,7 +292,7 @@ k5_spectra_adjoint_tc(const float* __restrict__ V, const float* __restrict__ gE,
             };
             // base descriptors; windows, slots and K steps are the same descriptors moved (desc_add)
             const uint64_t a2d = tc::desc_noswizzle(tab, 128, G::SBO_K2);
-            const uint64_t b2d = tc::desc_noswizzle(b2base, 128, G::SBO_K2);
+            const uint64_t b2d = tc::desc_noswizzle(b2base, 128, G::SBO_B2);
             const uint64_t ared = tc::desc_noswizzle(are, 128, G::SBO_A3);
             const uint64_t aimd = tc::desc_noswizzle(aim, 128, G::SBO_A3);
             const uint64_t gd = tc::desc_noswizzle(gbase, 128, G::SBO_G);

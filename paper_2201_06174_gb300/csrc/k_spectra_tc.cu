@@ -58,7 +58,7 @@ k1_spectra_tc(const float* __restrict__ V, float* __restrict__ E, int T, int X, 
     constexpr int H = G::H, P = G::P;
     extern __shared__ __align__(128) unsigned char smem[];
     unsigned char* s_a1 = smem;                              // stage-1 A (MN-major), then:
-    unsigned char* s_b2 = smem;                              // stage-2 B tiles, one per k_t (K-major)
+    unsigned char* s_b2 = smem;                              // stage-2 B tiles, one per k_t (MN-major)
     unsigned char* s_tab = smem + G::OFF_TAB;                // constant operands (bulk copy)
     unsigned char* s_are = smem + G::OFF_A3;                 // stage-3 A, real part (MN-major)
     unsigned char* s_aim = smem + G::OFF_A3 + G::A3_B;       // stage-3 A, imaginary part
@@ -123,7 +123,7 @@ k1_spectra_tc(const float* __restrict__ V, float* __restrict__ E, int T, int X, 
         // ============================ producer warp: one elected lane issues every MMA ========================
         {
             const uint32_t idesc1 = tc::idesc_f16(FMT, 128, 16, 1, 0);
-            const uint32_t idesc2 = tc::idesc_f16(FMT, 128, G::N2, 0, 0);
+            const uint32_t idesc2 = tc::idesc_f16(FMT, 128, G::N2, 0, 1);
             const uint32_t idesc3 = tc::idesc_f16(FMT, 128, G::N3, 1, 0);     // one output
             const uint32_t idesc3w = tc::idesc_f16(FMT, 128, G::W3, 1, 0);    // a pass
             const uint32_t tab = tc::smem_u32(s_tab), b2base = tc::smem_u32(s_b2);
@@ -140,7 +140,7 @@ k1_spectra_tc(const float* __restrict__ V, float* __restrict__ E, int T, int X, 
             };
             // base descriptors; windows and K steps are the same descriptors moved (desc_add)
             const uint64_t a2d = tc::desc_noswizzle(tab, 128, G::SBO_K2);
-            const uint64_t b2d = tc::desc_noswizzle(b2base, 128, G::SBO_K2);
+            const uint64_t b2d = tc::desc_noswizzle(b2base, 128, G::SBO_B2);
             const uint64_t ared = tc::desc_noswizzle(are, 128, G::SBO_A3);
             const uint64_t aimd = tc::desc_noswizzle(aim, 128, G::SBO_A3);
             auto issue_s2 = [&](int kt) {

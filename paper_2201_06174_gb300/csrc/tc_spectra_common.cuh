@@ -59,7 +59,8 @@ template <int N, bool WIDE = false> struct FwdGeo {
     static constexpr uint32_t SBO_A3 = kKRows * 16;
     static constexpr uint32_t SBO_K2 = kK2 / 8 * 128;    // 8-row group stride of the K-major A2 / B2
     static constexpr size_t A1_B = (size_t)NB1 * 4096;
-    static constexpr size_t B2_B = (size_t)N2 / 8 * SBO_K2;   // one k_t tile
+    static constexpr uint32_t SBO_B2 = SBO_K2 + 16;      // MN-major B2: 8-column groups, one 16-byte row apart in the banks
+    static constexpr size_t B2_B = (size_t)N2 / 8 * SBO_B2;   // one k_t tile
     static constexpr size_t B2ALL_B = (size_t)H * B2_B;
     static constexpr size_t R0_B = ((A1_B > B2ALL_B ? A1_B : B2ALL_B) + 127) / 128 * 128;  // A1, then B2 tiles
     // forward constant operands: [A2 | B1 | B3a | B3b | Eq. 1 weight table]
@@ -379,11 +380,11 @@ __device__ void d1_to_b2(uint32_t tmem, unsigned char* s_b2, int q, int lane, in
         const int pos = 128 * i + 32 * q + lane;
         const int x = pos / YP, y = pos % YP;
         if (x < kXHP) {
-            // K-major: byte(ncol, k2) = (ncol/8) SBO_K2 + (k2/8) 128 + (ncol%8) 16 + (k2%8) 2
-            const size_t o_re = (size_t)(y / 8) * G::SBO_K2 + (y % 8) * 16;
-            const size_t o_im = (size_t)((YP + y) / 8) * G::SBO_K2 + ((YP + y) % 8) * 16;
-            const size_t k_c = (size_t)(x / 8) * 128 + (x % 8) * 2;
-            const size_t k_s = (size_t)((kXHP + x) / 8) * 128 + ((kXHP + x) % 8) * 2;
+            // MN-major: byte(ncol, k2) = (ncol/8) SBO_B2 + k2 16 + (ncol%8) 2: the 32 y of a warp's store lie in 4
+            // rows that share no bank (K-major rows, one y each, met in 8 banks: 4 passes a store)
+            const size_t o_re = (size_t)(y / 8) * G::SBO_B2 + (y % 8) * 2;
+            const size_t o_im = (size_t)((YP + y) / 8) * G::SBO_B2 + (y % 8) * 2;
+            const size_t k_c = (size_t)x * 16, k_s = (size_t)(kXHP + x) * 16;
 #pragma unroll
             for (int kt = 0; kt < H; ++kt) {
                 const float g1r = v[kt];
