@@ -223,7 +223,7 @@ k5_spectra_adjoint_tc(const float* __restrict__ V, const float* __restrict__ gE,
         float a = 0.f;
 #pragma unroll
         for (int u = 0; u < N; ++u) {
-            const __half hv = *reinterpret_cast<const __half*>(s_a1 + (pos / 8) * 256 + (u / 8) * 128 + (u % 8) * 16 +
+            const __half hv = *reinterpret_cast<const __half*>(s_a1 + (pos / 8) * G::SBO_A1 + (u / 8) * 128 + (u % 8) * 16 +
                                                                (pos % 8) * 2);
             a = fmaf(tw.c[0][u], fabsf(__half2float(hv)), a);
         }
@@ -344,11 +344,11 @@ k5_spectra_adjoint_tc(const float* __restrict__ V, const float* __restrict__ gE,
                 bool alive = pwait(12);
                 if (alive) {   // stage 1, all k_t at once
                     const uint64_t b1 = tc::desc_noswizzle(tab + (uint32_t)G::TAB_B1, 128, 256);
-                    const uint64_t a1 = tc::desc_noswizzle(tc::smem_u32(s_a1), 128, 256);
+                    const uint64_t a1 = tc::desc_noswizzle(tc::smem_u32(s_a1), 128, G::SBO_A1);
                     if (tc::elect_one()) {
 #pragma unroll
                         for (int i = 0; i < G::NB1; ++i)
-                            tc::mma_f16(tmem + 16 * i, tc::desc_add(a1, 4096 * i), b1, idesc1, 0);
+                            tc::mma_f16(tmem + 16 * i, tc::desc_add(a1, G::BLK_A1 * i), b1, idesc1, 0);
                         tc::mma_commit(tc::smem_u32(&s_mbar[0]));
                     }
                     __syncwarp();
@@ -404,13 +404,13 @@ k5_spectra_adjoint_tc(const float* __restrict__ V, const float* __restrict__ gE,
                             for (int h = 0; h < 2; ++h) {
                                 const int y8 = 16 * (c & 1) + 8 * h;
                                 if (y8 < YP) {
-                                    // MN-major: byte(pos, k) = (pos/8) 256 + (k/8) 128 + (k%8) 16 + (pos%8) 2, pos = x YP + y
+                                    // MN-major: byte(pos, k) = (pos/8) SBO_A1 + (k/8) 128 + (k%8) 16 + (pos%8) 2, pos = x YP + y
                                     uint4 w;
                                     w.x = Pack<kFmt>::two(kDxScale * v[8 * h + 0], kDxScale * v[8 * h + 1]);
                                     w.y = Pack<kFmt>::two(kDxScale * v[8 * h + 2], kDxScale * v[8 * h + 3]);
                                     w.z = Pack<kFmt>::two(kDxScale * v[8 * h + 4], kDxScale * v[8 * h + 5]);
                                     w.w = Pack<kFmt>::two(kDxScale * v[8 * h + 6], kDxScale * v[8 * h + 7]);
-                                    *reinterpret_cast<uint4*>(s_at + ((lane * YP + y8) / 8) * 256 + k * 16) = w;
+                                    *reinterpret_cast<uint4*>(s_at + ((lane * YP + y8) / 8) * G::SBO_A1 + k * 16) = w;
                                 }
                             }
                         }
@@ -421,11 +421,11 @@ k5_spectra_adjoint_tc(const float* __restrict__ V, const float* __restrict__ gE,
                     tc::fence_after_sync();
                     // ---- adjoint of stage 1: gV block += A_t B_t(k_t), accumulated over k_t in tensor memory ----
                     const uint64_t btd = tc::desc_noswizzle(tab + (uint32_t)(G::TAB_BT + 512 * ktp), 128, 256);
-                    const uint64_t atd = tc::desc_noswizzle(at, 128, 256);
+                    const uint64_t atd = tc::desc_noswizzle(at, 128, G::SBO_A1);
                     if (tc::elect_one()) {
     #pragma unroll
                         for (int i = 0; i < G::NB1; ++i)
-                            tc::mma_f16(tmem + kColT + 16 * i, tc::desc_add(atd, 4096 * i), btd, idesct, ktp > 0 ? 1u : 0u);
+                            tc::mma_f16(tmem + kColT + 16 * i, tc::desc_add(atd, G::BLK_A1 * i), btd, idesct, ktp > 0 ? 1u : 0u);
                     }
                     __syncwarp();
                     return true;

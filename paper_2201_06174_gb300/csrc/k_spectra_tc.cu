@@ -181,10 +181,10 @@ k1_spectra_tc(const float* __restrict__ V, float* __restrict__ E, int T, int X, 
             bool alive = pwait(6, 0);
             if (alive) {   // stage 1, all k_t at once
                 const uint64_t b1 = tc::desc_noswizzle(tab + (uint32_t)G::TAB_B1, 128, 256);
-                const uint64_t a1 = tc::desc_noswizzle(tc::smem_u32(s_a1), 128, 256);
+                const uint64_t a1 = tc::desc_noswizzle(tc::smem_u32(s_a1), 128, G::SBO_A1);
                 if (tc::elect_one()) {
 #pragma unroll
-                    for (int i = 0; i < G::NB1; ++i) tc::mma_f16(tmem + 16 * i, tc::desc_add(a1, 4096 * i), b1, idesc1, 0);
+                    for (int i = 0; i < G::NB1; ++i) tc::mma_f16(tmem + 16 * i, tc::desc_add(a1, G::BLK_A1 * i), b1, idesc1, 0);
                     tc::mma_commit(tc::smem_u32(&s_mbar[0]));
                 }
                 __syncwarp();

@@ -58,7 +58,11 @@ template <int N, bool WIDE = false> struct FwdGeo {
     static constexpr int PASSES = kBY / OPP;   // 4 (n = 16) or 2 (n = 8), alternating buffers
     static constexpr uint32_t SBO_A3 = kKRows * 16;
     static constexpr uint32_t SBO_K2 = kK2 / 8 * 128;    // 8-row group stride of the K-major A2 / B2
-    static constexpr size_t A1_B = (size_t)NB1 * 4096;
+    // operands over positions (MN-major, 8 positions a group): one group 272 bytes on from the last, 16 more than its rows
+    // take, so that the 16-byte stores of neighbouring groups share no bank (a pitch of 256 met in 4 banks)
+    static constexpr uint32_t SBO_A1 = 272;
+    static constexpr uint32_t BLK_A1 = 16 * SBO_A1;           // 128 positions
+    static constexpr size_t A1_B = (size_t)NB1 * BLK_A1;
     static constexpr uint32_t SBO_B2 = SBO_K2 + 16;      // MN-major B2: 8-column groups, one 16-byte row apart in the banks
     static constexpr size_t B2_B = (size_t)N2 / 8 * SBO_B2;   // one k_t tile
     static constexpr size_t B2ALL_B = (size_t)H * B2_B;
@@ -360,8 +364,8 @@ __device__ float stage_brick(const float* __restrict__ V, int T, int X, int Y, i
             w.y = Pack<FMT>::two(vals[r][2] * inv_scale, vals[r][3] * inv_scale);
             w.z = Pack<FMT>::two(vals[r][4] * inv_scale, vals[r][5] * inv_scale);
             w.w = Pack<FMT>::two(vals[r][6] * inv_scale, vals[r][7] * inv_scale);
-            // MN-major: byte(pos, u) = (pos/8) 256 + (u/8) 128 + (u%8) 16 + (pos%8) 2
-            *reinterpret_cast<uint4*>(s_a1 + g * 256 + (u / 8) * 128 + (u % 8) * 16) = w;
+            // MN-major: byte(pos, u) = (pos/8) SBO_A1 + (u/8) 128 + (u%8) 16 + (pos%8) 2
+            *reinterpret_cast<uint4*>(s_a1 + g * G::SBO_A1 + (u / 8) * 128 + (u % 8) * 16) = w;
         }
     }
     return scale;
