@@ -83,7 +83,7 @@ template <int N> struct BtGeo : tcs::FwdGeo<N> {
     static constexpr size_t OFF_AT = OFF_BC + 2 * BDG_B;         // t-adjoint A operand [pos][16], MN-major
     static constexpr size_t OFF_GE = OFF_AT + F::A1_B;
     static constexpr size_t OFF_L1 = OFF_GE + (size_t)3 * F::P * kBY * 4;
-    static constexpr size_t OFF_MISC = (OFF_L1 + (size_t)F::P * kBY * 4 + 15) / 16 * 16;
+    static constexpr size_t OFF_MISC = OFF_L1 + (size_t)F::P * kBY * 16;
     static constexpr size_t SMEM = OFF_MISC + 8 * kBars + 16 + 2 * 32 * 4;
     static_assert((size_t)(kXHP * F::YP + F::XH * kBY) * 4 <= G_B, "L1 sums fit in the Gamma region");
     static_assert(TAB5_B % 16 == 0 && OFF_A3 % 16 == 0 && OFF_AT % 16 == 0, "alignment");
@@ -153,7 +153,7 @@ k5_spectra_adjoint_tc(const float* __restrict__ V, const float* __restrict__ gE,
     float* s_col = reinterpret_cast<float*>(smem + G::OFF_G);    // L1 column sums (set-up only)
     unsigned char* s_at = smem + G::OFF_AT;                      // t-adjoint A operand
     float* s_ge = reinterpret_cast<float*>(smem + G::OFF_GE);    // [3][P][16]
-    float* s_l1 = reinterpret_cast<float*>(smem + G::OFF_L1);    // [P][16]
+    float4* s_out = reinterpret_cast<float4*>(smem + G::OFF_L1);  // [P][16]: scaled gE of the three maps, kink band squared
     const float* s_wt = reinterpret_cast<const float*>(s_tab + G::TAB_WT);
     // mbarriers (arrival counts): [0], [1] forward buffer full (MMA commit); [2], [3] forward buffer read
     // (16 warps); [4] stage-3 A written (16); [5] stage-2 B tiles written (16); [6], [7] Gamma set written
@@ -245,7 +245,9 @@ k5_spectra_adjoint_tc(const float* __restrict__ V, const float* __restrict__ gE,
         float a = 0.f;
 #pragma unroll
         for (int ux = 0; ux < N; ++ux) a = fmaf(tw.c[0][ux], s_row[(xl + ux) * kBY + y0], a);
-        s_l1[i] = a;
+        const float thr = kKinkTau * a;
+        s_out[i] = make_float4(sigma_op * s_ge[i], sigma_op * s_ge[P * kBY + i], sigma_op * s_ge[2 * P * kBY + i],
+                               fmaxf(thr * thr, 1e-30f));
     }
     __syncthreads();   // L1 norms visible; the column-sum area (Gamma region) free again
     tc::fence_after_sync();
@@ -495,13 +497,13 @@ k5_spectra_adjoint_tc(const float* __restrict__ V, const float* __restrict__ gE,
         constexpr int HP = (H + 1) / 2;
         float2 wt[3][HP];
         auto load_wt = [&](int kt) {
+            float w[G::WTP];
+            tcs::load_weights<N>(s_wt, kt, ajx, w);
 #pragma unroll
             for (int kk = 0; kk < HP; ++kk) {
-                const float* w = s_wt + ((kt * H + ajx) * H + 2 * kk) * 3;
                 const bool two = 2 * kk + 1 < H;
-                wt[0][kk] = make_float2(w[0], two ? w[3] : 0.f);
-                wt[1][kk] = make_float2(w[1], two ? w[4] : 0.f);
-                wt[2][kk] = make_float2(w[2], two ? w[5] : 0.f);
+#pragma unroll
+                for (int m = 0; m < 3; ++m) wt[m][kk] = make_float2(w[6 * kk + m], two ? w[6 * kk + 3 + m] : 0.f);
             }
         };
         load_wt(0);
@@ -520,13 +522,11 @@ k5_spectra_adjoint_tc(const float* __restrict__ V, const float* __restrict__ gE,
                         const int j = grp * G::OPC + o;
                         const int y0 = pass * G::OPP + j;
                         const int gi = x0l * kBY + y0;
-                        const float g0 = s_ge[gi], g1 = s_ge[P * kBY + gi], g2 = s_ge[2 * P * kBY + gi];
-                        const float thr = kKinkTau * s_l1[gi];
-                        const float thr2 = fmaxf(thr * thr, 1e-30f);
-                        // rho of |k_y| = 2 kk, 2 kk + 1 (packed; sigma folded into the three gE factors)
-                        const float2 gs0 = make_float2(sigma_op * g0, sigma_op * g0);
-                        const float2 gs1 = make_float2(sigma_op * g1, sigma_op * g1);
-                        const float2 gs2 = make_float2(sigma_op * g2, sigma_op * g2);
+                        const float4 og = s_out[gi];
+                        const float thr2 = og.w;
+                        // rho of |k_y| = 2 kk, 2 kk + 1 (packed; sigma is in the three gE factors)
+                        const float2 gs0 = make_float2(og.x, og.x), gs1 = make_float2(og.y, og.y);
+                        const float2 gs2 = make_float2(og.z, og.z);
                         float2 rho[HP];
 #pragma unroll
                         for (int kk = 0; kk < HP; ++kk)

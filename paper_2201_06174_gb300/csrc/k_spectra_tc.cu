@@ -256,7 +256,7 @@ k1_spectra_tc(const float* __restrict__ V, float* __restrict__ E, int T, int X, 
             float wt[3][H];
 #pragma unroll
             for (int k = 0; k < H; ++k) {
-                const float* w = s_wt + ((kt * H + ajx) * H + k) * 3;
+                const float* w = s_wt + (kt * H + ajx) * G::WTP + k * 3;
                 wt[0][k] = w[0];
                 wt[1][k] = w[1];
                 wt[2][k] = w[2];

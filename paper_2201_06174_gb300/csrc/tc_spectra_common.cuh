@@ -73,7 +73,11 @@ template <int N, bool WIDE = false> struct FwdGeo {
     static constexpr int K3 = WIDE && N + OPP - 1 > 16 ? 32 : 16;       // its K rows
     static constexpr uint32_t SBO_B3 = K3 / 8 * 128;
     static constexpr size_t B3_B = (size_t)W3 / 8 * SBO_B3;
-    static constexpr size_t WT_B = ((size_t)H * H * H * 3 * 4 + 15) / 16 * 16;
+    // Eq. 1 weights: a row of 3 H per (k_t, |k_x|).  The adjoint reads it in 16-byte pieces, rows 4 words apart in the
+    // banks; the wide forward (K1-TC) word by word: in pieces its 128^3 call at n = 16 took 2334 instead of 2262 us
+    static constexpr int WTP =
+        WIDE ? 3 * H : (3 * H + 3) / 4 % 2 ? (3 * H + 3) / 4 * 4 : (3 * H + 3) / 4 * 4 + 4;
+    static constexpr size_t WT_B = ((size_t)H * H * WTP * 4 + 15) / 16 * 16;
     static constexpr size_t TAB_B1 = A2_B;
     static constexpr size_t TAB_B3A = TAB_B1 + 512;
     static constexpr size_t TAB_B3B = TAB_B3A + B3_B;
@@ -137,7 +141,7 @@ template <int N> __device__ __forceinline__ float tws(const Tw<N>& tw, int k, in
 
 // The forward constant operands of one (n, operand type) into `out` (TAB_B bytes): A2 (Toeplitz
 // stage-2 twiddles, K-major), B1 (stage-1 twiddles), B3a / B3b (stage-3 twiddles), the Eq. 1 weight
-// table [k_t][|k_x|][|k_y|][3] (r_m, or r_m^2 for the energy reading feat = 1, with the k_t multiplicity
+// table [k_t][|k_x|][|k_y|][3], rows of WTP (r_m, or r_m^2 for the energy reading feat = 1, with the k_t multiplicity
 // and the 1/n^3 of the mean folded in).
 template <int N, int FMT, bool WIDE = false>
 __device__ void build_fwd_tables(const Tw<N>& tw, unsigned char* out, int tid, int nt, int feat) {
@@ -180,9 +184,27 @@ __device__ void build_fwd_tables(const Tw<N>& tw, unsigned char* out, int tid, i
         float w0, w1, w2;
         if (feat == 1) f32::bin_weights<true>(kt, aj, k, mult / (float)(N * N * N), w0, w1, w2);
         else f32::bin_weights<false>(kt, aj, k, mult / (float)(N * N * N), w0, w1, w2);
-        wt[i * 3 + 0] = w0;
-        wt[i * 3 + 1] = w1;
-        wt[i * 3 + 2] = w2;
+        float* w = wt + i / H * G::WTP + k * 3;
+        w[0] = w0;
+        w[1] = w1;
+        w[2] = w2;
+    }
+    for (int i = tid; i < H * H * G::WTP; i += nt)
+        if (i % G::WTP >= 3 * H) wt[i] = 0.f;
+}
+
+// One row of the weight table: [|k_y|][3] at out[0 .. 3 H).
+template <int N>
+__device__ __forceinline__ void load_weights(const float* wt, int kt, int ajx, float (&out)[FwdGeo<N>::WTP]) {
+    using G = FwdGeo<N>;
+    const float4* w = reinterpret_cast<const float4*>(wt + (kt * G::H + ajx) * G::WTP);
+#pragma unroll
+    for (int i = 0; i < (3 * G::H + 3) / 4; ++i) {
+        const float4 f = w[i];
+        out[4 * i] = f.x;
+        out[4 * i + 1] = f.y;
+        out[4 * i + 2] = f.z;
+        out[4 * i + 3] = f.w;
     }
 }
 
