@@ -81,8 +81,8 @@ template <int N> struct BtGeo : tcs::FwdGeo<N> {
     static constexpr size_t G_B = 2 * GSET_B;
     static constexpr size_t OFF_BC = OFF_G + G_B;                // B_c | B_s (their own region)
     static constexpr size_t OFF_AT = OFF_BC + 2 * BDG_B;         // t-adjoint A operand [pos][16], MN-major
-    static constexpr size_t OFF_GE = OFF_AT + F::A1_B;
-    static constexpr size_t OFF_L1 = OFF_GE + (size_t)3 * F::P * kBY * 4;
+    static constexpr size_t OFF_GE = OFF_BC;                     // feature gradients (set-up only)
+    static constexpr size_t OFF_L1 = OFF_AT + F::A1_B;
     static constexpr size_t OFF_MISC = OFF_L1 + (size_t)F::P * kBY * 16;
     static constexpr size_t SMEM = OFF_MISC + 8 * kBars + 16 + 2 * 32 * 4;
     static_assert((size_t)(kXHP * F::YP + F::XH * kBY) * 4 <= G_B, "L1 sums fit in the Gamma region");
@@ -152,7 +152,7 @@ k5_spectra_adjoint_tc(const float* __restrict__ V, const float* __restrict__ gE,
     unsigned char* s_bs = s_bc + G::BDG_B;                       // B_s = [-dG2i | dG2r]
     float* s_col = reinterpret_cast<float*>(smem + G::OFF_G);    // L1 column sums (set-up only)
     unsigned char* s_at = smem + G::OFF_AT;                      // t-adjoint A operand
-    float* s_ge = reinterpret_cast<float*>(smem + G::OFF_GE);    // [3][P][16]
+    float* s_ge = reinterpret_cast<float*>(smem + G::OFF_GE);    // [3][P][16] (set-up only)
     float4* s_out = reinterpret_cast<float4*>(smem + G::OFF_L1);  // [P][16]: scaled gE of the three maps, kink band squared
     const float* s_wt = reinterpret_cast<const float*>(s_tab + G::TAB_WT);
     // mbarriers (arrival counts): [0], [1] forward buffer full (MMA commit); [2], [3] forward buffer read

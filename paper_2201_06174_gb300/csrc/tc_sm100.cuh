@@ -146,6 +146,29 @@ __device__ __forceinline__ void tmem_ld16x2(uint32_t taddr, uint32_t step, float
     }
 }
 
+// 32 lanes x 32 consecutive columns in 8 x 8 blocks: r[16 h + 4 c + 2 g + e] of thread t is lane 16 h + 8 g + t / 4 of the
+// warp's quarter, column 8 c + 2 (t % 4) + e (the fragment layout of the 8 x 8 matrix stores).
+__device__ __forceinline__ void tmem_ld32_blocks(uint32_t taddr, uint32_t (&r)[32]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        asm volatile(
+            "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+            "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+            : "=r"(r[16 * h + 0]), "=r"(r[16 * h + 1]), "=r"(r[16 * h + 2]), "=r"(r[16 * h + 3]), "=r"(r[16 * h + 4]),
+              "=r"(r[16 * h + 5]), "=r"(r[16 * h + 6]), "=r"(r[16 * h + 7]), "=r"(r[16 * h + 8]), "=r"(r[16 * h + 9]),
+              "=r"(r[16 * h + 10]), "=r"(r[16 * h + 11]), "=r"(r[16 * h + 12]), "=r"(r[16 * h + 13]),
+              "=r"(r[16 * h + 14]), "=r"(r[16 * h + 15])
+            : "r"(taddr + ((uint32_t)(16 * h) << 16)));
+    tmem_wait_ld(r);
+}
+
+// Four 8 x 8 blocks of 16-bit values, transposed: the 16-byte row at lane l's address is column l % 8 of block l / 8.
+__device__ __forceinline__ void store_blocks_trans(uint32_t saddr, uint32_t b0, uint32_t b1, uint32_t b2, uint32_t b3) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(saddr), "r"(b0), "r"(b1),
+                 "r"(b2), "r"(b3)
+                 : "memory");
+}
+
 // Asynchronous form: issue the load; the registers are valid only after tmem_wait_ld on them.
 __device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(

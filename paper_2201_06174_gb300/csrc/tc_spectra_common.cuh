@@ -38,7 +38,7 @@ namespace tcs {
 using f32::Tw;
 
 constexpr int kBY = 16;                 // outputs per CTA along y
-constexpr int kKRows = kBY + 15;        // K rows of the stage-3 A operand: window start + 16 taps
+constexpr int kKRows = kBY + 16;        // K rows of the stage-3 A operand: window start + 16 taps, a multiple of 8
 constexpr int kXHP = 24;                // halo rows along x staged (>= P + n - 1, multiple of 8)
 constexpr int kK2 = 2 * kXHP;           // stage-2 K: 24 cos taps + 24 sin taps
 constexpr uint32_t kWaitLimit = 1u << 22;
@@ -425,16 +425,24 @@ __device__ void d1_to_b2(uint32_t tmem, unsigned char* s_b2, int q, int lane, in
     }
 }
 
-// D2 (tensor memory columns [0, N2)) -> the stage-3 A operands: part 0 = real columns, 1 = imaginary.
+// D2 (tensor memory columns [0, N2)) -> the stage-3 A operands: part 0 = real columns, 1 = imaginary.  8 (rows) x 8 (y)
+// blocks, stored transposed: four stores of 512 bytes instead of one of 2 bytes a lane for each y.
 template <int N, int FMT>
 __device__ void d2_to_a3(uint32_t tmem, unsigned char* s_are, unsigned char* s_aim, int q, int lane, int part) {
     using G = FwdGeo<N>;
-    float v[32];
-    tc::tmem_ld32(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(part * G::YP), v);
-    const int m = 32 * q + lane;
-    unsigned char* dst = (part ? s_aim : s_are) + (m / 8) * G::SBO_A3 + (m % 8) * 2;
+    uint32_t r[32];
+    tc::tmem_ld32_blocks(tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(part * G::YP), r);
+    const uint32_t dst = tc::smem_u32(part ? s_aim : s_are) + (uint32_t)(4 * q * G::SBO_A3 + lane * 16);
 #pragma unroll
-    for (int y = 0; y < G::YH; ++y) *reinterpret_cast<uint16_t*>(dst + y * 16) = Pack<FMT>::one(v[y]);
+    for (int g = 0; g < 4; ++g) {   // rows 32 q + 8 g ..
+        uint32_t b[4];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {   // y 8 c ..; rows past the halo's stay zero
+            const int i = 16 * (g / 2) + 4 * c + 2 * (g % 2);
+            b[c] = 8 * c < G::YP ? Pack<FMT>::two(__uint_as_float(r[i]), __uint_as_float(r[i + 1])) : 0u;
+        }
+        tc::store_blocks_trans(dst + (uint32_t)(g * G::SBO_A3), b[0], b[1], b[2], b[3]);
+    }
     tc::fence_async_smem();
 }
 
