@@ -19,7 +19,7 @@
 // those of P - 3 and before are.
 // Bound: latency between the passes (about 12 k cycles a k_t tile, of which the MUFU pipe needs 4.1 k for the 17,408
 // square roots a voxel, the MMAs 3 to 4 k, and a group's four epilogues take 6.4 k); stage 1 takes 30 k of 235 k cycles a
-// brick.  64 x 96 x 96: 12.4 -> 6.9 ms (before: CTA-wide barriers around every pass, the FP32 sums of stage 1 again for
+// brick.  64 x 96 x 96: 12.4 -> 6.6 ms (before: CTA-wide barriers around every pass, the FP32 sums of stage 1 again for
 // every k_t, a maximum pass over every brick, operands laid out in 2-byte pieces with a division each).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -299,10 +299,19 @@ k1_spectra_tc32(const float* __restrict__ V, float* __restrict__ E, int T, int X
 #pragma unroll
                 for (int i = 0; i < YH - 32; ++i) *reinterpret_cast<uint16_t*>(dst + (32 + i) * 16) = Pack<FMT>::one(v[i]);
             } else {
-                float v[32];
-                tc::tmem_ld32(col, v);
+                uint32_t r[32];   // 8 (rows) x 8 (y) blocks, stored transposed
+                tc::tmem_ld32_blocks(col, r);
+                const uint32_t d = tc::smem_u32(s_a3 + (size_t)(2 * (kt & 1) + grp) * A_B) + (uint32_t)(4 * q * SBO_A + lane * 16);
 #pragma unroll
-                for (int i = 0; i < 32; ++i) *reinterpret_cast<uint16_t*>(dst + i * 16) = Pack<FMT>::one(v[i]);
+                for (int g = 0; g < 4; ++g) {
+                    uint32_t b[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        const int i = 16 * (g / 2) + 4 * c + 2 * (g % 2);
+                        b[c] = Pack<FMT>::two(__uint_as_float(r[i]), __uint_as_float(r[i + 1]));
+                    }
+                    tc::store_blocks_trans(d + (uint32_t)(g * SBO_A), b[0], b[1], b[2], b[3]);
+                }
             }
             tc::fence_async_smem();
         }
