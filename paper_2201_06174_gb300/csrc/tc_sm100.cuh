@@ -162,6 +162,22 @@ __device__ __forceinline__ void tmem_ld32_blocks(uint32_t taddr, uint32_t (&r)[3
     tmem_wait_ld(r);
 }
 
+// The same for 16 columns: r[8 h + 4 c + 2 g + e].
+__device__ __forceinline__ void tmem_ld16_blocks(uint32_t taddr, uint32_t (&r)[16]) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        asm volatile("tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                     : "=r"(r[8 * h + 0]), "=r"(r[8 * h + 1]), "=r"(r[8 * h + 2]), "=r"(r[8 * h + 3]),
+                       "=r"(r[8 * h + 4]), "=r"(r[8 * h + 5]), "=r"(r[8 * h + 6]), "=r"(r[8 * h + 7])
+                     : "r"(taddr + ((uint32_t)(16 * h) << 16)));
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                   "+r"(r[15])
+                 :
+                 : "memory");
+}
+
 // Four 8 x 8 blocks of 16-bit values, transposed: the 16-byte row at lane l's address is column l % 8 of block l / 8.
 __device__ __forceinline__ void store_blocks_trans(uint32_t saddr, uint32_t b0, uint32_t b1, uint32_t b2, uint32_t b3) {
     asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1,%2,%3,%4};" ::"r"(saddr), "r"(b0), "r"(b1),

@@ -64,7 +64,8 @@ template <int N, bool WIDE = false> struct FwdGeo {
     static constexpr uint32_t BLK_A1 = 16 * SBO_A1;           // 128 positions
     static constexpr size_t A1_B = (size_t)NB1 * BLK_A1;
     static constexpr uint32_t SBO_B2 = SBO_K2 + 16;      // MN-major B2: 8-column groups, one 16-byte row apart in the banks
-    static constexpr size_t B2_B = (size_t)N2 / 8 * SBO_B2;   // one k_t tile
+    // one k_t tile, 16 bytes on in the banks from the last: the 8 rows of a transposed store are of 8 tiles
+    static constexpr size_t B2_B = ((size_t)N2 / 8 * SBO_B2 + 111) / 128 * 128 + 16;
     static constexpr size_t B2ALL_B = (size_t)H * B2_B;
     static constexpr size_t R0_B = ((A1_B > B2ALL_B ? A1_B : B2ALL_B) + 127) / 128 * 128;  // A1, then B2 tiles
     // forward constant operands: [A2 | B1 | B3a | B3b | Eq. 1 weight table]
@@ -395,32 +396,45 @@ __device__ float stage_brick(const float* __restrict__ V, int T, int X, int Y, i
 
 // D1 (tensor memory columns [16 i, 16 i + 16) of stage-1 block i) -> one stage-2 B tile per k_t.
 // Blocks i = grp, grp + ngrp, ... are read by the warps of group grp (lane quarter q).
+// B2 is MN-major: byte(ncol, k2) = (ncol/8) SBO_B2 + k2 16 + (ncol%8) 2, so the 8 x 8 blocks of D1 (8 y of one x, 8 columns
+// of stage 1) are stored transposed: block column c, cos k_t or sin k_t, becomes the 16-byte row of its tile's x.  G1r goes
+// to (re, cos) and negated to (im, sin), G1i = -sin to (re, sin) and (im, cos); for k_t = 0 and n/2 it is 0.
 template <int N, int FMT>
 __device__ void d1_to_b2(uint32_t tmem, unsigned char* s_b2, int q, int lane, int grp, int ngrp) {
     using G = FwdGeo<N>;
     constexpr int H = G::H, YP = G::YP;
+    constexpr uint32_t kIm = YP / 8 * G::SBO_B2, kSin = kXHP * 16;
+    static_assert(kXHP * YP % 32 == 0, "whole warps of positions");
     const uint32_t lane_base = (uint32_t)(32 * q) << 16;
+    const uint32_t b2 = tc::smem_u32(s_b2);
     for (int i = grp; i < G::NB1; i += ngrp) {
-        float v[32];
-        tc::tmem_ld32(tmem + lane_base + (uint32_t)(16 * i), v);   // columns 16 i .. 16 i + 15 used
-        const int pos = 128 * i + 32 * q + lane;
-        const int x = pos / YP, y = pos % YP;
-        if (x < kXHP) {
-            // MN-major: byte(ncol, k2) = (ncol/8) SBO_B2 + k2 16 + (ncol%8) 2: the 32 y of a warp's store lie in 4
-            // rows that share no bank (K-major rows, one y each, met in 8 banks: 4 passes a store)
-            const size_t o_re = (size_t)(y / 8) * G::SBO_B2 + (y % 8) * 2;
-            const size_t o_im = (size_t)((YP + y) / 8) * G::SBO_B2 + (y % 8) * 2;
-            const size_t k_c = (size_t)x * 16, k_s = (size_t)(kXHP + x) * 16;
+        const int pos = 128 * i + 32 * q;
+        if (pos >= kXHP * YP) break;   // (warp-uniform)
+        uint32_t r[16];
+        tc::tmem_ld16_blocks(tmem + lane_base + (uint32_t)(16 * i), r);
+        // this lane's row address: positions pos + 8 (lane / 8) .., one x; block column lane % 8
+        const int p8 = pos + lane / 8 * 8, x = p8 / YP, y = p8 % YP, j = lane % 8;
+        const uint32_t at = b2 + (uint32_t)(y / 8 * G::SBO_B2 + x * 16);
 #pragma unroll
-            for (int kt = 0; kt < H; ++kt) {
-                const float g1r = v[kt];
-                const float g1i = (kt == 0 || 2 * kt == N) ? 0.f : -v[H - 1 + kt];
-                unsigned char* b2 = s_b2 + (size_t)kt * G::B2_B;
-                *reinterpret_cast<uint16_t*>(b2 + o_re + k_c) = Pack<FMT>::one(g1r);
-                *reinterpret_cast<uint16_t*>(b2 + o_re + k_s) = Pack<FMT>::one(g1i);
-                *reinterpret_cast<uint16_t*>(b2 + o_im + k_c) = Pack<FMT>::one(g1i);
-                *reinterpret_cast<uint16_t*>(b2 + o_im + k_s) = Pack<FMT>::one(-g1r);
+        for (int c = 0; c < N / 8; ++c) {
+            uint32_t v[4], w[4];
+            const int c0 = 8 * c + 2 * (lane % 4);   // this lane's values are of columns c0 and c0 + 1
+            const uint32_t flip = (c0 >= H ? 0x8000u : 0u) | (c0 + 1 >= H ? 0x80000000u : 0u);
+#pragma unroll
+            for (int g = 0; g < 4; ++g) {
+                const int k = 8 * (g / 2) + 4 * c + 2 * (g % 2);
+                const uint32_t f = Pack<FMT>::two(__uint_as_float(r[k]), __uint_as_float(r[k + 1]));
+                v[g] = f ^ flip;
+                w[g] = f ^ 0x80008000u;
             }
+            const bool cs = 8 * c + j < H;
+            const uint32_t tile = at + (uint32_t)(cs ? 8 * c + j : 8 * c + j - H + 1) * (uint32_t)G::B2_B;
+            tc::store_blocks_trans(tile + (cs ? 0u : kSin), v[0], v[1], v[2], v[3]);
+            tc::store_blocks_trans(tile + kIm + (cs ? kSin : 0u), w[0], w[1], w[2], w[3]);
+        }
+        if (j < 4) {   // G1i of k_t = 0 (j = 0, 1) and n/2 (j = 2, 3)
+            const uint32_t z = at - b2 + (j & 2 ? (uint32_t)((H - 1) * G::B2_B) : 0u) + (j & 1 ? kIm : kSin);
+            *reinterpret_cast<uint4*>(s_b2 + z) = make_uint4(0u, 0u, 0u, 0u);
         }
     }
 }
