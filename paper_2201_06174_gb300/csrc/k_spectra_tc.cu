@@ -48,6 +48,24 @@ __global__ void k1_tc_tables(const __grid_constant__ Tw<N> tw, unsigned char* __
     tcs::build_fwd_tables<N, FMT, true>(tw, out, threadIdx.x, blockDim.x, feat);
 }
 
+// CNT sums in each of 2 W neighbouring lanes -> this lane's share of their totals in v[0 ..]; returns the first one's index.
+template <int W, int CNT>
+__device__ __forceinline__ int fold_lanes(float (&v)[24], int lane) {
+    if constexpr (W == 0) {
+        return 0;
+    } else {
+        constexpr int KEEP = (CNT + 1) / 2;
+        const bool up = (lane & W) != 0;
+#pragma unroll
+        for (int i = 0; i < KEEP; ++i) {
+            const float hi = KEEP + i < CNT ? v[KEEP + i] : 0.f;
+            const float got = __shfl_xor_sync(0xffffffffu, up ? v[i] : hi, W);
+            v[i] = (up ? hi : v[i]) + got;
+        }
+        return (up ? KEEP : 0) + fold_lanes<W / 2, KEEP>(v, lane);
+    }
+}
+
 // EN: the energy reading of the feature (|F|^2 per bin; the weight table then holds r_m^2)
 template <int N, int FMT, bool EN>
 __global__ void __launch_bounds__(kThreads, 2)
@@ -328,31 +346,28 @@ k1_spectra_tc(const float* __restrict__ V, float* __restrict__ E, int T, int X, 
     // E: [3][T][X][Y], or the lattice [3][Tc][Xc][Yc] (ceil(T / s) ...) for stride s > 1
     const int Xc = (X + stride - 1) / stride, Yc = (Y + stride - 1) / stride;
     const size_t NV = (size_t)((T + stride - 1) / stride) * Xc * Yc;
-    const int x = xb + x0l;
     const bool good = *s_fail == 0 && warp < kConsumers;   // the producer warp holds no results
     const float out_scale = EN ? scale * scale : scale;     // the features of the unscaled brick
+    // each exchange halves the sums a lane holds: bit b of k_x decides which half it keeps (23 or 21 shuffles and two or three
+    // stores a lane, against 24 sums of 3 or 4 shuffles each and 24 stores of one lane in n)
+    float v[24];
 #pragma unroll
-    for (int pass = 0; pass < G::PASSES; ++pass)
+    for (int i = 0; i < 24; ++i) v[i] = acc[i / 3][i % 3];
+    constexpr int kLeft = N == 16 ? 2 : 3;
+    const int first = fold_lanes<N / 2, 24>(v, kx);
+    const int x = xb + x0l;
 #pragma unroll
-        for (int cc = 0; cc < 2; ++cc)
-#pragma unroll
-            for (int o = 0; o < G::OPC; ++o) {
-                const int slot = (pass * 2 + cc) * G::OPC + o;
-                const int y0 = pass * G::OPP + (half + 2 * cc) * G::OPC + o;
-#pragma unroll
-                for (int c = 0; c < 3; ++c) {
-                    float s = acc[slot][c];
-#pragma unroll
-                    for (int w = 1; w < N; w <<= 1) s += __shfl_xor_sync(0xffffffffu, s, w);
-                    const int y = yb + y0;
-                    if (kx == 0 && x < X && y < Y && good) {
-                        if (stride == 1)
-                            E[c * NV + ((size_t)t0 * X + x) * Y + y] = s * out_scale;
-                        else if (x % stride == 0 && y % stride == 0)   // the lattice (a rare path)
-                            E[c * NV + ((size_t)(t0 / stride) * Xc + x / stride) * Yc + y / stride] = s * out_scale;
-                    }
-                }
-            }
+    for (int i = 0; i < kLeft; ++i) {
+        const int id = first + i, c = id % 3, slot = id / 3;
+        const int y = yb + slot / (2 * G::OPC) * G::OPP + (half + 2 * (slot / G::OPC % 2)) * G::OPC + slot % G::OPC;
+        const bool extra = N == 16 && i == 1 && (kx & 1);   // 3 sums over 2 lanes
+        if (!extra && x < X && y < Y && good) {
+            if (stride == 1)
+                E[c * NV + ((size_t)t0 * X + x) * Y + y] = v[i] * out_scale;
+            else if (x % stride == 0 && y % stride == 0)   // the lattice (a rare path)
+                E[c * NV + ((size_t)(t0 / stride) * Xc + x / stride) * Yc + y / stride] = v[i] * out_scale;
+        }
+    }
     tc::fence_before_sync();
     __syncthreads();
     if (warp == 0) tc::tmem_dealloc(tmem, kTmemCols);
