@@ -314,6 +314,16 @@ __device__ float stage_brick(const float* __restrict__ V, int T, int X, int Y, i
     const float* stg = reinterpret_cast<const float*>(s_stage);
     const bool interior = t0 - N / 2 >= 0 && t0 + N / 2 <= T && xb - N / 2 >= 0 && xb - N / 2 + XH <= X && ty >= 0 &&
                           ty + YP <= Y;
+    // a border brick: its y samples by the extension, once for all of a thread's items where these have one y8
+    constexpr bool kOneY = NT % YG == 0 && (G::NB1 * 16) % YG == 0;
+    const bool y_inside = ty >= 0 && ty + YP <= Y;
+    int gy[8];
+    auto extend_y = [&](int y8) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            gy[i] = y_inside ? ty + y8 + i : y8 + i < YH ? ext_index(ty + y8 + i, Y, bnd) : -1;
+    };
+    if (kOneY && !tma && !interior) extend_y(8 * (tid % YG));
     float vals[PER][8];
     float vmax = 0.f;
     bool bad = false;
@@ -350,10 +360,12 @@ __device__ float stage_brick(const float* __restrict__ V, int T, int X, int Y, i
         } else {
             const int gt = ext_index(t0 - N / 2 + u, T, bnd);
             const int gx = ext_index(xb - N / 2 + x, X, bnd);
+            if (!kOneY) extend_y(y8);
+            if (live && (gt | gx) >= 0) {
+                const float* row = V + ((size_t)gt * X + gx) * Y;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int gy = ext_index(ty + y8 + i, Y, bnd);
-                if (live && y8 + i < YH && (gt | gx | gy) >= 0) vals[r][i] = __ldg(V + ((size_t)gt * X + gx) * Y + gy);
+                for (int i = 0; i < 8; ++i)
+                    if (gy[i] >= 0) vals[r][i] = __ldg(row + gy[i]);
             }
         }
 #pragma unroll
