@@ -16,7 +16,7 @@
 // Bound: the MUFU pipe, n^3/2 + n^2/2 roots per voxel at 16 per clock and SM (n = 16: 0.90 ms at 128^3), with about
 // 110 issue slots per thread and output for its 16 bins beside 128 MUFU cycles.  The 48 sums, 16 bins and 27 weights
 // take 168 registers a thread: 12 warps per SM, whose 16 independent bins each hide the latencies.
-// 128^3: n = 16 7.23 -> 2.18 ms, n = 8 1.07 -> 0.31 ms; 48 x 64 x 64, n = 32: 21.2 -> 3.2 ms (before: direct DFTs in
+// 128^3: n = 16 7.23 -> 2.07 ms, n = 8 1.07 -> 0.28 ms; 48 x 64 x 64, n = 32: 21.2 -> 2.7 ms (before: direct DFTs in
 // stages 1 and 2 and for each run's first output, a halo for every row of 32 outputs, a six-operation rotation
 // per bin and output).  Error against FP64, relative L2 of E: 7e-8, 6e-8 and 8e-8 (before 1.3e-7, 7e-8 and 1.3e-7).
 // The brick is staged minus one of its voxels: only the DC bin of a rect cube moves, which Eq. 1 leaves out, so a
@@ -175,10 +175,11 @@ __device__ __forceinline__ float brick_shift(const float* __restrict__ p) {
     return isfinite(v) ? v : 0.f;
 }
 
-// Halo position (x, y) of the brick: the n samples of its column along t, minus vshift.
+// Halo position (x, y) of the brick: the n samples of its column along t, minus vshift.  s_gt: the planes of the n taps by
+// the border extension (each column of a brick at the volume's first or last planes would find them again).
 template <int N>
-__device__ __forceinline__ void load_column(const float* __restrict__ V, int T, int X, int Y, int bnd, int t0, int gx,
-                                            int gy, float vshift, float (&v)[N]) {
+__device__ __forceinline__ void load_column(const float* __restrict__ V, int T, int X, int Y, int t0,
+                                            const int* __restrict__ s_gt, int gx, int gy, float vshift, float (&v)[N]) {
     const bool in = (gx | gy) >= 0;
     const float* p = V + (in ? (size_t)gx * Y + gy : 0);
     const size_t plane = (size_t)X * Y;
@@ -189,7 +190,7 @@ __device__ __forceinline__ void load_column(const float* __restrict__ V, int T, 
     } else {
 #pragma unroll
         for (int u = 0; u < N; ++u) {
-            const int gt = ext_index(t0 - N / 2 + u, T, bnd);
+            const int gt = s_gt[u];
             v[u] = (in && gt >= 0 ? __ldg(p + gt * plane) : 0.f) - vshift;
         }
     }
@@ -207,13 +208,16 @@ k1_slide(const float* __restrict__ V, float* __restrict__ E, int T, int X, int Y
     float2* s_g2 = s_g1 + G::G1 + grp * G::G2;            // [x0][k_x][y] of the group's current tile
     auto group_sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + grp), "n"(G::GT) : "memory"); };
     const int yb = blockIdx.x * G::BY, xb = blockIdx.y * RX, t0 = blockIdx.z;
+    __shared__ int s_gt[N];
+    if (tid < N) s_gt[tid] = ext_index(t0 - N / 2 + tid, T, bnd);
+    __syncthreads();
     const float vshift = brick_shift(V + ((size_t)t0 * X + xb) * Y + yb);
 
     for (int it = tid; it < XH * YH; it += G::NT) {
         const int x = it / YH, y = it - x * YH;
         float v[N];
         float2 o[N / 2];
-        load_column<N>(V, T, X, Y, bnd, t0, ext_index(xb - N / 2 + x, X, bnd), ext_index(yb - N / 2 + y, Y, bnd),
+        load_column<N>(V, T, X, Y, t0, s_gt, ext_index(xb - N / 2 + x, X, bnd), ext_index(yb - N / 2 + y, Y, bnd),
                        vshift, v);
         f32::rfft<N>(v, o);
 #pragma unroll
@@ -322,6 +326,9 @@ k1_slide32(const float* __restrict__ V, float* __restrict__ E, int T, int X, int
     __shared__ float s_odd[RX][3][RUN];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int yb = blockIdx.x * BY, xb = blockIdx.y * RX, t0 = blockIdx.z;
+    __shared__ int s_gt[N];
+    if (tid < N) s_gt[tid] = ext_index(t0 - N / 2 + tid, T, bnd);
+    __syncthreads();
     const float vshift = brick_shift(V + ((size_t)t0 * X + xb) * Y + yb);
     const int x0l = warp >> 1, odd = warp & 1;
 
@@ -329,7 +336,7 @@ k1_slide32(const float* __restrict__ V, float* __restrict__ E, int T, int X, int
         for (int it = tid; it < XH * YH; it += NT) {
             const int x = it / YH, y = it - x * YH;
             float v[N];
-            load_column<N>(V, T, X, Y, bnd, t0, ext_index(xb - N / 2 + x, X, bnd), ext_index(yb - N / 2 + y, Y, bnd),
+            load_column<N>(V, T, X, Y, t0, s_gt, ext_index(xb - N / 2 + x, X, bnd), ext_index(yb - N / 2 + y, Y, bnd),
                            vshift, v);
             if (g == 0) tiles4<0>(v, s_g1 + it, XH * YH);
             else if (g == 1) tiles4<4>(v, s_g1 + it, XH * YH);

@@ -19,7 +19,7 @@
 // those of P - 3 and before are.
 // Bound: latency between the passes (about 12 k cycles a k_t tile, of which the MUFU pipe needs 4.1 k for the 17,408
 // square roots a voxel, the MMAs 3 to 4 k, and a group's four epilogues take 6.4 k); stage 1 takes 30 k of 235 k cycles a
-// brick.  64 x 96 x 96: 12.4 -> 6.6 ms (before: CTA-wide barriers around every pass, the FP32 sums of stage 1 again for
+// brick.  64 x 96 x 96: 12.4 -> 6.3 ms (before: CTA-wide barriers around every pass, the FP32 sums of stage 1 again for
 // every k_t, a maximum pass over every brick, operands laid out in 2-byte pieces with a division each).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -186,6 +186,8 @@ k1_spectra_tc32(const float* __restrict__ V, float* __restrict__ E, int T, int X
     for (int i = tid; i < (int)(B2_B / 16); i += kThreads)
         reinterpret_cast<uint4*>(s_b2)[i] = make_uint4(0u, 0u, 0u, 0u);
 
+    __shared__ int s_gt[N];   // the planes of the taps
+    if (warp == 1) s_gt[lane] = ext_index(t0 - N / 2 + lane, T, bnd);
     // ---- the brick's maximum, over the planes' -----------------------------------------------------------
     if (warp == 0) {
         const int gt = ext_index(t0 - N / 2 + lane, T, bnd);
@@ -219,7 +221,7 @@ k1_spectra_tc32(const float* __restrict__ V, float* __restrict__ E, int T, int X
         } else {
 #pragma unroll
             for (int u = 0; u < N; ++u) {
-                const int gt = ext_index(t0 - N / 2 + u, T, bnd);
+                const int gt = s_gt[u];
                 v[u] = in && gt >= 0 ? __ldg(p + gt * plane) : 0.f;
             }
         }
