@@ -16,7 +16,7 @@
 // The instruction cache sets how far the loop over outputs is unrolled: by 8 (w^(k (j + 8)) = +-w^(k j) for n = 16), and
 // not at all in tile 0, whose packed rows need the most code for an eighth of the work (there every window is an FFT).
 // Bound: issue slots, about 450 per thread and output of 16 bins with the FFTs and the small bins (128 MUFU cycles), 54 %
-// of them used by 12 warps an SM at 168 registers.  The adjoint call, 128^3: n = 16 25.0 -> 6.4 ms, n = 8 2.54 -> 0.98
+// of them used by 12 warps an SM at 168 registers.  The adjoint call, 128^3: n = 16 25.0 -> 6.1 ms, n = 8 2.54 -> 0.98
 // (before: one x0 per brick, direct DFTs in stages 1 and 2 and both of their adjoints, 31 point evaluations of 32
 // multiply-adds per run of 8 outputs, and two passes over the grid for the small bins, 0.1 per voxel here); 24^3, n = 16:
 // 353 -> 180 us.  Error against FP64 9.9e-7 -> 9.8e-7 (n = 16), 8.0e-7 -> 8.8e-7 (n = 8), most of it in the directions
@@ -142,12 +142,13 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
         const int m = i / (RX * kRun), x = xb + (i / kRun) % RX, y = yb + i % kRun;
         s_ge[i] = x < X && y < Y ? __ldg(gE + m * NV + ((size_t)t0 * X + x) * Y + y) : 0.f;
     }
+    group_sync();   // s_src
     float* s_col = reinterpret_cast<float*>(s_g2);   // [x][y], before the first tile's G2
     float* s_row = s_col + XH * YH;                  // [x][j]
     const bool t_in = t0 - N / 2 >= 0 && t0 + N / 2 <= T;
     for (int it = tid; it < XH * YH; it += GT) {
         const int x = it / YH, y = it - x * YH;
-        const int gx = ext_index(xb - N / 2 + x, X, bnd), gy = ext_index(yb - N / 2 + y, Y, bnd);
+        const int gx = s_src[N + x], gy = ext_index(yb - N / 2 + y, Y, bnd);
         const bool in = (gx | gy) >= 0;
         const float* p = V + (in ? (size_t)gx * Y + gy : 0);
         float v[N], a = 0.f;
@@ -159,7 +160,7 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
         } else {
 #pragma unroll
             for (int u = 0; u < N; ++u) {
-                const int gt = ext_index(t0 - N / 2 + u, T, bnd);
+                const int gt = s_src[u];
                 v[u] = in && gt >= 0 ? __ldg(p + gt * plane) : 0.f;
             }
         }
