@@ -79,16 +79,17 @@ def op_rates():
                      for k, v in PEAKS["mufu"].items())
 # K1 DRAM traffic per launch (bytes) from an ncu capture of the same kernel and workload;
 # None until captured for the current kernel.
-K1_TRAFFIC = {("salt128", 16, "fp32"): 8711168,   # sliding, 32-output form; profiles/salt128_n16_fp32_fwd_bwd.md
-              ("salt128", 16, "bf16"): 8546816,   # profiles/salt128_n16_bf16_fwd_bwd.md (per launch)
+K1_TRAFFIC = {("salt128", 16, "fp32"): 8498688,   # profiles/kernels_128cubed_n16.md (per launch)
+              ("salt128", 16, "bf16"): 8518400,
               # one-pass capture of the full-scale launch (1.56 GB read + 3.39 GB written: ncu's 3-digit
               # figures); profiles/full462x951x651_n16_bf16_fwd_bwd.md
               ("full462x951x651", 16, "bf16"): 4950000000}
-# K5 alone (the brick blocks it writes dominate): 34.7 MB read + 689.5 MB written per 128^3 launch of 16,384
-# bricks (profiles/salt128_n16_bf16_fwd_bwd.md); a brick's traffic does not depend on the volume, so the
+# K5 alone (the brick blocks it writes dominate): 41.7 MB read + 685.8 MB written per 128^3 launch of 16,384
+# bricks (profiles/kernels_128cubed_n16.md); a brick's traffic does not depend on the volume, so the
 # full-scale call (2,254,098 bricks over its t-slab launches) is that per-brick figure times its bricks.
-K5_TRAFFIC = {("salt128", 16, "bf16"): 724247040,
-              ("full462x951x651", 16, "bf16"): 99641345482}
+K5_TRAFFIC = {("salt128", 16, "bf16"): 727448576,
+              ("salt128", 16, "fp32"): 579679232,
+              ("full462x951x651", 16, "bf16"): 100081810319}
 
 
 def measured_peaks():
@@ -116,12 +117,15 @@ def mma_per_brick(kind: str, n: int):
     yp = 8 * -(-(16 + n - 1) // 8)
     nb1 = -(-(24 * yp) // 128)
     fwd = [(nb1, 16), (3 * h, 2 * yp), (32 * h, 2 * n)]
+    if kind == "k1_wide":   # K1-TC: one MMA of N = 128 per part, pass of 64 / n outputs and 16 K rows
+        outs = 64 // n
+        return fwd[:2] + [(2 * (16 // outs) * (1 if n + outs - 1 <= 16 else 2) * h, 128)]
     return fwd if kind == "k1" else fwd + [(32 * h, 32), (16 * h, 64), (nb1 * h, 16)]
 
 
 def tensor_issue(kind: str, n: int, shape, ms: float):
     """The tensor pipe's instruction floor of a tensor-core kernel: its MMAs per brick at the measured cost per
-    MMA of each width (sal_measure_mma_rate; a width above 64 taken at the 64-column cost), the bricks spread
+    MMA of each width (sal_measure_mma_rate; a width above the measured ones taken at the 64-column cost), the bricks spread
     evenly over the SMs at the max SM clock; frac = floor / measured time."""
     cyc = PEAKS.get("mma_cycles")
     if not cyc or n not in (8, 16):
@@ -138,8 +142,7 @@ def tensor_issue(kind: str, n: int, shape, ms: float):
 
 def roofline(kernel, prec, n, nvox, ms, flops_mult, traffic, mufu_op="sqrt", feature="abs", flops_per_voxel=None):
     """Roofline of a spectral kernel.  FP32 form: its contraction flops (the per-voxel figure
-    4hn + 8hn^2 + 8hn^3, x2 for the adjoint; the sliding form's own count where it runs) on the FP32
-    FMA pipe.  BF16/FP16 form: the
+    4hn + 8hn^2 + 8hn^3, x2 for the adjoint) on the FP32 FMA pipe; where it slides, roots_roofline.  BF16/FP16 form: the
     contraction runs on the tensor cores (reported as `tensor`), and the binding pipe is the
     abs(F) epilogue, h n^2 square roots per voxel on the MUFU pipe; with the energy reading of the
     feature there is no root, and the epilogue's FP32 arithmetic (about 4 FMA-pipe operations per
@@ -167,6 +170,28 @@ def roofline(kernel, prec, n, nvox, ms, flops_mult, traffic, mufu_op="sqrt", fea
     return {"kernel": kernel, "bound": "alu", "pipe": f"MUFU ({what})", "achieved": bins,
             "peak": pk, "unit": f"T{mufu_op}/s", "frac": bins / pk, "traffic": traffic,
             "peak_note": PEAKS["mufu_note"], "tensor": tensor}
+
+
+def f32_roots_per_voxel(n: int) -> int:
+    """Square roots per voxel of the FP32 kernels' tiled half spectrum (rect taper, stride 1): n/2 tiles of n^2 bins,
+    the first of which holds k_t = 0 and n/2 in one, with their self-paired rows' bins apart."""
+    return n ** 3 // 2 + n ** 2 // 2
+
+
+def roots_roofline(kernel, n, nvox, ms, traffic, op, feature="abs"):
+    """Roofline of the FP32 kernels that slide along y: their roots on the MUFU pipe, at its measured rate; with the
+    energy reading, which takes none, about 4 FMA-pipe operations per bin, as for the tensor-core forms."""
+    form = "sliding DFT along y over n/2 tiles of the half spectrum"
+    if feature == "energy":
+        ops, pk = 4.0 * f32_roots_per_voxel(n) * nvox / (ms / 1e3) / 1e12, PEAKS["fma_tops"]
+        return {"kernel": kernel, "bound": "alu", "pipe": "FP32 FMA (energy: ~4 operations per bin)", "achieved": ops,
+                "peak": pk, "unit": "Tops/s", "frac": ops / pk, "traffic": traffic,
+                "peak_note": f"{PEAKS['sms']} SM x 128 lanes x {PEAKS['sm_ghz']:.2f} GHz", "form": form}
+    rate = f32_roots_per_voxel(n) * nvox / (ms / 1e3) / 1e12
+    pk = PEAKS["mufu"].get(op, 16 * PEAKS["sms"] * PEAKS["sm_ghz"] * 1e9 / 1e12)
+    return {"kernel": kernel, "bound": "alu", "pipe": f"MUFU (one {op} per bin)", "achieved": rate, "peak": pk,
+            "unit": f"T{op}/s", "frac": rate / pk, "traffic": traffic, "peak_note": PEAKS["mufu_note"],
+            "form": form}
 
 
 def max_over_ranks(values, dist=None, device="cpu"):
@@ -198,20 +223,20 @@ def k1_flops_per_voxel_spatial(n: int, adjoint: bool = False) -> int:
     return lines * 5 * n * (n.bit_length() - 1)
 
 
-# Outputs per thread of the FP32 K1's sliding form (rect taper, stride 1): the first of each run by the
-# direct stage-3 sum, the others by the recursion.
+# A sliding form with direct sums along t and x, by outputs per run: the first of each run by the direct stage-3 sum, the
+# others by the recursion (a yardstick for the FP32 kernels, whose FFTs and tiles need less; the windows that slide).
 K1_F32_SLIDING_RUN = {8: 8, 16: 16, 32: 8}
 
 
 def k1_flops_per_voxel_sliding(n: int) -> int:
-    """Algorithmic flops per voxel of the FP32 K1's sliding form: stages along t and x as in the direct
+    """Algorithmic flops per voxel of that sliding form: stages along t and x as in the direct
     form (4hn + 8hn^2); along y one complex add and one complex rotation per bin and output (8hn^2),
     and the direct sum (8hn^3) for one output of each run."""
     h = n // 2 + 1
     return 4 * h * n + 8 * h * n * n + 8 * h * n * n + 8 * h * n ** 3 // K1_F32_SLIDING_RUN[n]
 
 
-K5_F32_SLIDING_RUN = {8: 4, 16: 8}   # outputs per thread run of the FP32 adjoint (its YC)
+K5_F32_SLIDING_RUN = {8: 4, 16: 8}   # the same yardstick for the adjoint (the windows whose adjoint slides)
 
 
 def k5_flops_per_voxel_sliding(n: int) -> int:
@@ -491,6 +516,7 @@ def main():
     if gpu_id and not gpu_id.startswith("GPU-"):
         gpu_id = "GPU-" + gpu_id
     set_alu_peaks(sal, dev_props.multi_processor_count, max_sm_clock_mhz(gpu_id))
+    PEAKS["mma_cycles"][128] = sal.sal_measure_mma_rate(128)[0]   # K1-TC's stage 3
     for _ in range(max(args.warmup, 3)):
         step()
     barrier()
@@ -674,32 +700,31 @@ def main():
     sliding = args.prec == "fp32" and sc == 1 and n in K1_F32_SLIDING_RUN and not spatial
     k1_rl = roofline("k1_spatial_f32" if spatial else f"k1_spectra_{tag}", args.prec, n, ncubes, k1_ms, 1,
                      K1_TRAFFIC.get(trk), feature=args.feature,
-                     flops_per_voxel=(k1_flops_per_voxel_spatial(n) if spatial else
-                                      k1_flops_per_voxel_sliding(n) if sliding else None))
+                     flops_per_voxel=k1_flops_per_voxel_spatial(n) if spatial else None)
     if sliding:
-        k1_rl["form"] = "sliding DFT along y (flops of that form)"
+        k1_rl = roots_roofline("k1_slide", n, ncubes, k1_ms, K1_TRAFFIC.get(trk), "sqrt", args.feature)
     if spatial:
         k1_rl["form"] = "spatial reading: per-window separable radix-2 FFTs in shared memory (flops of that form)"
     if sc > 1:
         k1_rl["cubes_per_launch"] = ncubes
     if args.prec != "fp32" and sc == 1 and not spatial and n in (8, 16):
-        k1_rl["tensor_issue"] = tensor_issue("k1", n, V.shape, k1_ms)
+        k1_rl["tensor_issue"] = tensor_issue("k1_wide", n, V.shape, k1_ms)
     if args.form == "fwdbwd":
         k5_ms = per_call[names.index("k5_local_spectra_project_backward")] / args.steps
         # the timed call is memset + K5 + the overlap-add gather; the traffic entry is K5's own
-        # the FP32 adjoint at n = 8, 16 runs both y-passes as sliding recursions (k5_flops_per_voxel_sliding);
-        # otherwise its flops are twice the direct forward's
+        # the FP32 adjoint at n = 8, 16 slides along y in both directions; otherwise its flops are twice the
+        # direct forward's
         k5_sliding = args.prec == "fp32" and n in K5_F32_SLIDING_RUN and not spatial
         k5_name = "k5_spatial_adjoint_f32" if spatial else f"k5_spectra_adjoint_{tag}"
         rl = roofline(f"{k5_name} (call incl. memset and the two overlap-add passes)", args.prec, n, nvox, k5_ms,
-                      1 if k5_sliding or spatial else 2, K5_TRAFFIC.get(trk),
+                      1 if spatial else 2, K5_TRAFFIC.get(trk),
                       mufu_op="rsqrt" if args.prec != "fp32" else "sqrt", feature=args.feature,
-                      flops_per_voxel=(k1_flops_per_voxel_spatial(n, adjoint=True) if spatial else
-                                       k5_flops_per_voxel_sliding(n) if k5_sliding else None))
+                      flops_per_voxel=k1_flops_per_voxel_spatial(n, adjoint=True) if spatial else None)
         if spatial:
             rl["form"] = "spatial reading's adjoint: forward recompute, signs, combined inverse (flops of that form)"
-        if k5_sliding:
-            rl["form"] = "forward recompute and inverse along y by sliding recursions (flops of that form)"
+        if k5_sliding:   # with a stride it computes the lattice planes
+            rl = roots_roofline("k5_slide (call incl. the two overlap-add passes)", n, -(-T_ // sc) * X_ * Y_, k5_ms,
+                                K5_TRAFFIC.get(trk), "rsqrt", args.feature)
         if args.prec != "fp32" and sc == 1 and n in (8, 16) and not spatial:
             rl["tensor_issue"] = tensor_issue("k5", n, V.shape, k5_ms)
         rl["k1"] = k1_rl
