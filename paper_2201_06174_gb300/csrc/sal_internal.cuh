@@ -39,8 +39,8 @@ struct TwiddleTable {
 
 enum : int { BND_SYMMETRIC = 0, BND_PERIODIC = 1, BND_ZERO = 2 };
 
-// Border extension of one axis; -1 where the zero extension applies.
-__host__ __device__ __forceinline__ int ext_index(int i, int n, int mode) {
+// Border extension of one axis; -1 where the zero extension applies.  Any distance, by a division.
+__host__ __device__ __forceinline__ int ext_index_any(int i, int n, int mode) {
     if ((unsigned)i < (unsigned)n) return i;
     if (mode == BND_PERIODIC) {
         int r = i % n;
@@ -51,6 +51,21 @@ __host__ __device__ __forceinline__ int ext_index(int i, int n, int mode) {
     int r = i % P;
     if (r < 0) r += P;
     return r < n ? r : P - 1 - r;
+}
+
+// The same, within one length of the axis (most windows and stencils) without a division: the FP32 call with a template on
+// 10 x 9 x 37 voxels 53.3 -> 51.8 us, small center-surround calls 1 to 2 %.  The tensor-core forms, which look few samples
+// up, keep the smaller code (their adjoint at 128^3: 5266 against 5289 us).
+__host__ __device__ __forceinline__ int ext_index(int i, int n, int mode) {
+    if ((unsigned)i < (unsigned)n) return i;
+    if (mode == BND_PERIODIC) {
+        if ((unsigned)(i + n) < (unsigned)n) return i + n;
+        if ((unsigned)(i - n) < (unsigned)n) return i - n;
+    } else if (mode == BND_SYMMETRIC) {
+        if ((unsigned)(-1 - i) < (unsigned)n) return -1 - i;
+        if ((unsigned)(2 * n - 1 - i) < (unsigned)n) return 2 * n - 1 - i;
+    }
+    return ext_index_any(i, n, mode);
 }
 
 // Scratch for the volume-wide reductions (device memory owned by the handle).

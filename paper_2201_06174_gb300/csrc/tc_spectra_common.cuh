@@ -321,7 +321,7 @@ __device__ float stage_brick(const float* __restrict__ V, int T, int X, int Y, i
     auto extend_y = [&](int y8) {
 #pragma unroll
         for (int i = 0; i < 8; ++i)
-            gy[i] = y_inside ? ty + y8 + i : y8 + i < YH ? ext_index(ty + y8 + i, Y, bnd) : -1;
+            gy[i] = y_inside ? ty + y8 + i : y8 + i < YH ? ext_index_any(ty + y8 + i, Y, bnd) : -1;
     };
     if (kOneY && !tma && !interior) extend_y(8 * (tid % YG));
     float vals[PER][8];
@@ -358,8 +358,8 @@ __device__ float stage_brick(const float* __restrict__ V, int T, int X, int Y, i
                 for (int i = 0; i < 8; ++i) vals[r][i] = __ldg(src + i);
             }
         } else {
-            const int gt = ext_index(t0 - N / 2 + u, T, bnd);
-            const int gx = ext_index(xb - N / 2 + x, X, bnd);
+            const int gt = ext_index_any(t0 - N / 2 + u, T, bnd);
+            const int gx = ext_index_any(xb - N / 2 + x, X, bnd);
             if (!kOneY) extend_y(y8);
             if (live && (gt | gx) >= 0) {
                 const float* row = V + ((size_t)gt * X + gx) * Y;
