@@ -1,0 +1,64 @@
+"""What one extreme value may touch in the FP32 forms that slide along y: an output (forward) or a sample (adjoint) whose
+windows do not hold it keeps the accuracy it has without it."""
+import numpy as np
+import pytest
+
+import oracle
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+# volumes large enough for the forward's long runs; brick corners (xb, yb) of the second brick along x and along y
+FORWARD = {8: ((20, 48, 96), (8, 32)), 16: ((9, 36, 96), (12, 32)), 32: ((4, 30, 64), (6, 32))}
+RUN = {8: 8, 16: 16, 32: 8}   # outputs along y that share one recursion: a value leaves a rounding error to those after it
+
+
+@pytest.fixture(scope="module")
+def sal():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2201_06174_gb300 as s
+    s.load()
+    return s
+
+
+def _features(sal, V, n, boundary="zero"):
+    eng = sal.Saliency(V.shape, sal.Params(n=n, boundary=boundary))
+    try:
+        E = torch.empty((3,) + V.shape, device="cuda")
+        sal.sal_local_spectra_project(eng.h, torch.from_numpy(V).cuda(), E)
+        return E.cpu().numpy().astype(np.float64)
+    finally:
+        eng.close()
+
+
+def _held(shape, p, n, more=0):
+    """Outputs whose window holds sample p, or which lie up to `more` outputs behind such a one along y."""
+    t, x, y = (np.arange(L) for L in shape)
+    a, b, c = (t - n // 2 <= p[0]) & (p[0] < t + n // 2), (x - n // 2 <= p[1]) & (p[1] < x + n // 2), \
+        (y - n // 2 - more <= p[2]) & (p[2] < y + n // 2)
+    return a[:, None, None] & b[None, :, None] & c[None, None, :]
+
+
+@pytest.mark.parametrize("value", [1e6, -1e30])
+@pytest.mark.parametrize("at", ["corner", "inner", "both"])
+@pytest.mark.parametrize("n", [8, 16])   # (32: every window of a brick holds all of its voxels)
+def test_an_outlier_costs_other_windows_no_precision(sal, n, at, value):
+    """Outliers at a brick's first voxel and at one in its middle: a few dozen FP32 roundings per feature elsewhere."""
+    shape, (xb, yb) = FORWARD[n]
+    r = np.random.RandomState(n)
+    V = r.randn(*shape).astype(np.float32)
+    t0 = shape[0] // 2
+    spots = {"corner": [(t0, xb, yb)], "inner": [(t0, xb + n // 2 - 1, yb + n // 2 - 1)]}
+    spots["both"] = spots["corner"] + spots["inner"]
+    held = np.zeros(shape, bool)
+    for p in spots[at]:
+        V[p] = value
+        held |= _held(shape, p, n, 15)
+    near = np.zeros(shape, bool)   # the bricks that hold the spots, and those that begin behind them
+    near[t0, xb - 4:xb + 14, yb - 4:yb + 36] = True
+    pts = np.argwhere(near & ~held)
+    pts = pts[r.permutation(len(pts))[:{8: 600, 16: 300}[n]]]
+    got = _features(sal, V, n)[:, pts[:, 0], pts[:, 1], pts[:, 2]].T
+    want = oracle.features_at(V, pts, n, boundary="zero")
+    assert np.abs(got - want).max(initial=0) <= 32 * 2.0 ** -24 * np.abs(want).min()
