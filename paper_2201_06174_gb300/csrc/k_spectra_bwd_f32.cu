@@ -29,6 +29,10 @@
 //   4. adjoint of stage 2 (x) -> Gamma_G1[k_t][u_x][y];
 //   5. adjoint of stage 1 (t), real part -> the brick's block [u_t][u_x][y] of gVext, written to
 //      scratch; a separate gather kernel sums the overlapping blocks in a fixed order.
+#include <cooperative_groups.h>
+
+#include <algorithm>
+
 #include "spectra_f32_exact.cuh"
 
 namespace sal {
@@ -37,6 +41,7 @@ namespace {
 using f32::Exact2f;
 using f32::FF;
 using f32::ff_add;
+using f32::ff_gather;
 using f32::ff_mul;
 using f32::ff_mul1;
 using f32::kSmallBin;
@@ -410,15 +415,122 @@ k5_listed_apply_f32(float* __restrict__ blocks, const int* __restrict__ lists, l
     }
 }
 
-// One brick (t0, x0, y_start ..), cta its index among the launch's.  EN: the energy reading of the feature (Gamma = 2 rho
-// F, no kink band).  DENSE: a part of a brick of the sliding form, of geometry dg: outputs past dg.BY are none of its
-// own, every small bin is resolved in place, and the block is added to blk.
+// ---- Bricks of the sliding form with more small bins than it lists -------------------------------------------------
+// Every small bin of such a brick from float-float spectra formed separably, as the FP32 ones are: G1 of four k_t at a time
+// and G2 of all rows in shared memory, then 16 terms a bin instead of the direct sum's 4096 (n = 16).  The x0 of a brick are
+// dealt to the CTAs of a cluster, which add their parts to the brick's block in the order of x0.
+constexpr int kDenseRun = 16;      // outputs of a sliding brick along y
+constexpr int kDenseCluster = 4;
+template <int N> struct DGeo {
+    using G = BGeo<N>;
+    static constexpr int XY = kDenseRun + N - 1;   // odd: rows XY float4 apart meet no bank conflict
+    static constexpr int KG = 4;                   // k_t a group, in the FP32 G1's place
+    static constexpr size_t X2_OFF = (G::SMEM + 15) / 16 * 16;
+    static constexpr size_t EX_OFF = X2_OFF + (size_t)G::ROWS * XY * 16;
+    static constexpr size_t SMEM = EX_OFF + (size_t)4 * N * 4;
+    static constexpr int CTAS = SMEM <= 100 * 1024 ? 2 : 1;   // per SM
+    static_assert((size_t)KG * N * XY * 16 <= G::G_BYTES && G::IN_BYTES % 16 == 0 && SMEM <= 227 * 1024, "geometry");
+};
+
+// The float-float G2 of a staged brick (rect cube), [row][XY] as (re hi, re lo, im hi, im lo).  s_t: KG N XY float4.
+template <int N>
+__device__ void exact_rows(const float* s_in, float4* s_t, float4* s_x2, const float (*s_ex)[N]) {
+    using G = BGeo<N>;
+    using D = DGeo<N>;
+    constexpr int XY = D::XY, NT = G::NT;
+    for (int k0 = 0; k0 < G::H; k0 += D::KG) {
+        const int items = min(D::KG, G::H - k0) * N * XY;
+        for (int it = threadIdx.x; it < items; it += NT) {
+            const int y = it % XY, ux = it / XY % N, kt = k0 + it / (XY * N);
+            FF re = {0.f, 0.f}, im = {0.f, 0.f};
+#pragma unroll
+            for (int ut = 0; ut < N; ++ut) {
+                const float v = s_in[(ut * N + ux) * G::YH + y];
+                const int ph = (kt * ut) % N;
+                ff_gather(re, v, s_ex[0][ph], s_ex[1][ph]);
+                ff_gather(im, v, -s_ex[2][ph], -s_ex[3][ph]);
+            }
+            re = f32::ff_fast_two_sum(re.hi, re.lo);
+            im = f32::ff_fast_two_sum(im.hi, im.lo);
+            s_t[it] = make_float4(re.hi, re.lo, im.hi, im.lo);
+        }
+        __syncthreads();
+        for (int it = threadIdx.x; it < items; it += NT) {
+            const int y = it % XY, kx = it / XY % N, kl = it / (XY * N);
+            FF re = {0.f, 0.f}, im = {0.f, 0.f};
+#pragma unroll 4
+            for (int ux = 0; ux < N; ++ux) {
+                const float4 g = s_t[(kl * N + ux) * XY + y];
+                const int ph = (kx * ux) % N;
+                const FF c = {s_ex[0][ph], s_ex[1][ph]}, sn = {s_ex[2][ph], s_ex[3][ph]}, ns = {-sn.hi, -sn.lo};
+                re = ff_add(re, ff_add(ff_mul(FF{g.x, g.y}, c), ff_mul(FF{g.z, g.w}, sn)));
+                im = ff_add(im, ff_add(ff_mul(FF{g.z, g.w}, c), ff_mul(FF{g.x, g.y}, ns)));
+            }
+            s_x2[((k0 + kl) * N + kx) * XY + y] = make_float4(re.hi, re.lo, im.hi, im.lo);
+        }
+        __syncthreads();
+    }
+}
+
+// F / |F| of bin k_y of the window whose n samples of G2 start at g; 0 where F is 0 in float-float arithmetic.
+template <int N>
+__device__ __noinline__ float2 exact_direction(const float4* g, int ky, float l1, const float (*s_ex)[N]) {
+    FF re = {0.f, 0.f}, im = {0.f, 0.f};
+#pragma unroll 4
+    for (int u = 0; u < N; ++u) {
+        const float4 v = g[u];
+        const int ph = (ky * u) % N;
+        const FF c = {s_ex[0][ph], s_ex[1][ph]}, sn = {s_ex[2][ph], s_ex[3][ph]}, ns = {-sn.hi, -sn.lo};
+        re = ff_add(re, ff_add(ff_mul(FF{v.x, v.y}, c), ff_mul(FF{v.z, v.w}, sn)));
+        im = ff_add(im, ff_add(ff_mul(FF{v.z, v.w}, c), ff_mul(FF{v.x, v.y}, ns)));
+    }
+    const float mx = fmaxf(fabsf(re.hi), fabsf(im.hi));
+    if (!(mx > kZeroBin * l1)) return make_float2(0.f, 0.f);
+    const float fr = re.hi / mx, fi = im.hi / mx;   // scaled first: no underflow
+    const float s = 1.f / sqrtf(fmaf(fr, fr, fi * fi));
+    return make_float2(s * fr, s * fi);
+}
+
+// Adjoint of stage 1 (t), real part, of the brick's Gamma_G1 [H][N][YH]: the block [u_t][u_x][y], slices `slice` and rows
+// `pitch` floats apart, the first `ny` positions of each row; written, or added (ADD).
+template <int N, bool ADD>
+__device__ __forceinline__ void write_block(float* blk, size_t slice, int pitch, int ny, const Tw<N>& tw) {
+    using G = BGeo<N>;
+    constexpr int H = G::H, YH = G::YH;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const float2* s_gg1 = reinterpret_cast<const float2*>(smem_raw);
+    for (int it = threadIdx.x; it < N * YH; it += G::NT) {
+        const int ux = it / YH, y = it % YH;
+        float2 g[H];
+#pragma unroll
+        for (int k = 0; k < H; ++k) g[k] = s_gg1[(size_t)(k * N + ux) * YH + y];
+        float had[N];   // all loads first
+        if (ADD) {
+#pragma unroll
+            for (int u = 0; u < N; ++u) had[u] = y < ny ? blk[u * slice + ux * pitch + y] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < N; ++u) {
+            float z = 0.f;
+#pragma unroll
+            for (int k = 0; k < H; ++k) {
+                z = fmaf(g[k].x, tw.c[k][u], z);
+                if (k != 0 && 2 * k != N) z = fmaf(-g[k].y, tw.s[k][u], z);
+            }
+            if (!ADD) blk[u * slice + ux * pitch + y] = z;
+            else if (y < ny) blk[u * slice + ux * pitch + y] = had[u] + z;
+        }
+    }
+}
+
+// One brick (t0, x0, y_start ..), cta its index among the launch's: Gamma_G1 [H][N][YH] at the start of shared memory (after a
+// barrier).  EN: the energy reading of the feature (Gamma = 2 rho F, no kink band).  DENSE: one x0 of a brick of the sliding
+// form: outputs past kDenseRun are none of its own, and small bins are resolved as above.
 template <int N, bool EN, bool DENSE>
-__device__ __forceinline__ void adjoint_brick(const float* __restrict__ V, const float* __restrict__ gE, float* blk,
-                                              int T, int X, int Y, int bnd, int t0, int x0, int y_start,
-                                              const float* __restrict__ wtab, int taper, const Tw<N>& tw,
-                                              const Exact2f<N>& ex, const VanishTab& vt, int* __restrict__ lists,
-                                              long long cta, long long ncta, const SpectraAdjointGeometry& dg) {
+__device__ __forceinline__ void adjoint_brick(const float* __restrict__ V, const float* __restrict__ gE, int T, int X, int Y,
+                                              int bnd, int t0, int x0, int y_start, const float* __restrict__ wtab,
+                                              int taper, const Tw<N>& tw, const Exact2f<N>& ex, const VanishTab& vt,
+                                              int* __restrict__ lists, long long cta, long long ncta) {
     using G = BGeo<N>;
     using B = typename G::B;
     constexpr int H = G::H, BY = G::BY, YC = G::YC, YH = G::YH, ROWS = G::ROWS, NT = G::NT, WIN = G::WIN;
@@ -436,14 +548,17 @@ __device__ __forceinline__ void adjoint_brick(const float* __restrict__ V, const
 
     const int tid = threadIdx.x;
     const size_t NV = (size_t)T * X * Y;
+    using D = DGeo<N < 8 ? 8 : N>;   // (DENSE: the windows that slide)
+    const float4* s_x2 = reinterpret_cast<const float4*>(smem_raw + D::X2_OFF);       // [ROWS][XY]
+    const float(*s_ex)[N] = reinterpret_cast<const float(*)[N]>(smem_raw + D::EX_OFF);   // [4][N], the kernel's
 
-    if (!EN)
+    if (!EN && !DENSE)
         for (int i = tid; i < 2 * N; i += NT)
             s_src[i] = i < N ? ext_index(t0 - N / 2 + i, T, bnd) : ext_index(x0 - N / 2 + i - N, X, bnd);
     B::stage_brick(V, s_in, T, X, Y, bnd, t0, x0, y_start);
     for (int i = tid; i < 3 * BY; i += NT) {
         const int m = i / BY, yl = i % BY, y = y_start + yl;
-        s_ge[i] = y < Y && (!DENSE || yl < dg.BY) ? __ldg(gE + m * NV + ((size_t)t0 * X + x0) * Y + y) : 0.f;
+        s_ge[i] = y < Y && (!DENSE || yl < kDenseRun) ? __ldg(gE + m * NV + ((size_t)t0 * X + x0) * Y + y) : 0.f;
     }
     __syncthreads();
     // window L1 norms A[y0] = sum_u h(u_t) h(u_x) h(u_y) |V|, as column sums then a y box sum
@@ -462,6 +577,8 @@ __device__ __forceinline__ void adjoint_brick(const float* __restrict__ V, const
     }
     B::stage2(s_g1, s_g2, tw);
     __syncthreads();
+    if constexpr (DENSE)
+        exact_rows<N>(s_in, reinterpret_cast<float4*>(s_g1), reinterpret_cast<float4*>(smem_raw + D::X2_OFF), s_ex);
 
     // ---- step 2: forward stage 3, Gamma, inverse along y into the private window -------------
     const int row = tid % ROWS;
@@ -477,6 +594,7 @@ __device__ __forceinline__ void adjoint_brick(const float* __restrict__ V, const
         !EN && (((vanish_mask(vt, 0, t0, N) >> (row / N)) | (vanish_mask(vt, 1, x0, N) >> (row % N))) & 1u);
     for (int yi = 0; yi < YC; ++yi) {
         const int yl = ych * YC + yi;
+        if (DENSE && yl >= kDenseRun) break;
         {
             float pr[H], pi[H], qr[H], qi[H];
 #pragma unroll
@@ -544,7 +662,25 @@ __device__ __forceinline__ void adjoint_brick(const float* __restrict__ V, const
             // bins that vanish for every input keep Gamma = 0; so does an all-zero cube (A_p = 0)
             if (small != 0u && (row_vanishes || !(s_l1[yl] > 0.f))) small = 0u;
             if (small != 0u) small &= ~vanish_mask(vt, 2, y_start + yl, N);
-            s_small[yi * NT + tid] = (uint16_t)small;
+            if (!DENSE) s_small[yi * NT + tid] = (uint16_t)small;
+        }
+        if constexpr (DENSE) {
+            const float4* xrow = s_x2 + row * D::XY + yl;
+#pragma unroll
+            for (int q = 0; q < N; ++q) {
+                const int k = q <= N / 2 ? q : N - q;
+                if ((small >> q) & 1u) {
+                    const float2 d = exact_direction<N>(xrow, q, s_l1[yl], s_ex);
+                    const float rho = fmaf(g0, wt[0][k], fmaf(g1, wt[1][k], g2 * wt[2][k]));
+                    ar[k] = fmaf(rho, d.x, ar[k]);
+                    ai[k] = fmaf(rho, d.y, ai[k]);
+                    if (k != 0 && 2 * k != N) {
+                        const float sg = q < N / 2 ? rho : -rho;
+                        br[k] = fmaf(-sg, d.y, br[k]);
+                        bi[k] = fmaf(sg, d.x, bi[k]);
+                    }
+                }
+            }
         }
 #pragma unroll
         for (int u = 0; u < N; ++u) {
@@ -565,10 +701,10 @@ __device__ __forceinline__ void adjoint_brick(const float* __restrict__ V, const
             *w = acc;
         }
     }
-    if (!EN) {
+    if constexpr (!EN && !DENSE) {
         // the small bins go to the listed-bin pass when a list is given and they fit in it
         unsigned* s_wbits = reinterpret_cast<unsigned*>(smem_raw + G::WB_OFF);
-        const bool listed = !DENSE && lists && list_small_bins<NT, YC>(s_small, s_wbits,
+        const bool listed = lists && list_small_bins<NT, YC>(s_small, s_wbits,
                                                              lists + list_cta_offset(ncta) + cta * kListStride,
                                                              lists + 4, lists, cta);
         if (!listed)
@@ -627,25 +763,6 @@ __device__ __forceinline__ void adjoint_brick(const float* __restrict__ V, const
         }
     }
     __syncthreads();
-
-    // ---- step 5: adjoint of stage 1 (t), real part -> scratch block [u_t][u_x][y] -------------
-    for (int it = tid; it < N * YH; it += NT) {
-        const int ux = it / YH, y = it % YH;
-        float2 g[H];
-#pragma unroll
-        for (int k = 0; k < H; ++k) g[k] = s_gg1[(size_t)(k * N + ux) * YH + y];
-#pragma unroll
-        for (int u = 0; u < N; ++u) {
-            float z = 0.f;
-#pragma unroll
-            for (int k = 0; k < H; ++k) {
-                z = fmaf(g[k].x, tw.c[k][u], z);
-                if (k != 0 && 2 * k != N) z = fmaf(-g[k].y, tw.s[k][u], z);
-            }
-            if (!DENSE) blk[(size_t)u * G::SLICE + ux * YH + y] = z;
-            else if (y < dg.YH) blk[(size_t)u * dg.slice + ux * dg.YH + y] += z;
-        }
-    }
 }
 
 // A CTA per brick (one x0).  The rect cube at n = 8, 16 takes the sliding form (k_spectra_bwd_f32_slide.cu).
@@ -656,32 +773,54 @@ k5_spectra_adjoint_f32(const float* __restrict__ V, const float* __restrict__ gE
                        int taper, const __grid_constant__ Tw<N> tw, const __grid_constant__ Exact2f<N> ex,
                        const __grid_constant__ VanishTab vt, int* __restrict__ lists) {
     const long long cta = ((long long)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x;
+    using G = BGeo<N>;
     // t_step s > 1: the lattice planes of stride-s windows
-    adjoint_brick<N, EN, false>(V, gE, blocks + cta * BGeo<N>::BLOCK_FLOATS, T, X, Y, bnd,
-                                t_begin + blockIdx.z * t_step, blockIdx.y, blockIdx.x * BGeo<N>::BY, wtab, taper, tw,
-                                ex, vt, lists, cta, (long long)gridDim.x * gridDim.y * gridDim.z,
-                                SpectraAdjointGeometry{});
+    adjoint_brick<N, EN, false>(V, gE, T, X, Y, bnd, t_begin + blockIdx.z * t_step, blockIdx.y, blockIdx.x * G::BY, wtab,
+                                taper, tw, ex, vt, lists, cta, (long long)gridDim.x * gridDim.y * gridDim.z);
+    // ---- step 5: adjoint of stage 1 (t), real part -> scratch block [u_t][u_x][y] -------------
+    write_block<N, false>(blocks + cta * G::BLOCK_FLOATS, G::SLICE, G::YH, G::YH, tw);
 }
 
-// The bricks the sliding form leaves (dense[brick] set: more small bins than it lists): the blocks walk over the marks,
-// a marked brick's x0 one after the other into its block.
+// The bricks the sliding form leaves (dense[brick] set: more small bins than it lists): cluster c looks through the marks of
+// bricks c, c + C, .. 32 at a time.  Constant volumes, n = 16: 48^3 42 ms (a direct sum per bin, a CTA per brick: 3.87 s),
+// 6 x 8 x 10 1.1 ms (409 ms); n = 8: 3.0 ms (70 ms) and 0.19 ms (5.8 ms).  Bound: the latency of float-float chains.
 template <int N>
-__global__ void __launch_bounds__(BGeo<N>::NT, BCfg<N>::MINB)
+__global__ void __cluster_dims__(kDenseCluster, 1, 1) __launch_bounds__(BGeo<N>::NT, DGeo<N>::CTAS)
 k5_dense_f32(const float* __restrict__ V, const float* __restrict__ gE, float* __restrict__ blocks, int T, int X, int Y,
              int bnd, int t_begin, int t_step, int t_count, const float* __restrict__ wtab,
              const __grid_constant__ Tw<N> tw, const __grid_constant__ Exact2f<N> ex,
              const __grid_constant__ VanishTab vt, const SpectraAdjointGeometry dg, const int* __restrict__ dense) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const auto cluster = cooperative_groups::this_cluster();
+    float* s_ex = reinterpret_cast<float*>(smem_raw + DGeo<N>::EX_OFF);
+    for (int i = threadIdx.x; i < 4 * N; i += BGeo<N>::NT) {
+        const int a = i / N, m = i % N;
+        s_ex[i] = a == 0 ? ex.ch[m] : a == 1 ? ex.cl[m] : a == 2 ? ex.sh[m] : ex.sl[m];
+    }
+    const int rank = blockIdx.x % kDenseCluster, lane = threadIdx.x & 31;
+    const long long c = blockIdx.x / kDenseCluster, C = gridDim.x / kDenseCluster;
     const int nseg = (Y + dg.BY - 1) / dg.BY, nxs = (X + dg.BX - 1) / dg.BX;
     const long long total = (long long)nseg * nxs * t_count;
-    for (long long b = blockIdx.x; b < total; b += gridDim.x) {
-        if (!dense[b]) continue;   // block-uniform
-        const int sg = (int)(b % nseg), xs = (int)(b / nseg % nxs), t0 = t_begin + (int)(b / ((long long)nseg * nxs)) * t_step;
-        float* blk = blocks + b * dg.block_floats;
-        for (int i = threadIdx.x; i < dg.block_floats; i += BGeo<N>::NT) blk[i] = 0.f;
-        for (int x0 = xs * dg.BX; x0 < min(X, xs * dg.BX + dg.BX); ++x0) {
-            __syncthreads();   // the block is zeroed; the previous x0 is done with it and with shared memory
-            adjoint_brick<N, false, true>(V, gE, blk + (size_t)(x0 - xs * dg.BX) * dg.YH, T, X, Y, bnd, t0, x0,
-                                          sg * dg.BY, wtab, 0, tw, ex, vt, nullptr, 0, 1, dg);
+    for (long long b0 = c; b0 < total; b0 += 32 * C) {
+        const long long mine = b0 + lane * C;
+        unsigned todo = __ballot_sync(0xffffffffu, mine < total && dense[mine] != 0);   // the same in the whole cluster
+        for (; todo; todo &= todo - 1) {
+            const long long b = b0 + (__ffs(todo) - 1) * C;
+            const int sg = (int)(b % nseg), xs = (int)(b / nseg % nxs);
+            const int t0 = t_begin + (int)(b / ((long long)nseg * nxs)) * t_step;
+            float* blk = blocks + b * dg.block_floats;
+            for (int i = rank * BGeo<N>::NT + threadIdx.x; i < dg.block_floats; i += kDenseCluster * BGeo<N>::NT) blk[i] = 0.f;
+            const int xl = xs * dg.BX, nx = min(X - xl, dg.BX);
+            cluster.sync();   // the block is zeroed
+            for (int x = rank; x - rank < nx; x += kDenseCluster) {
+                if (x < nx)
+                    adjoint_brick<N, false, true>(V, gE, T, X, Y, bnd, t0, xl + x, sg * dg.BY, wtab, 0, tw, ex, vt, nullptr,
+                                                  0, 1);
+                for (int r = 0; r < kDenseCluster; ++r) {
+                    if (r == rank && x < nx) write_block<N, true>(blk + (size_t)x * dg.YH, dg.slice, dg.YH, dg.YH, tw);
+                    cluster.sync();
+                }
+            }
         }
     }
 }
@@ -697,7 +836,7 @@ cudaError_t prepare_n() {
         e = cudaFuncSetAttribute(k5_spectra_adjoint_f32<N, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if constexpr (kHasSliding<N>) {
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k5_dense_f32<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            e = cudaFuncSetAttribute(k5_dense_f32<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DGeo<N>::SMEM);
     }
     return e;
 }
@@ -739,8 +878,10 @@ cudaError_t launch_dense(const TwiddleTable& t, const float* wtab, const float* 
     using G = BGeo<N>;
     const SpectraAdjointGeometry g = spectra_adjoint_f32_slide_geometry(N);
     const long long total = (long long)((Y + g.BY - 1) / g.BY) * ((X + g.BX - 1) / g.BX) * t_count;
-    const int grid = (int)(total < 2 * device_sms() ? total : 2 * device_sms());
-    k5_dense_f32<N><<<grid, G::NT, G::SMEM, s>>>(V, gE, blocks, T, X, Y, bnd, t_begin, t_step, t_count, wtab,
+    if (g.BY != kDenseRun || g.YH != DGeo<N>::XY) return cudaErrorInvalidValue;
+    const long long clusters = std::max(1, DGeo<N>::CTAS * device_sms() / kDenseCluster);
+    const int grid = (int)std::min(total, clusters) * kDenseCluster;
+    k5_dense_f32<N><<<grid, G::NT, DGeo<N>::SMEM, s>>>(V, gE, blocks, T, X, Y, bnd, t_begin, t_step, t_count, wtab,
                                                  f32::make_tw<N>(t), make_exact2f<N>(0),
                                                  make_vanish_tab(N, T, X, Y, bnd, 0), g, dense);
     note_launches(1);

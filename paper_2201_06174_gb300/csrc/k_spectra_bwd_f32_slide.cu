@@ -32,6 +32,7 @@ using f32::Exact2f;
 using f32::fast_rsqrt;
 using f32::FF;
 using f32::ff_add;
+using f32::ff_gather;
 using f32::ff_mul;
 using f32::kSmallBin;
 using f32::kZeroBin;
@@ -61,14 +62,6 @@ template <int N, int GROUPS_ = AGeo<N>::GROUPS> struct Adj {
     static_assert((SMEM + 1024) * CTAS <= 228 * 1024, "geometry");
     static_assert((size_t)XH * YH + XH * kRun <= 2 * G2 && kList <= 2 * G2, "L1 sums and the sorted list fit in G2");
 };
-
-// s += v (ch + cl): the rounded product by an error-free sum, its residuals into the low part.
-__device__ __forceinline__ void ff_gather(FF& s, float v, float ch, float cl) {
-    const float p = v * ch, e = fmaf(v, cl, fmaf(v, ch, -p));
-    const float t = s.hi + p, b = t - s.hi;
-    s.lo += ((s.hi - (t - b)) + (p - b)) + e;
-    s.hi = t;
-}
 
 // A small bin: x0 within the brick (5 bits), output (4), k_t (4), k_x (4), k_y (4).
 __device__ __forceinline__ int small_code(int x0l, int j, int kt, int kx, int ky) {

@@ -111,6 +111,14 @@ __device__ __forceinline__ FF ff_mul1(float a, FF b) {   // a exact in FP32
     return ff_fast_two_sum(p, fmaf(a, b.lo, fmaf(a, b.hi, -p)));
 }
 
+// s += v (ch + cl): the rounded product by an error-free sum, its residuals into the low part.
+__device__ __forceinline__ void ff_gather(FF& s, float v, float ch, float cl) {
+    const float p = v * ch, e = fmaf(v, cl, fmaf(v, ch, -p));
+    const float t = s.hi + p, b = t - s.hi;
+    s.lo += ((s.hi - (t - b)) + (p - b)) + e;
+    s.hi = t;
+}
+
 // The float-float constants of the exact recompute of small bins: cos, sin (2 pi m / n) and the taper
 // (rect, or the periodic Hann window 1/2 - cos(2 pi u / n) / 2), from the host's double-precision libm,
 // each split into an FP32 head and the FP32 rounding of the remainder.
