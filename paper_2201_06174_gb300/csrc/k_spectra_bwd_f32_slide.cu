@@ -1,25 +1,29 @@
 // K5-F32, sliding form (rect cube, n = 8, 16): adjoint of the local-spectrum feature step in FP32, as
 // k_spectra_bwd_f32.cu defines it (Gamma, small bins), over the tiles and register FFTs of the sliding forward
 // (spectra_f32_fft.cuh).  One group of threads takes one brick: one t0, RX positions x0, 16 outputs y0.
-//   stages 1 and 2 as in K1; per tile, a thread per (x0, k_x) then follows its row along y: the first window by an
-//   FFT, the others by the anchored recursion F_{j+1}[k] = F_j[k] + d_j w^(k j).  |F| does not see the phase, and with
-//   Gamma_j the gradient of F_j in the same phase and P_j = sum_{i <= j} Gamma_i the gradient of the row is
-//     dG2[p] = e_p - e_{p-n},   e_j = sum_k P_j[k] w^(-k j)  (j < 15),   e_p = sum_k P_15[k] w^(-k p)  (p >= 15),
+//   stages 1 and 2 as in K1; per tile, a thread per (x0, k_x) then follows its row along y in runs of R outputs (4 for
+//   n = 8, 8 for n = 16): a run's first window by an FFT, the others by the anchored recursion F_{j+1}[k] = F_j[k] +
+//   d_j w^(k j).  |F| does not see the phase, and with Gamma_j the gradient of F_j in the same phase and P_j = sum_{i <= j}
+//   Gamma_i the run's part of the row's gradient is
+//     e_p (p < n),   e_p - e_{p-n} (p >= n),   e_j = sum_k P_j[k] w^(-k j)  (j < R-1),   e_p = sum_k P_{R-1}[k] w^(-k p) after,
 //   one evaluation at a point per output (two additions a bin, the adjoint of the recursion) and one inverse FFT per
-//   run; dG2 replaces G2 in the thread's own row;
+//   run; the n - 1 positions a run shares with the next stay in registers, and the gradient replaces G2 in the thread's
+//   own row.  The sums P run over R outputs and no more: what is left of a strong output where its windows have ended (the
+//   differences e_p - e_{p-n}), and a NaN, reach R - 1 outputs on (runs of all 16: up to 15, and 2 to 4 times the error
+//   beside an output of 1e5 times the others' gradient; at n = 16 that took 6.2 instead of 6.9 ms on 128^3);
 //   adjoint of stage 2: an inverse FFT per (x0, y), then per halo position the sum of the x0 whose cubes hold it,
 //   which replaces the tile's G1; after all tiles the adjoint of stage 1 writes the brick's block.
 // Small bins (|F| <= 2^-16 of the window's L1 norm) take Gamma = 0 in the tile loop and go to the brick's list; at the
 // end, in the order of their codes, its warps recompute them as direct float-float sums, and their rank-one gradients
 // are added to the gradient of G1 (256 terms each; at the block they would be 4096).  A brick with more than kList
 // such bins (constant regions: every bin) is marked and left to k5_dense_f32.
-// The instruction cache sets how far the loop over outputs is unrolled: by 8 (w^(k (j + 8)) = +-w^(k j) for n = 16), and
-// not at all in tile 0, whose packed rows need the most code for an eighth of the work (there every window is an FFT).
-// Bound: issue slots, about 450 per thread and output of 16 bins with the FFTs and the small bins (128 MUFU cycles), 54 %
-// of them used by 12 warps an SM at 168 registers.  The adjoint call, 128^3: n = 16 25.0 -> 6.1 ms, n = 8 2.54 -> 0.98
+// The instruction cache sets how far the loop over outputs is unrolled: by R, and not at all in tile 0, whose packed rows
+// need the most code for an eighth of the work (there every window is an FFT).
+// Bound: issue slots, about 500 per thread and output of 16 bins with the FFTs and the small bins (128 MUFU cycles), by 12
+// warps an SM at 168 registers.  The adjoint call, 128^3: n = 16 25.0 -> 6.9 ms, n = 8 2.54 -> 0.87
 // (before: one x0 per brick, direct DFTs in stages 1 and 2 and both of their adjoints, 31 point evaluations of 32
 // multiply-adds per run of 8 outputs, and two passes over the grid for the small bins, 0.1 per voxel here); 24^3, n = 16:
-// 353 -> 180 us.  Error against FP64 9.9e-7 -> 9.8e-7 (n = 16), 8.0e-7 -> 8.8e-7 (n = 8), most of it in the directions
+// 353 -> 186 us.  Error against FP64 9.7e-7 -> 9.8e-7 (n = 16), 8.0e-7 -> 8.3e-7 (n = 8), most of it in the directions
 // of the weak bins just above the small-bin level.
 #include "spectra_f32_exact.cuh"
 #include "spectra_f32_fft.cuh"
@@ -47,8 +51,8 @@ constexpr int kChunk = 64;   // small bins whose Gamma is held at a time
 // two in a CTA of 384 (whole multiples of four warps, the granule of register allocation), one CTA an SM; the groups
 // meet at barriers of their own.  With no more bricks than SMs a CTA takes one (12 x 16 x 20: 248 -> 205 us a call).
 template <int N> struct AGeo;
-template <> struct AGeo<8> { static constexpr int RX = 16, GROUPS = 1, CTAS = 4; };
-template <> struct AGeo<16> { static constexpr int RX = 12, GROUPS = 2, CTAS = 1; };
+template <> struct AGeo<8> { static constexpr int RX = 16, R = 4, GROUPS = 1, CTAS = 4; };
+template <> struct AGeo<16> { static constexpr int RX = 12, R = 8, GROUPS = 2, CTAS = 1; };
 template <int N, int GROUPS_ = AGeo<N>::GROUPS> struct Adj {
     static constexpr int GROUPS = GROUPS_, CTAS = AGeo<N>::CTAS;
     static constexpr int RX = AGeo<N>::RX, GT = RX * N, NT = GT * GROUPS, TILES = N / 2, H = N / 2 + 1;
@@ -94,7 +98,7 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
          const __grid_constant__ VanishTab vt, int* __restrict__ dense) {
     using G = Adj<N, GROUPS>;
     using B = Bins<N, false>;
-    constexpr int RX = G::RX, XH = G::XH, YH = G::YH, GT = G::GT, H = G::H, TILES = G::TILES, NW = B::NW;
+    constexpr int RX = G::RX, R = AGeo<N>::R, XH = G::XH, YH = G::YH, GT = G::GT, H = G::H, TILES = G::TILES, NW = B::NW;
     constexpr size_t TILE_W = (size_t)3 * H * N;   // weights of a tile, [map][k][row] (f32_slide_table_fill)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float s_ex[4][N];   // cos, sin (2 pi m / n) as float-float pairs, indexed by the lanes' own phases
@@ -216,9 +220,9 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
 #pragma unroll
                 for (int w = 0; w < NW; ++w) wt[m][w] = __ldg(wtab + tile * TILE_W + (m * H + w) * N + kx);
             B f, P;
-            f.template first<N>(row);
+            float2 c[N - 1];   // what the runs so far give to positions h .. h + n - 2
 #pragma unroll
-            for (int q = 0; q < N / 2; ++q) P.r[q] = P.i[q] = make_float2(0.f, 0.f);
+            for (int i = 0; i < N - 1; ++i) c[i] = make_float2(0.f, 0.f);
             // rho per |k_y| of output j: sum_m gE_m w_m
             auto weights = [&](int j, float (&rho)[NW]) {
                 const float g0 = ge[j], g1 = ge[RX * kRun + j], g2 = ge[2 * RX * kRun + j];
@@ -243,20 +247,22 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
                     (ge[j] != 0.f || ge[RX * kRun + j] != 0.f || ge[2 * RX * kRun + j] != 0.f))
                     note_small<N>(s_van[0], s_van[1 + x0l], my, tile, tid, j, small_a, small_b, s_small, s_count);
             };
-            if (tile != 0) {
+            // tile 0: packed rows hold two signals (k_t = 0 and n/2) in each pair.  Every window anew, in its own phase
+            // (the sums P turn with it)
+            const float* wb = wtab + TILES * TILE_W + kx;
+            const bool packed = kx == 0 || kx == N / 2;
+            const float pk = packed ? 1.f : 0.f, qk = 1.f - 2.f * pk;
 #pragma unroll 1
-                for (int h = 0; h < kRun; h += 8) {
-                    const float odd = N == 16 && h == 8 ? -1.f : 1.f;
-                    if (h > 0) {   // anew from its window: the recursion's rounding runs over 7 steps at most
-                        f.template first<N>(row + h);
-                        f.flip_odd(odd);   // anchored at the start of the run
-                    }
+            for (int h = 0; h < kRun; h += R) {
+                f.template first<N>(row + h);   // phases are those of the run's first window
 #pragma unroll
-                    for (int b = 0; b < 8; ++b) {
+                for (int q = 0; q < N / 2; ++q) P.r[q] = P.i[q] = make_float2(0.f, 0.f);
+                if (tile != 0) {
+#pragma unroll
+                    for (int b = 0; b < R; ++b) {
                         const int j = h + b;
-                        const bool last = b == 7 && h + 8 == kRun;
                         float2 d = make_float2(0.f, 0.f);
-                        if (b < 7) {   // before row[j] becomes the gradient's
+                        if (b + 1 < R) {   // before row[j] becomes the gradient's
                             const float2 u = row[j], v = row[j + N];
                             d = make_float2(v.x - u.x, v.y - u.y);
                         }
@@ -294,90 +300,103 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
                             P.r[q] = __ffma2_rn(sc[q], f.r[q], P.r[q]);
                             P.i[q] = __ffma2_rn(sc[q], f.i[q], P.i[q]);
                         }
-                        if (!last) row[j] = P.at(b, odd);
-                        if (b < 7) f.slide(d, b, odd);
-                    }
-                }
-            } else {
-                // tile 0: packed rows hold two signals (k_t = 0 and n/2) in each pair.  Every window anew, in its own phase
-                // (the sums P turn with it)
-                const float* wb = wtab + TILES * TILE_W + kx;
-                const bool packed = kx == 0 || kx == N / 2;
-                const float pk = packed ? 1.f : 0.f, qk = 1.f - 2.f * pk;
-#pragma unroll 1
-                for (int j = 0; j < kRun; ++j) {
-                    if (j > 0) f.template first<N>(row + j);
-                    float rho[NW];
-                    weights(j, rho);
-                    const float g0 = ge[j], g1 = ge[RX * kRun + j], g2 = ge[2 * RX * kRun + j];
-                    const float thr2 = level(j), thr2p = packed ? 4.f * thr2 : thr2;   // a packed pair holds 2 F
-                    unsigned small_a = 0u, small_b = 0u;
-                    auto scale = [&](float m2, float r, float lim, unsigned& small, int bit) -> float {
-                        if (EN) return 2.f * r;
-                        if (m2 > lim) return r * fast_rsqrt(m2);
-                        small |= 1u << bit;
-                        return 0.f;
-                    };
-                    auto rho_b = [&](int w) -> float {   // the second value of the pair
-                        return fmaf(g0, __ldg(wb + w * N),
-                                    fmaf(g1, __ldg(wb + (H + w) * N), g2 * __ldg(wb + (2 * H + w) * N)));
-                    };
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {   // the self-paired bins 0 and n/2
-                        const float re = h ? f.r[0].y : f.r[0].x, im = h ? f.i[0].y : f.i[0].x;
-                        const int k = h ? N / 2 : 0;
-                        const float sa = scale(fmaf(re, re, (1.f - pk) * im * im), rho[k], thr2, small_a, k);
-                        const float ga = sa * re;
-                        float gb = sa * im;
-                        if (packed) gb = scale(im * im, rho_b(k), thr2, small_b, k) * im;
-                        if (h) {
-                            P.r[0].y += ga;
-                            P.i[0].y += gb;
-                        } else {
-                            P.r[0].x += ga;
-                            P.i[0].x += gb;
+                        if (b + 1 < R) {
+                            const float2 e = P.at(b);
+                            row[j] = make_float2(e.x + c[b].x, e.y + c[b].y);
+                            c[b] = e;
+                            f.slide(d, b);
                         }
                     }
+                } else {
+#pragma unroll 1
+                    for (int b = 0; b < R; ++b) {
+                        const int j = h + b;
+                        if (b > 0) f.template first<N>(row + j);
+                        float rho[NW];
+                        weights(j, rho);
+                        const float g0 = ge[j], g1 = ge[RX * kRun + j], g2 = ge[2 * RX * kRun + j];
+                        const float thr2 = level(j), thr2p = packed ? 4.f * thr2 : thr2;   // a packed pair holds 2 F
+                        unsigned small_a = 0u, small_b = 0u;
+                        auto scale = [&](float m2, float r, float lim, unsigned& small, int bit) -> float {
+                            if (EN) return 2.f * r;
+                            if (m2 > lim) return r * fast_rsqrt(m2);
+                            small |= 1u << bit;
+                            return 0.f;
+                        };
+                        auto rho_b = [&](int w) -> float {   // the second value of the pair
+                            return fmaf(g0, __ldg(wb + w * N),
+                                        fmaf(g1, __ldg(wb + (H + w) * N), g2 * __ldg(wb + (2 * H + w) * N)));
+                        };
 #pragma unroll
-                    for (int q = 1; q < N / 2; ++q) {
-                        const float2 Rr = f.r[q], Ii = f.i[q];
-                        const float r1 = fmaf(pk, Rr.y, Rr.x), i1 = fmaf(-pk, Ii.y, Ii.x);
-                        const float r2 = fmaf(pk, Rr.x, qk * Rr.y), i2 = fmaf(pk, Ii.x, Ii.y);
-                        const float sa = scale(fmaf(r1, r1, i1 * i1), rho[q], thr2p, small_a, q);
-                        const float sb = scale(fmaf(r2, r2, i2 * i2), rho_b(q), thr2p, small_b, q);
-                        const float ur = sa * r1, ui = sa * i1, vr = sb * r2, vi = sb * i2;
-                        P.r[q].x += fmaf(pk, vr, ur);
-                        P.i[q].x += fmaf(pk, vi, ui);
-                        P.r[q].y += fmaf(pk, ur, qk * vr);
-                        P.i[q].y += fmaf(-pk, ui, vi);
+                        for (int k = 0; k <= N / 2; k += N / 2) {   // the self-paired bins 0 and n/2
+                            const float re = k ? f.r[0].y : f.r[0].x, im = k ? f.i[0].y : f.i[0].x;
+                            const float sa = scale(fmaf(re, re, (1.f - pk) * im * im), rho[k], thr2, small_a, k);
+                            const float ga = sa * re;
+                            float gb = sa * im;
+                            if (packed) gb = scale(im * im, rho_b(k), thr2, small_b, k) * im;
+                            if (k) {
+                                P.r[0].y += ga;
+                                P.i[0].y += gb;
+                            } else {
+                                P.r[0].x += ga;
+                                P.i[0].x += gb;
+                            }
+                        }
+#pragma unroll
+                        for (int q = 1; q < N / 2; ++q) {
+                            const float2 Rr = f.r[q], Ii = f.i[q];
+                            const float r1 = fmaf(pk, Rr.y, Rr.x), i1 = fmaf(-pk, Ii.y, Ii.x);
+                            const float r2 = fmaf(pk, Rr.x, qk * Rr.y), i2 = fmaf(pk, Ii.x, Ii.y);
+                            const float sa = scale(fmaf(r1, r1, i1 * i1), rho[q], thr2p, small_a, q);
+                            const float sb = scale(fmaf(r2, r2, i2 * i2), rho_b(q), thr2p, small_b, q);
+                            const float ur = sa * r1, ui = sa * i1, vr = sb * r2, vi = sb * i2;
+                            P.r[q].x += fmaf(pk, vr, ur);
+                            P.i[q].x += fmaf(pk, vi, ui);
+                            P.r[q].y += fmaf(pk, ur, qk * vr);
+                            P.i[q].y += fmaf(-pk, ui, vi);
+                        }
+                        if (!EN && (small_a | small_b)) note(j, small_a, small_b);
+                        if (b + 1 < R) {
+                            const float2 e = P.sum();
+                            row[j] = make_float2(e.x + c[0].x, e.y + c[0].y);
+#pragma unroll
+                            for (int i = 0; i + 1 < N - 1; ++i) c[i] = c[i + 1];   // (a loop that is not unrolled: by turns)
+                            c[N - 2] = e;
+                            P.turn();
+                        }
                     }
-                    if (!EN && (small_a | small_b)) note(j, small_a, small_b);
-                    if (j + 1 < kRun) {
-                        row[j] = P.sum();
-                        P.turn();
-                    }
+                    float2 o[N - 1];
+#pragma unroll
+                    for (int i = 0; i < N - 1; ++i) o[(i + R - 1) % (N - 1)] = c[i];
+#pragma unroll
+                    for (int i = 0; i < N - 1; ++i) c[i] = o[i];
                 }
-            }
-            float2 z[N];   // sum_k P_15[k] w^(-k p); tile 0: P is in the phase of the last window, w^(-15 k) ahead
+                // c: e_0 .. e_{R-2} of this run, then what is left of the runs before.  z: sum_k P_{R-1}[k] w^(-k i) at position
+                // h + i, of period n; in tile 0 P is in the phase of the last window, w^(-(R-1) k) ahead
+                float2 z[N];
 #pragma unroll
-            for (int q = 0; q < N; ++q) z[q] = P.get(q);
-            f32::ifft<N>(z);
-#pragma unroll
-            for (int u = 0; u < N; ++u) {
-                const int p = YH - 1 - u;   // the n positions from 15 on, the last first
-                float2 e = tile == 0 ? z[f32::fft_pos<N>((p + N - (kRun - 1) % N) % N)] : z[f32::fft_pos<N>(p % N)];
-                if (p >= N) {
-                    const float2 v = row[p - N];
-                    e.x -= v.x;
-                    e.y -= v.y;
+                for (int q = 0; q < N; ++q) z[q] = P.get(q);
+                f32::ifft<N>(z);
+                auto at = [&](int i) -> float2 {
+                    return tile == 0 ? z[f32::fft_pos<N>((i + N - (R - 1)) % N)] : z[f32::fft_pos<N>(i % N)];
+                };
+                {
+                    const float2 e = at(R - 1);
+                    row[h + R - 1] = make_float2(e.x + c[R - 1].x, e.y + c[R - 1].y);
                 }
-                row[p] = e;
+                float2 o[N - 1];
+#pragma unroll
+                for (int i = R; i < R + N - 1; ++i) {
+                    const float2 e = at(i % N);
+                    o[i - R] = i < N - 1    ? make_float2(e.x + c[i].x, e.y + c[i].y)
+                               : i == N - 1 ? e
+                                            : make_float2(e.x - c[i % N].x, e.y - c[i % N].y);
+                }
+#pragma unroll
+                for (int i = 0; i < N - 1; ++i) c[i] = o[i];
             }
 #pragma unroll
-            for (int p = kRun - 2; p >= N; --p) {
-                const float2 u = row[p - N], e = row[p];
-                row[p] = make_float2(e.x - u.x, e.y - u.y);
-            }
+            for (int i = 0; i < N - 1; ++i) row[kRun + i] = c[i];
         }
         group_sync();
         // adjoint of stage 2: inverse FFT over k_x of each (x0, y), in place as [x0][u][y]

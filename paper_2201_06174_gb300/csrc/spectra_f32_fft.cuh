@@ -189,48 +189,40 @@ template <int M, bool ODD> struct Bins {
     }
     // bin q += the entering minus the leaving sample times w^(k j), anchored at the start of the run:
     // F_{j+1}[k] = F_j[k] + d w^(k j) (d already times w32^j for the odd bins), w^(q j) = (-i)^s w^(m mod 8).
-    // odd: the sign of the odd q (M = 16: w^(q (j + 8)) = (-1)^q w^(q j), so a loop over j mod 8 passes -1 for j >= 8)
-    __device__ __forceinline__ void slide(float2 d, int j, float odd = 1.f) {
-        float2 p[2][8];
+    __device__ __forceinline__ void slide(float2 d, int j) {
+        float2 p[8];
 #pragma unroll
-        for (int m = 0; m < 8; m += 32 / M) {
-            p[0][m] = rot32(d, m);
-            p[1][m] = make_float2(odd * p[0][m].x, odd * p[0][m].y);
-        }
+        for (int m = 0; m < 8; m += 32 / M) p[m] = rot32(d, m);
 #pragma unroll
         for (int q = 0; q < M; ++q) {
             const int m = (q * j * (32 / M)) & 31, s = m / 8;
-            const float2 a = p[q & 1][m % 8];
+            const float2 a = p[m % 8];
             const float dr = s == 0 ? a.x : s == 1 ? a.y : s == 2 ? -a.x : -a.y;
             const float di = s == 0 ? a.y : s == 1 ? -a.x : s == 2 ? -a.y : a.x;
             if (second(q)) { r[slot(q)].y += dr; i[slot(q)].y += di; }
             else { r[slot(q)].x += dr; i[slot(q)].x += di; }
         }
     }
-    // adjoint of slide: sum_q F[q] e^(+2 pi i k j / n), odd as there
-    __device__ __forceinline__ float2 at(int j, float odd = 1.f) const {
-        float2 p[2][8];
+    // adjoint of slide: sum_q F[q] e^(+2 pi i k j / n)
+    __device__ __forceinline__ float2 at(int j) const {
+        float2 p[8];
 #pragma unroll
-        for (int m = 0; m < 8; ++m) p[0][m] = p[1][m] = make_float2(0.f, 0.f);
+        for (int m = 0; m < 8; ++m) p[m] = make_float2(0.f, 0.f);
 #pragma unroll
         for (int q = 0; q < M; ++q) {
             const int m = (q * j * (32 / M)) & 31, t = m / 8;
             const float2 f = get(q);
-            p[q & 1][m % 8].x += t == 0 ? f.x : t == 1 ? -f.y : t == 2 ? -f.x : f.y;
-            p[q & 1][m % 8].y += t == 0 ? f.y : t == 1 ? f.x : t == 2 ? -f.y : -f.x;
+            p[m % 8].x += t == 0 ? f.x : t == 1 ? -f.y : t == 2 ? -f.x : f.y;
+            p[m % 8].y += t == 0 ? f.y : t == 1 ? f.x : t == 2 ? -f.y : -f.x;
         }
         float2 e = make_float2(0.f, 0.f);
 #pragma unroll
         for (int m = 0; m < 8; m += 32 / M) {
-            const float2 a = rot32(make_float2(fmaf(odd, p[1][m].x, p[0][m].x), fmaf(odd, p[1][m].y, p[0][m].y)), -m);
+            const float2 a = rot32(p[m], -m);
             e.x += a.x;
             e.y += a.y;
         }
         return e;
-    }
-    __device__ __forceinline__ void flip_odd(float odd) {
-#pragma unroll
-        for (int q = 1; q < M; q += 2) set(q, make_float2(odd * get(q).x, odd * get(q).y));
     }
     // for loops that are not unrolled, sums kept in the phase of the current window: F <- F e^(2 pi i k / n) when the
     // window moves by one, and the sum of all bins

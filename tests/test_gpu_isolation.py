@@ -62,3 +62,56 @@ def test_an_outlier_costs_other_windows_no_precision(sal, n, at, value):
     got = _features(sal, V, n)[:, pts[:, 0], pts[:, 1], pts[:, 2]].T
     want = oracle.features_at(V, pts, n, boundary="zero")
     assert np.abs(got - want).max(initial=0) <= 32 * 2.0 ** -24 * np.abs(want).min()
+
+
+ADJOINT_RUN = {8: 4, 16: 8}   # outputs along y whose gradients are formed from one run of sums
+
+
+def _adjoint(sal, V, gE, n):
+    eng = sal.Saliency(V.shape, sal.Params(n=n, boundary="zero"))
+    try:
+        gV = torch.empty(V.shape, device="cuda")
+        sal.sal_local_spectra_project_backward(eng.h, torch.from_numpy(V).cuda(), torch.from_numpy(gE).cuda(), gV)
+        return gV.cpu().numpy().astype(np.float64)
+    finally:
+        eng.close()
+
+
+def _reached(shape, p, n, more=0):
+    """Samples in the window of output p, or of one of the `more` outputs behind it along y."""
+    a, b, c = ((np.arange(L) >= q - n // 2) & (np.arange(L) < q + n // 2 + m) for L, q, m in zip(shape, p, (0, 0, more)))
+    return a[:, None, None] & b[None, :, None] & c[None, None, :]
+
+
+@pytest.mark.parametrize("value", [1e5, 1e30])
+@pytest.mark.parametrize("n,shape,p", [(8, (9, 30, 60), (4, 14, 16)), (8, (9, 30, 60), (4, 14, 21)),
+                                       (16, (17, 40, 70), (8, 18, 16)), (16, (17, 40, 70), (8, 18, 34))])
+def test_a_strong_gradient_costs_other_samples_no_precision(sal, n, shape, p, value):
+    """One output's gradient far above the others': samples outside its window and those of the rest of its run keep the
+    adjoint's bar of 1e-5 relative to what they are."""
+    r = np.random.RandomState(n)
+    V, gE = r.randn(*shape).astype(np.float32), r.randn(3, *shape).astype(np.float32)
+    clean = _adjoint(sal, V, gE, n)
+    gE[(slice(None),) + p] = value
+    got, want = _adjoint(sal, V, gE, n), oracle.features_adjoint(V, gE, n, boundary="zero")
+    far = ~_reached(shape, p, n, ADJOINT_RUN[n] - 1)
+    rms = np.sqrt(np.mean(want[far] ** 2))
+    assert np.abs(got - want)[far].max() <= 1e-5 * rms
+    assert np.abs(got - clean)[far].max() <= 1e-5 * rms
+
+
+@pytest.mark.parametrize("n,shape,p", [(8, (9, 30, 60), (4, 14, 16)), (16, (17, 40, 70), (8, 18, 16))])
+def test_the_adjoint_keeps_a_nan_to_its_runs(sal, n, shape, p):
+    """In a gradient: the samples of its run's windows.  In the volume: those of the runs of every output that holds it."""
+    r = np.random.RandomState(n)
+    V, gE = r.randn(*shape).astype(np.float32), r.randn(3, *shape).astype(np.float32)
+    more = ADJOINT_RUN[n] - 1
+    gE[(1,) + p] = np.nan
+    bad = np.isnan(_adjoint(sal, V, gE, n))
+    assert bad[_reached(shape, p, n)].all() and not bad[~_reached(shape, p, n, more)].any()
+    gE[(1,) + p] = 1.0
+    V[p] = np.nan
+    bad = np.isnan(_adjoint(sal, V, gE, n))
+    t, x, y = np.nonzero(bad)
+    assert abs(t - p[0]).max() <= n and abs(x - p[1]).max() < n
+    assert y.min() >= p[2] - n + 1 and y.max() <= p[2] + n - 1 + more
