@@ -7,7 +7,7 @@
 //            at load), a real FFT, every tile's G1[x][y] kept in shared memory (n = 32: four tiles at a time);
 //   stage 2 (x): a thread per (x0, y): an n-point FFT of G1 -> G2[x0][k_x][y] of the tile;
 //   stage 3 (y): a thread per (x0, k_x) and run of 16 outputs (n = 32: two threads, the even and the odd k_y):
-//            the first window by an FFT, each later one by the sliding DFT anchored at the run's start,
+//            the first window by an FFT (n = 8, 32: and the ninth), each later one by the sliding DFT anchored there,
 //              F_{j+1}[k] = F_j[k] + (G2[j + n] - G2[j]) w^(k j),   w = e^(-2 pi i / n),
 //            whose phase differs from that of the window itself by w^(k j): |F| is the same.  The products d w^m
 //            need one complex multiply per distinct octant angle, the rest are sign changes and swaps, so a
@@ -16,7 +16,7 @@
 // Bound: the MUFU pipe, n^3/2 + n^2/2 roots per voxel at 16 per clock and SM (n = 16: 0.90 ms at 128^3), with about
 // 110 issue slots per thread and output for its 16 bins beside 128 MUFU cycles.  The 48 sums, 16 bins and 27 weights
 // take 168 registers a thread: 12 warps per SM, whose 16 independent bins each hide the latencies.
-// 128^3: n = 16 7.23 -> 2.07 ms, n = 8 1.07 -> 0.28 ms; 48 x 64 x 64, n = 32: 21.2 -> 2.7 ms (before: direct DFTs in
+// 128^3: n = 16 7.23 -> 2.07 ms, n = 8 1.07 -> 0.28 ms; 48 x 64 x 64, n = 32: 21.2 -> 2.3 ms (before: direct DFTs in
 // stages 1 and 2 and for each run's first output, a halo for every row of 32 outputs, a six-operation rotation
 // per bin and output).  Error against FP64, relative L2 of E: 7e-8, 6e-8 and 8e-8 (before 1.3e-7, 7e-8 and 1.3e-7).
 // The brick is staged minus one of its voxels (brick_shift): only the DC bin of a rect cube moves, which Eq. 1 leaves out, so a
@@ -38,13 +38,18 @@ template <int N> struct WGeo {
     static constexpr size_t FLOATS = (TILES + 1) * TILE;
 };
 
-// One tile of one thread: RUN outputs along the row g, |F| weighted into acc[output][map].
+// One tile of one thread: RUN outputs along the row g, |F| weighted into acc[output][map].  The recursion starts anew from an
+// FFT every 16 outputs for n = 16 and every 8 for the others, no further than an extreme sample's rounding, or a NaN, may
+// reach behind its windows (16 at n = 8 and 32 made features up to 15 outputs away lose what 8 keep).  The two halves of a run
+// as one loop that is not unrolled, which also keeps n = 32 in the instruction cache: 48 x 64 x 64 2.75 -> 2.29 ms; n = 8,
+// 128^3: 273 -> 277 us.
 template <int N, int M, bool ODD, bool EN, int RUN>
 __device__ __forceinline__ void slide_tile(const float2* __restrict__ g, const float* __restrict__ wtab, int tile,
                                            int row, float (&acc)[RUN][3]) {
     using W = WGeo<N>;
     using B = Bins<M, ODD>;
-    constexpr int NW = B::NW;
+    constexpr int NW = B::NW, PART = RUN < 8 || N == 16 ? RUN : 8;
+    static_assert(PART == RUN || 2 * PART == RUN, "two halves");
     float wt[3][NW];
 #pragma unroll
     for (int m = 0; m < 3; ++m)
@@ -52,70 +57,82 @@ __device__ __forceinline__ void slide_tile(const float2* __restrict__ g, const f
         for (int w = 0; w < NW; ++w)
             wt[m][w] = __ldg(wtab + tile * W::TILE + (m * W::H + B::ky(w, N)) * N + row);
     B f;
-    f.template first<N>(g);
     const float* wb = wtab + W::TILES * W::TILE + row;
     const float pk = (row == 0 || row == N / 2) ? 1.f : 0.f;   // tile 0: a packed row
+#pragma unroll 1
+    for (int h = 0; h < RUN; h += PART, g += PART) {
+        f.template first<N>(g);
 #pragma unroll
-    for (int j = 0; j < RUN; ++j) {
-        if (j > 0) {
-            const float2 a = g[j - 1], b = g[j - 1 + N];   // sample leaving, sample entering
-            float2 d = make_float2(b.x - a.x, b.y - a.y);
-            if (ODD) d = f32::rot32(d, j - 1);
-            f.slide(d, j - 1);
-        }
-        float s[NW];
-        if (tile != 0) {
-#pragma unroll
-            for (int q = 0; q < M / 2; ++q) {
-                const float2 m2 = __ffma2_rn(f.i[q], f.i[q], __fmul2_rn(f.r[q], f.r[q]));
-                const float a = bin_mag<EN>(m2.x), b = bin_mag<EN>(m2.y);
-                if (!ODD && q == 0) {
-                    s[0] = a;
-                    s[M / 2] = b;
-                } else {
-                    s[q] = a + b;
-                }
+        for (int j = 0; j < PART; ++j) {
+            if (j > 0) {
+                const float2 a = g[j - 1], b = g[j - 1 + N];   // sample leaving, sample entering
+                float2 d = make_float2(b.x - a.x, b.y - a.y);
+                if (ODD) d = f32::rot32(d, j - 1);
+                f.slide(d, j - 1);
             }
-        } else {
-            // tile 0: packed rows give F_0 + conj.. (x2) and F_{n/2} (x2) from the pair, the others their two bins
+            float s[NW];
+            if (tile != 0) {
 #pragma unroll
-            for (int q = 0; q < M / 2; ++q) {
-                const float2 R = f.r[q], I = f.i[q];
-                float a, b, c = 0.f, e = 0.f;   // first signal (a, c), second signal (b, e)
-                if (!ODD && q == 0) {
-                    a = bin_mag<EN>(fmaf(R.x, R.x, (1.f - pk) * I.x * I.x));   // bin 0
-                    b = bin_mag<EN>(pk * I.x * I.x);
-                    c = bin_mag<EN>(fmaf(R.y, R.y, (1.f - pk) * I.y * I.y));   // bin n/2
-                    e = bin_mag<EN>(pk * I.y * I.y);
-                    s[0] = a;
-                    s[M / 2] = c;
-#pragma unroll
-                    for (int m = 0; m < 3; ++m) {
-                        acc[j][m] = fmaf(__ldg(wb + m * W::H * N), b, acc[j][m]);
-                        acc[j][m] = fmaf(__ldg(wb + (m * W::H + N / 2) * N), e, acc[j][m]);
+                for (int q = 0; q < M / 2; ++q) {
+                    const float2 m2 = __ffma2_rn(f.i[q], f.i[q], __fmul2_rn(f.r[q], f.r[q]));
+                    const float a = bin_mag<EN>(m2.x), b = bin_mag<EN>(m2.y);
+                    if (!ODD && q == 0) {
+                        s[0] = a;
+                        s[M / 2] = b;
+                    } else {
+                        s[q] = a + b;
                     }
-                } else {
-                    const float r1 = fmaf(pk, R.y, R.x), i1 = fmaf(-pk, I.y, I.x);
-                    const float r2 = fmaf(pk, R.x, (1.f - 2.f * pk) * R.y), i2 = fmaf(pk, I.x, I.y);
-                    a = bin_mag<EN>(fmaf(r1, r1, i1 * i1));
-                    b = bin_mag<EN>(fmaf(r2, r2, i2 * i2));
-                    s[q] = a;
+                }
+            } else {
+                // tile 0: packed rows give F_0 + conj.. (x2) and F_{n/2} (x2) from the pair, the others their two bins
 #pragma unroll
-                    for (int m = 0; m < 3; ++m)
-                        acc[j][m] = fmaf(__ldg(wb + (m * W::H + B::ky(q, N)) * N), b, acc[j][m]);
+                for (int q = 0; q < M / 2; ++q) {
+                    const float2 R = f.r[q], I = f.i[q];
+                    float a, b, c = 0.f, e = 0.f;   // first signal (a, c), second signal (b, e)
+                    if (!ODD && q == 0) {
+                        a = bin_mag<EN>(fmaf(R.x, R.x, (1.f - pk) * I.x * I.x));   // bin 0
+                        b = bin_mag<EN>(pk * I.x * I.x);
+                        c = bin_mag<EN>(fmaf(R.y, R.y, (1.f - pk) * I.y * I.y));   // bin n/2
+                        e = bin_mag<EN>(pk * I.y * I.y);
+                        s[0] = a;
+                        s[M / 2] = c;
+#pragma unroll
+                        for (int m = 0; m < 3; ++m) {
+                            acc[j][m] = fmaf(__ldg(wb + m * W::H * N), b, acc[j][m]);
+                            acc[j][m] = fmaf(__ldg(wb + (m * W::H + N / 2) * N), e, acc[j][m]);
+                        }
+                    } else {
+                        const float r1 = fmaf(pk, R.y, R.x), i1 = fmaf(-pk, I.y, I.x);
+                        const float r2 = fmaf(pk, R.x, (1.f - 2.f * pk) * R.y), i2 = fmaf(pk, I.x, I.y);
+                        a = bin_mag<EN>(fmaf(r1, r1, i1 * i1));
+                        b = bin_mag<EN>(fmaf(r2, r2, i2 * i2));
+                        s[q] = a;
+#pragma unroll
+                        for (int m = 0; m < 3; ++m)
+                            acc[j][m] = fmaf(__ldg(wb + (m * W::H + B::ky(q, N)) * N), b, acc[j][m]);
+                    }
                 }
             }
-        }
 #pragma unroll
-        for (int m = 0; m < 3; ++m) {
-            float2 e = make_float2(0.f, 0.f);
+            for (int m = 0; m < 3; ++m) {
+                float2 e = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int w = 0; w + 1 < NW; w += 2)
-                e = __ffma2_rn(make_float2(wt[m][w], wt[m][w + 1]), make_float2(s[w], s[w + 1]), e);
-            float t = e.x + e.y;
-            if (NW & 1) t = fmaf(wt[m][NW - 1], s[NW - 1], t);
-            acc[j][m] += t;
+                for (int w = 0; w + 1 < NW; w += 2)
+                    e = __ffma2_rn(make_float2(wt[m][w], wt[m][w + 1]), make_float2(s[w], s[w + 1]), e);
+                float t = e.x + e.y;
+                if (NW & 1) t = fmaf(wt[m][NW - 1], s[NW - 1], t);
+                acc[j][m] += t;
+            }
         }
+        if (PART < RUN)   // the other half's sums where this half's were: the loop is not unrolled
+#pragma unroll
+            for (int j = 0; j < PART; ++j)
+#pragma unroll
+                for (int m = 0; m < 3; ++m) {
+                    const float t = acc[j][m];
+                    acc[j][m] = acc[RUN - PART + j][m];
+                    acc[RUN - PART + j][m] = t;
+                }
     }
 }
 

@@ -115,3 +115,23 @@ def test_the_adjoint_keeps_a_nan_to_its_runs(sal, n, shape, p):
     t, x, y = np.nonzero(bad)
     assert abs(t - p[0]).max() <= n and abs(x - p[1]).max() < n
     assert y.min() >= p[2] - n + 1 and y.max() <= p[2] + n - 1 + more
+
+
+@pytest.mark.parametrize("value", [1e6, np.nan])
+@pytest.mark.parametrize("n", [8, 16, 32])
+def test_the_forward_keeps_an_extreme_value_to_its_runs(sal, n, value):
+    """An outlier anywhere reaches the outputs of its windows and those of their runs; the others are what they are
+    without it."""
+    shape, (xb, yb) = FORWARD[n]
+    r = np.random.RandomState(n)
+    V = r.randn(*shape).astype(np.float32)
+    p = (shape[0] // 2, xb + 2, yb + 3 - n // 2)   # in the windows of a brick's first outputs alone, so most of its run is free
+    V[p] = 0.0
+    clean = _features(sal, V, n)
+    V[p] = value
+    E = _features(sal, V, n)
+    own, free = _held(shape, p, n), ~_held(shape, p, n, RUN[n] - 1)
+    if np.isnan(value):
+        assert np.isnan(E[:, own]).all()
+    # two roundings of a feature, a few dozen 2^-24 each (another value may be taken from a brick at staging)
+    assert np.abs(E - clean)[:, free].max() <= 64 * 2.0 ** -24 * clean[:, free].min()
