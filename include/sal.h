@@ -171,7 +171,7 @@ sal_status sal_saliency_backward(sal_handle* h, const float* V, const float* W, 
  * The paper has no counterpart.  It computes what sal_combine computes, with the same arguments
  * and results (ls_delta as in sal_params), on the current device: S3, S and the non-NULL D, W_in,
  * W_out must be device memory of that device (else SAL_ERR_INVALID_ARG before any work).
- * Its reduction scratch is one file-scope device array of about 0.6 MiB that every GPU that
+ * Its reduction scratch is one file-scope device array of about 0.4 MiB that every GPU that
  * loads the library holds until the process exits.  Limit: T*X*Y <= 16,777,216 voxels; larger
  * volumes return SAL_ERR_UNSUPPORTED before any work.  The first call on a device looks up the
  * array's device address (cudaGetSymbolAddress) with that device current and keeps it for the

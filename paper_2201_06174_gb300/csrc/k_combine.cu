@@ -61,9 +61,9 @@ k3_minmax_finalize(const float* __restrict__ mm_part, int nparts, int nmaps, flo
 // The template fit by one block: W from the Gram partials (strided threads, then a tree), into norm and W_out.
 __device__ void fit_weights(const double* g_part, int nparts, double delta, float* norm, float* W_out, double* wsum) {
     __shared__ double s[9][kThreads];
-    for (int c = 0; c < 9; ++c) {
+    for (int c = 0; c < kGramSums; ++c) {
         double a = 0.0;
-        for (int i = threadIdx.x; i < nparts; i += kThreads) a += __ldcg(g_part + i * 16 + c);
+        for (int i = threadIdx.x; i < nparts; i += kThreads) a += __ldcg(g_part + i * kGramSums + c);
         s[c][threadIdx.x] = a;
     }
     __syncthreads();
@@ -129,7 +129,7 @@ k3_gram(const float* __restrict__ S3, const float* __restrict__ D, long long NV,
             for (int c = 0; c < 9; ++c) red[c][threadIdx.x] += red[c][threadIdx.x + s];
         __syncthreads();
     }
-    if (threadIdx.x < 9) g_part[blockIdx.x * 16 + threadIdx.x] = red[threadIdx.x][0];
+    if (threadIdx.x < kGramSums) g_part[blockIdx.x * kGramSums + threadIdx.x] = red[threadIdx.x][0];
     if (counter && tail::last_block(counter, tail::C_GRAM)) fit_weights(g_part, gridDim.x, delta, norm, W_out, wsum);
 }
 
@@ -263,7 +263,7 @@ constexpr int kNoAllocSlots = 4096;              // partial slots held by the st
 constexpr long long kNoAllocMaxVoxels = kNoAllocVoxPerBlock * kNoAllocSlots;  // 16,777,216
 
 struct NoAllocScratch {
-    double g_part[kNoAllocSlots * 16];
+    double g_part[kNoAllocSlots * sal::kGramSums];
     double wsum[16];
     float mm_part[kNoAllocSlots * 8];
     float norm[16];

@@ -58,7 +58,7 @@ constexpr size_t OFF_B2 = (G1_B + 127) / 128 * 128;
 constexpr size_t OFF_TAB = OFF_B2 + B2_B;                // A2, then the stage-3 B (the constant operands)
 constexpr size_t TAB_B = A2_B + B_B;
 constexpr size_t OFF_A = OFF_TAB + TAB_B;
-constexpr size_t WT_B = (size_t)3 * H * N * 4;           // Eq. 1 weights of one k_t, [map][|k_y|][k_x]; two, by k_t
+constexpr size_t WT_B = ((size_t)3 * H * H * 4 + 15) / 16 * 16;   // Eq. 1 weights of one k_t, [map][|k_y|][|k_x|]; two, by k_t
 constexpr size_t OFF_WT = OFF_A + 4 * A_B;               // (A_re, A_im) twice, by k_t
 constexpr size_t OFF_MISC = OFF_WT + 2 * WT_B;
 // mbarriers (arrivals): pass P complete (commit; by P % 6, so that a group waits for every phase of those it uses), buffer
@@ -369,7 +369,7 @@ k1_spectra_tc32(const float* __restrict__ V, float* __restrict__ E, int T, int X
 #pragma unroll
         for (int c = 0; c < 3; ++c)
 #pragma unroll
-            for (int k = 0; k < H; ++k) wt[c][k] = s_wt[(kt & 1) * (WT_B / 4) + (c * H + k) * N + kx];
+            for (int k = 0; k < H; ++k) wt[c][k] = s_wt[(kt & 1) * (WT_B / 4) + (c * H + k) * H + min(kx, N - kx)];
 #pragma unroll
         for (int i = 0; i < kOwn; ++i) {
             const int P = kt * kPasses + 2 * i + grp, buf = P % kBufs;
@@ -468,10 +468,6 @@ cudaError_t spectra_tc32_prepare(int fmt) {
 
 size_t spectra_tc32_tables_bytes() { return kWtOff + WT_FLOATS * sizeof(float); }
 
-size_t spectra_tc32_max_bytes(int T, int X, int Y) {
-    return (size_t)T * ((X + P - 1) / P) * ((Y + BY - 1) / BY) * sizeof(float);
-}
-
 cudaError_t spectra_tc32_tables_build(int fmt, const TwiddleTable& t, int feat, void* dst, cudaStream_t s) {
     static_assert(WT_FLOATS * sizeof(float) < (1u << 20), "a host copy");
     unsigned char* out = static_cast<unsigned char*>(dst);
@@ -481,16 +477,15 @@ cudaError_t spectra_tc32_tables_build(int fmt, const TwiddleTable& t, int feat, 
     note_launches(1);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    float* wt = new float[WT_FLOATS];
+    float* wt = new float[WT_FLOATS]();
     for (int kt = 0; kt < H; ++kt)
         for (int k = 0; k < H; ++k)
-            for (int kx = 0; kx < N; ++kx) {
+            for (int j = 0; j < H; ++j) {
                 const float mult = (kt == 0 || 2 * kt == N) ? 1.f : 2.f;
-                const int j = kx < N / 2 ? kx : kx - N;
                 float w[3];
                 if (feat == 1) f32::bin_weights<true>(kt, j, k, mult / (float)(N * N * N), w[0], w[1], w[2]);
                 else f32::bin_weights<false>(kt, j, k, mult / (float)(N * N * N), w[0], w[1], w[2]);
-                for (int c = 0; c < 3; ++c) wt[((size_t)(kt * 3 + c) * H + k) * N + kx] = w[c];
+                for (int c = 0; c < 3; ++c) wt[(size_t)kt * (WT_B / 4) + (c * H + k) * H + j] = w[c];
             }
     e = cudaMemcpyAsync(out + kWtOff, wt, WT_FLOATS * sizeof(float), cudaMemcpyHostToDevice, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);   // wt is pageable and leaves

@@ -29,7 +29,8 @@ struct sal_handle {
     void* tc_tables = nullptr;  // constant tensor-core operands of K1 (BF16/FP16 forms)
     void* adj_tables = nullptr; // constant tensor-core operands of K5 (FP16)
     float* f32_wt = nullptr;    // Eq. 1 weight table of the FP32 K1 / K5 (n <= 16)
-    float* slide_wt = nullptr;  // Eq. 1 weight table of the sliding FP32 K1 (stride 1) and K5 (n <= 16): rect cubes
+    float* slide_wt = nullptr;  // Eq. 1 weight table of the sliding FP32 K1 (stride 1) and K5 (n <= 16): rect cubes, where
+                                // the budget holds it
     float* sp_tab = nullptr;    // spatial-domain reading: the Eq. 1 ratio table
     float* vpad = nullptr;      // V with rows padded to ypad floats (tensor-core forms, Y not a multiple of 4)
     int ypad = 0;
@@ -342,15 +343,15 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
     if (e != cudaSuccess) { delete h; return cuda_fail(nullptr, e, "kernel attributes"); }
 
     const size_t plane3 = (size_t)3 * h->N * sizeof(float);
-    const size_t small = (size_t)sal::kRedBlocks * 8 * sizeof(float) + (size_t)sal::kRedBlocks * 16 * sizeof(double)
-                         + 32 * sizeof(float) + 16 * sizeof(double) + 256;   // (the block counters in the last)
+    const size_t parts = (size_t)sal::kRedBlocks * std::max(8 * sizeof(float), sal::kGramSums * sizeof(double));
+    const size_t small = parts + 32 * sizeof(float) + 16 * sizeof(double) + 256;   // (the block counters in the last)
     const bool tc_fwd = h->prec != SAL_FP32 && sal::spectra_tc_supported(h->n);
     const bool tc32 = h->prec != SAL_FP32 && h->n == 32;
     const size_t tab_bytes = tc_fwd ? sal::spectra_tc_tables_bytes(h->n) : tc32 ? sal::spectra_tc32_tables_bytes() : 0;
     const size_t adj_bytes = tc_fwd ? sal::spectra_adjoint_tc_tables_bytes(h->n) : 0;
     const bool f32_tab = h->prec == SAL_FP32 && sal::spectra_f32_supported(h->n) && h->feature != 2;
     const size_t wt_bytes = f32_tab ? sal::f32_weight_table_floats(h->n) * sizeof(float) : 0;
-    const size_t sl_bytes = slide ? sal::f32_slide_table_floats(h->n) * sizeof(float) : 0;
+    size_t sl_bytes = slide ? sal::f32_slide_table_floats(h->n) * sizeof(float) : 0;
     const size_t sp_bytes = h->feature == 2 ? sal::spatial_weight_table_floats(h->n) * sizeof(float) : 0;
     const int sc = p->stride;
     const size_t ec_bytes = sc > 1 ? (size_t)3 * ((T + sc - 1) / sc) * ((X + sc - 1) / sc) * ((Y + sc - 1) / sc) *
@@ -359,8 +360,11 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
     // the tensor-core forms stage interior bricks by TMA from a row-padded copy when rows are not 16-byte multiples
     const int ypad = (Y + 3) & ~3;
     const size_t vpad_bytes = tc_fwd && h->feature != 2 && ypad != Y ? (size_t)T * X * ypad * sizeof(float) : 0;
-    const size_t need = 2 * plane3 + small + tab_bytes + adj_bytes + ec_bytes + wt_bytes + sl_bytes + sp_bytes +
-                        vpad_bytes;
+    size_t need = 2 * plane3 + small + tab_bytes + adj_bytes + ec_bytes + wt_bytes + sl_bytes + sp_bytes + vpad_bytes;
+    if (sl_bytes && h->budget && need > h->budget) {   // without the sliding forms' table: the direct forms run
+        need -= sl_bytes;
+        sl_bytes = 0;
+    }
     if (h->budget && need > h->budget) {
         delete h;
         return fail(nullptr, SAL_ERR_OOM, "scratch (" + std::to_string(need) + " B) exceeds hbm_budget_bytes");
@@ -389,11 +393,10 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
     h->ypad = h->vpad ? ypad : 0;
     char* b = static_cast<char*>(h->small);
     h->red.g_part = reinterpret_cast<double*>(b);
-    b += (size_t)sal::kRedBlocks * 16 * sizeof(double);
+    h->red.mm_part = reinterpret_cast<float*>(b);
+    b += parts;
     h->red.wsum = reinterpret_cast<double*>(b);
     b += 16 * sizeof(double);
-    h->red.mm_part = reinterpret_cast<float*>(b);
-    b += (size_t)sal::kRedBlocks * 8 * sizeof(float);
     h->red.norm = reinterpret_cast<float*>(b);
     h->red.counter = reinterpret_cast<unsigned*>(b + 32 * sizeof(float));
     {
@@ -448,7 +451,7 @@ sal_status sal_create(const sal_params* p_in, int T, int X, int Y, sal_handle** 
         const sal_status us = upload_table(h, wt, &h->f32_wt);
         if (us != SAL_OK) return us;
     }
-    if (slide) {
+    if (sl_bytes) {
         std::vector<float> wt(sal::f32_slide_table_floats(h->n));
         sal::f32_slide_table_fill(h->n, h->feature, wt.data());
         const sal_status us = upload_table(h, wt, &h->slide_wt);
@@ -567,7 +570,7 @@ sal_status ensure_backward_scratch(sal_handle* h) {
     if (h->n == 32) return fail(h, SAL_ERR_UNSUPPORTED, "the backward is built for n in {2,4,8,16}");
     if (h->gE) return SAL_OK;
     const int sc = h->stride;
-    h->adj_slide = h->prec == SAL_FP32 && h->feature != 2 && h->taper == 0 && (h->n == 8 || h->n == 16);
+    h->adj_slide = h->slide_wt && (h->n == 8 || h->n == 16);
     sal::SpectraAdjointGeometry g;
     size_t per_t, per_ext, ext_fixed;
     auto sizes = [&]() {

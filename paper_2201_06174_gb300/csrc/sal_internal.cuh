@@ -68,10 +68,13 @@ __host__ __device__ __forceinline__ int ext_index(int i, int n, int mode) {
     return ext_index_any(i, n, mode);
 }
 
-// Scratch for the volume-wide reductions (device memory owned by the handle).
+constexpr int kGramSums = 9;     // sums of the template fit: the Gram matrix's upper triangle and the right-hand side
+
+// Scratch for the volume-wide reductions (device memory owned by the handle, where the two kinds of partials share theirs: no
+// call has both at a time).
 struct Reduce {
     float* mm_part;     // [kRedBlocks][8]  per-block min/max partials
-    double* g_part;     // [kRedBlocks][16] per-block FP64 partial sums
+    double* g_part;     // [kRedBlocks][kGramSums] per-block FP64 partial sums
     float* norm;        // [16]: lo[3], inv[3], W[3], loC, invC, flags
     double* wsum;       // [16]: reduced FP64 sums (Gram, gradient of W)
     unsigned* counter;  // [4]: blocks of a launch that are done, by kernel (reduce_tail.cuh); null: no fused tails
@@ -129,8 +132,7 @@ cudaError_t spectra_tc32_prepare(int fmt);
 // tables: its constant operands and Eq. 1 weights, built once per handle (synchronises the stream)
 size_t spectra_tc32_tables_bytes();
 cudaError_t spectra_tc32_tables_build(int fmt, const TwiddleTable& tw, int feat, void* tables, cudaStream_t s);
-// pmax: scratch of spectra_tc32_max_bytes (the bricks' plane maxima)
-size_t spectra_tc32_max_bytes(int T, int X, int Y);
+// pmax: scratch for the bricks' plane maxima, T ceil(X / 4) ceil(Y / 16) floats (no more than a map)
 cudaError_t spectra_tc32_launch(int fmt, const TwiddleTable& tw, const void* tables, float* pmax, const float* V,
                                 float* E, int T, int X, int Y, int bnd, int feat, int stride, int* err,
                                 cudaStream_t s);
