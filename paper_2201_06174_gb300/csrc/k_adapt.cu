@@ -32,13 +32,16 @@ namespace sal {
 namespace {
 
 enum : int { ADAPT_LMS = 0, ADAPT_NLMS = 1, ADAPT_RLS = 2 };
+enum : int { kTodoChain = 1, kTodoErrors = 2 };
 
 __global__ void __launch_bounds__(32)
 k3_adapt(const float* __restrict__ S3, const float* __restrict__ D, int T, int X, int Y, int method, double mu,
          double eps, double lambda, double delta, int sec, const float* __restrict__ norm, float* __restrict__ W_out,
          float* __restrict__ err2, const int* __restrict__ todo) {
-    // todo (nullable): per chain, whether the regrouped form has left it to this kernel
-    if (todo && !todo[blockIdx.x]) return;
+    // todo (nullable): per chain, what the regrouped form has left to this kernel: nothing, all (kTodoChain) or only the
+    // errors (kTodoErrors: its weights stand, and are the same whether err2 is asked for or not)
+    const int left = todo ? todo[blockIdx.x] : kTodoChain;
+    if (left == 0) return;
     __shared__ double s_x[2][4][32];   // two chunks of 32 steps: x_t, x_x, x_y, d
     const long long NV = (long long)T * X * Y;
     const int lane = threadIdx.x;
@@ -111,7 +114,7 @@ k3_adapt(const float* __restrict__ S3, const float* __restrict__ D, int T, int X
         }
         __syncwarp();
     }
-    if (lane == 0) {
+    if (lane == 0 && left == kTodoChain) {
         W_out[blockIdx.x * 3 + 0] = (float)w0;
         W_out[blockIdx.x * 3 + 1] = (float)w1;
         W_out[blockIdx.x * 3 + 2] = (float)w2;
@@ -316,7 +319,7 @@ k3_adapt_segments(const float* __restrict__ S3, const float* __restrict__ D, Seg
         double* o = segs + ((long long)y * g.nseg + seg) * St::K;
 #pragma unroll
         for (int i = 0; i < St::K; ++i) o[i] = s.v[i];
-        if (s.bad()) todo[y / g.sec] = 1;
+        if (s.bad()) todo[y / g.sec] = kTodoChain;
     }
     // the group's state: a tree over its 32 segments in order (absent ones are the identity)
 #pragma unroll
@@ -336,7 +339,7 @@ k3_adapt_segments(const float* __restrict__ S3, const float* __restrict__ D, Seg
         double* o = groups + ((long long)y * g.ngroup + blockIdx.x) * St::K;
 #pragma unroll
         for (int i = 0; i < St::K; ++i) o[i] = s.v[i];
-        if (s.bad()) todo[y / g.sec] = 1;
+        if (s.bad()) todo[y / g.sec] = kTodoChain;
     }
 }
 
@@ -390,7 +393,7 @@ k3_adapt_chain(SegGeo g, const double* __restrict__ groups, double* __restrict__
     const int bad = __syncthreads_or(unsound);
     if (bad || todo[blockIdx.x]) {
         __syncthreads();
-        if (tid == 0) todo[blockIdx.x] = 1;
+        if (tid == 0) todo[blockIdx.x] = kTodoChain;
         return;   // block-uniform: the step-by-step filter takes this chain
     }
     Sa st;
@@ -409,7 +412,7 @@ k3_adapt_chain(SegGeo g, const double* __restrict__ groups, double* __restrict__
 #pragma unroll
             for (int m = 0; m < 3; ++m) W_out[blockIdx.x * 3 + m] = (float)w[m];
         } else {
-            todo[blockIdx.x] = 1;
+            todo[blockIdx.x] = kTodoChain;
         }
     }
     if (!starts) return;
@@ -476,7 +479,7 @@ k3_adapt_errors(const float* __restrict__ S3, const float* __restrict__ D, SegGe
     double w[3], P[6];
     const long long per = (long long)g.X * g.T, r0 = (long long)seg * g.L;
     if (!st.weights(w, P)) {   // a segment inside the chain where R is still near singular
-        todo[y / g.sec] = 1;
+        if (todo[y / g.sec] == 0) todo[y / g.sec] = kTodoErrors;
         return;
     }
     const double iv[3] = {norm[3], norm[4], norm[5]}, nlo[3] = {-(norm[0] * iv[0]), -(norm[1] * iv[1]), -(norm[2] * iv[2])};
