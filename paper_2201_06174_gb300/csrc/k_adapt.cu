@@ -559,10 +559,11 @@ void regrouped_launch(const float* S3, const float* D, const SegPlan& p, const f
 }  // namespace
 
 // The regrouped form wherever its scratch fits (about 6 bytes a voxel against the 12 of the handle's feature planes;
-// sections of less than about 40 samples do not) and the chains are at least kMinChain steps long: below that the
-// step-by-step filter's 0.8 us a step costs less than three more launches.  RLS only with lambda = 1, where its
-// information form is a plain sum.
-constexpr long long kMinChain = 64;
+// sections of less than about 40 samples do not) and the chains are long enough: its launches take 78 to 109 us (LMS), 84 to
+// 121 (NLMS) and 48 to 94 (RLS) without and with the errors on 12 x 16 x 20 voxels, in which the step-by-step filter, all
+// chains side by side, takes 192 steps of 0.36 (LMS), 0.80 and 1.77 us.  RLS only with lambda = 1, where its information
+// form is a plain sum.
+constexpr long long min_chain(int method) { return method == ADAPT_LMS ? 272 : method == ADAPT_NLMS ? 136 : 64; }
 
 cudaError_t adapt_launch(const float* S3, const float* D, int T, int X, int Y, int method, double mu, double eps,
                          double lambda, double delta, int sections, const float* norm, float* W_out, float* err2,
@@ -570,7 +571,7 @@ cudaError_t adapt_launch(const float* S3, const float* D, int T, int X, int Y, i
     const int sec = sections > 0 ? std::min(sections, Y) : Y;
     const int blocks = (Y + sec - 1) / sec;
     SegPlan p = seg_plan(T, X, Y, sec);
-    const bool regroup = scratch && p.bytes <= scratch_bytes && (long long)T * X * sec >= kMinChain &&
+    const bool regroup = scratch && p.bytes <= scratch_bytes && (long long)T * X * sec >= min_chain(method) &&
                          (Y + kSegY - 1) / kSegY <= 65535 && (method != ADAPT_RLS || lambda == 1.0);
     const int* todo = nullptr;
     if (regroup) {

@@ -71,3 +71,22 @@ def test_a_chain_that_grows_follows_the_filter(sal, sections):
     # x carries the 1e-7 of an FP32 reciprocal, up to 270 steps of it
     assert np.abs(W - want).max() <= 270 * 1e-6 * np.abs(want).max()
     assert np.linalg.norm(err2 - want_e) <= 2 * 270 * 1e-6 * np.linalg.norm(want_e)
+
+
+@pytest.mark.parametrize("method,shape,regrouped", [
+    ("lms", (16, 17, 3), True), ("lms", (15, 18, 3), False), ("lms", (12, 16, 20), False),
+    ("nlms", (8, 17, 5), True), ("nlms", (9, 15, 5), False), ("rls", (8, 8, 9), True), ("rls", (7, 9, 9), False),
+])
+def test_short_chains_run_step_by_step(sal, method, shape, regrouped):
+    """On both sides of the chain length from which the regrouped form's launches cost less than the filter's steps (two
+    launches, the bounds and the filter): the same values."""
+    r = np.random.RandomState(3)
+    S3 = (np.abs(r.randn(3, *shape)) * 0.2 + 0.05).astype(np.float32)
+    D = (S3[0] * 1.5 + 0.1 * r.randn(*shape)).astype(np.float32)
+    before = sal.sal_launch_count()
+    W, W_only, err2 = _run(sal, S3, D, method=method, sections=1)
+    assert sal.sal_launch_count() - before == (5 + 4 if regrouped else 2 + 2)
+    want, want_e = _filter(S3, D, 1, method=method)
+    assert np.array_equal(W, W_only)
+    assert np.abs(W - want).max() <= 1e-5 * max(1.0, np.abs(want).max())
+    assert np.linalg.norm(err2 - want_e) <= 1e-5 * np.linalg.norm(want_e)
