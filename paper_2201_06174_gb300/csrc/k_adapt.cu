@@ -26,7 +26,7 @@
 #include <algorithm>
 #include <cfloat>
 
-#include "sal_internal.cuh"
+#include "reduce_tail.cuh"
 
 namespace sal {
 namespace {
@@ -37,7 +37,8 @@ enum : int { kTodoChain = 1, kTodoErrors = 2 };
 __global__ void __launch_bounds__(32)
 k3_adapt(const float* __restrict__ S3, const float* __restrict__ D, int T, int X, int Y, int method, double mu,
          double eps, double lambda, double delta, int sec, const float* __restrict__ norm, float* __restrict__ W_out,
-         float* __restrict__ err2, const int* __restrict__ todo) {
+         float* __restrict__ err2, const int* __restrict__ todo, unsigned* __restrict__ counter) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) counter[tail::C_MAPS] = 0u;   // (reduce_tail.cuh)
     // todo (nullable): per chain, what the regrouped form has left to this kernel: nothing, all (kTodoChain) or only the
     // errors (kTodoErrors: its weights stand, and are the same whether err2 is asked for or not)
     const int left = todo ? todo[blockIdx.x] : kTodoChain;
@@ -566,8 +567,9 @@ void regrouped_launch(const float* S3, const float* D, const SegPlan& p, const f
 constexpr long long min_chain(int method) { return method == ADAPT_LMS ? 272 : method == ADAPT_NLMS ? 136 : 64; }
 
 cudaError_t adapt_launch(const float* S3, const float* D, int T, int X, int Y, int method, double mu, double eps,
-                         double lambda, double delta, int sections, const float* norm, float* W_out, float* err2,
+                         double lambda, double delta, int sections, const Reduce& r, float* W_out, float* err2,
                          void* scratch, size_t scratch_bytes, cudaStream_t s) {
+    const float* norm = r.norm;
     const int sec = sections > 0 ? std::min(sections, Y) : Y;
     const int blocks = (Y + sec - 1) / sec;
     SegPlan p = seg_plan(T, X, Y, sec);
@@ -586,7 +588,8 @@ cudaError_t adapt_launch(const float* S3, const float* D, int T, int X, int Y, i
         else regrouped_launch<false>(S3, D, p, norm, W_out, err2, b, s);
         todo = reinterpret_cast<const int*>(b + p.todo);
     }
-    k3_adapt<<<blocks, 32, 0, s>>>(S3, D, T, X, Y, method, mu, eps, lambda, delta, sec, norm, W_out, err2, todo);
+    k3_adapt<<<blocks, 32, 0, s>>>(S3, D, T, X, Y, method, mu, eps, lambda, delta, sec, norm, W_out, err2, todo,
+                                  r.counter);
     note_launches(1);
     return cudaGetLastError();
 }

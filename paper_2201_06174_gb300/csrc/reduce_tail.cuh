@@ -12,8 +12,10 @@ namespace sal {
 namespace tail {
 
 constexpr int kTailThreads = 256;
-// The counters of a handle, one per kernel of a call.  Each is zero again when its launch ends; a launch also clears the
-// others', so that calls that overlapped on one handle (which it does not allow) leave nothing behind for the next.
+// The counters of a handle, one per kernel of a call.  Each is zero again when its launch ends, unless calls overlapped on the
+// handle (which it does not allow).  What these leave is cleared before it is counted on again: a launch clears the others'
+// counters, every call begins with C_MAPS, and each call that uses it has a launch behind it that clears C_MAPS (the adaptive
+// filter's own, where no second counter is in use).
 enum : int { C_MAPS = 0, C_GRAM = 1, C_COMBINE = 2, C_WEIGHTS = 3 };
 enum : int { N_LO = 0, N_INV = 3, N_W = 6, N_LOC = 9, N_INVC = 10 };   // layout of Reduce::norm
 

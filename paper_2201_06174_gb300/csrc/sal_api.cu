@@ -770,7 +770,7 @@ sal_status sal_adapt_weights(sal_handle* h, const float* S3, const float* D, con
     cudaError_t e;
     if ((e = sal::minmax_bounds_launch(S3, h->N, h->red, st)) != cudaSuccess) return cuda_fail(h, e, "adapt: bounds");
     if ((e = sal::adapt_launch(S3, D, h->T, h->X, h->Y, (int)p->method, p->mu, p->eps, p->lambda, p->delta,
-                               p->sections, h->red.norm, W_out, err2, h->E, (size_t)3 * h->N * sizeof(float), st)) !=
+                               p->sections, h->red, W_out, err2, h->E, (size_t)3 * h->N * sizeof(float), st)) !=
         cudaSuccess)
         return cuda_fail(h, e, "adapt");
     return SAL_OK;

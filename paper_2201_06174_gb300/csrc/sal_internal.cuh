@@ -155,7 +155,7 @@ cudaError_t minmax_bounds_launch(const float* S3, long long N, const Reduce& r, 
 // W_out [blocks][3]; err2 (nullable) the squared error of every step in filter order.  scratch: device memory
 // (8-byte aligned) for the regrouped form of the chains, about 6 bytes a voxel; with less the chains run step by step.
 cudaError_t adapt_launch(const float* S3, const float* D, int T, int X, int Y, int method, double mu, double eps,
-                         double lambda, double delta, int sections, const float* norm, float* W_out, float* err2,
+                         double lambda, double delta, int sections, const Reduce& r, float* W_out, float* err2,
                          void* scratch, size_t scratch_bytes, cudaStream_t s);
 
 // ---- K2: directional center-surround ----------------------------------------------------------
