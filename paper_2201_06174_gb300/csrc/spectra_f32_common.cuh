@@ -102,7 +102,7 @@ template <int N_, int BY_, int NT_> struct Brick {
         const int tid = threadIdx.x;
         const int yy = tid % YH;
         const int r0 = tid / YH;
-        const int gy = ext_index(y_start - N / 2 + yy, Y, bnd);
+        const int gy = ext_index_any(y_start - N / 2 + yy, Y, bnd);
         if (r0 < RSTEP) {
             float v[ITERS];
 #pragma unroll
@@ -111,8 +111,8 @@ template <int N_, int BY_, int NT_> struct Brick {
                 v[i] = 0.f;
                 if (r < N * N) {
                     const int ut = r / N, ux = r % N;
-                    const int gt = ext_index(t0 - N / 2 + ut, T, bnd);
-                    const int gx = ext_index(x0 - N / 2 + ux, X, bnd);
+                    const int gt = ext_index_any(t0 - N / 2 + ut, T, bnd);
+                    const int gx = ext_index_any(x0 - N / 2 + ux, X, bnd);
                     if ((gt | gx | gy) >= 0) v[i] = __ldg(V + ((size_t)gt * X + gx) * Y + gy);
                 }
             }
