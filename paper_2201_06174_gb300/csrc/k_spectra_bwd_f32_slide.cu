@@ -237,8 +237,12 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
                 }
                 rho[NW - 1] = fmaf(g0, wt[0][NW - 1], fmaf(g1, wt[1][NW - 1], g2 * wt[2][NW - 1]));
             };
-            // the small-bin level of output j, squared; it also keeps subnormal |F|^2 away from rsqrt
-            auto level = [&](int j) { return fmaxf(kSmallBin * l1[j] * (kSmallBin * l1[j]), 1e-30f); };
+            // the small-bin level of output j, squared; it also keeps subnormal |F|^2 away from rsqrt.  A window of zeros has no
+            // direction: what the recursion leaves there is the rounding of samples that have left it
+            auto level = [&](int j) {
+                const float a = kSmallBin * l1[j];
+                return l1[j] == 0.f ? 3.4e38f : fmaxf(a * a, 1e-30f);
+            };
             // small bins at output j (bit k_y; tile 0: bit q of the pairs' first and second values) onto the list
             auto note = [&](int j, unsigned small_a, unsigned small_b) {
                 const uint32_t my = s_van[1 + RX + j];

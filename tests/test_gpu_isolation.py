@@ -135,3 +135,18 @@ def test_the_forward_keeps_an_extreme_value_to_its_runs(sal, n, value):
         assert np.isnan(E[:, own]).all()
     # two roundings of a feature, a few dozen 2^-24 each (another value may be taken from a brick at staging)
     assert np.abs(E - clean)[:, free].max() <= 64 * 2.0 ** -24 * clean[:, free].min()
+
+
+@pytest.mark.parametrize("n", [8, 16])
+def test_windows_of_zeros_have_no_gradient(sal, n):
+    """A muted volume: zeros behind the samples along y, and beside them.  Outputs whose windows hold nothing else get no
+    gradient through |F| = 0, wherever in a run they lie."""
+    r = np.random.RandomState(n)
+    shape = (5, 20, 3 * n + 21)
+    for end in range(n // 2, n // 2 + 9):
+        V, gE = np.zeros(shape, np.float32), r.randn(3, *shape).astype(np.float32)
+        V[:, 4:9, :end] = r.randn(5, 5, end)
+        got = _adjoint(sal, V, gE, n)
+        assert (got[:, :, end + 2 * n - 1:] == 0).all()
+        want = oracle.features_adjoint(V, gE, n, boundary="zero")
+        assert np.linalg.norm(got - want) <= 1e-5 * np.linalg.norm(want)
