@@ -420,11 +420,11 @@ k5_listed_apply_f32(float* __restrict__ blocks, const int* __restrict__ lists, l
 // and G2 of all rows in shared memory, then 16 terms a bin instead of the direct sum's 4096 (n = 16).  The x0 of a brick are
 // dealt to the CTAs of a cluster, which add their parts to the brick's block in the order of x0.
 constexpr int kDenseRun = 16;      // outputs of a sliding brick along y
-constexpr int kDenseCluster = 4;
 template <int N> struct DGeo {
     using G = BGeo<N>;
     static constexpr int XY = kDenseRun + N - 1;   // odd: rows XY float4 apart meet no bank conflict
     static constexpr int KG = 4;                   // k_t a group, in the FP32 G1's place
+    static constexpr int CLUSTER = N == 8 ? 8 : 4;   // CTAs a brick's 16 (n = 16: 12) x0 are dealt to
     static constexpr size_t X2_OFF = (G::SMEM + 15) / 16 * 16;
     static constexpr size_t EX_OFF = X2_OFF + (size_t)G::ROWS * XY * 16;
     static constexpr size_t SMEM = EX_OFF + (size_t)4 * N * 4;
@@ -783,14 +783,15 @@ k5_spectra_adjoint_f32(const float* __restrict__ V, const float* __restrict__ gE
 
 // The bricks the sliding form leaves (dense[brick] set: more small bins than it lists): cluster c looks through the marks of
 // bricks c, c + C, .. 32 at a time.  Constant volumes, n = 16: 48^3 42 ms (a direct sum per bin, a CTA per brick: 3.87 s),
-// 6 x 8 x 10 1.1 ms (409 ms); n = 8: 3.0 ms (70 ms) and 0.19 ms (5.8 ms).  Bound: the latency of float-float chains.
+// 6 x 8 x 10 1.1 ms (409 ms); n = 8: 3.0 ms (70 ms) and 0.15 ms (5.8 ms).  Bound: the latency of float-float chains.
 template <int N>
-__global__ void __cluster_dims__(kDenseCluster, 1, 1) __launch_bounds__(BGeo<N>::NT, DGeo<N>::CTAS)
+__global__ void __cluster_dims__(DGeo<N>::CLUSTER, 1, 1) __launch_bounds__(BGeo<N>::NT, DGeo<N>::CTAS)
 k5_dense_f32(const float* __restrict__ V, const float* __restrict__ gE, float* __restrict__ blocks, int T, int X, int Y,
              int bnd, int t_begin, int t_step, int t_count, const float* __restrict__ wtab,
              const __grid_constant__ Tw<N> tw, const __grid_constant__ Exact2f<N> ex,
              const __grid_constant__ VanishTab vt, const SpectraAdjointGeometry dg, const int* __restrict__ dense) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    constexpr int kDenseCluster = DGeo<N>::CLUSTER;
     const auto cluster = cooperative_groups::this_cluster();
     float* s_ex = reinterpret_cast<float*>(smem_raw + DGeo<N>::EX_OFF);
     for (int i = threadIdx.x; i < 4 * N; i += BGeo<N>::NT) {
@@ -879,8 +880,8 @@ cudaError_t launch_dense(const TwiddleTable& t, const float* wtab, const float* 
     const SpectraAdjointGeometry g = spectra_adjoint_f32_slide_geometry(N);
     const long long total = (long long)((Y + g.BY - 1) / g.BY) * ((X + g.BX - 1) / g.BX) * t_count;
     if (g.BY != kDenseRun || g.YH != DGeo<N>::XY) return cudaErrorInvalidValue;
-    const long long clusters = std::max(1, DGeo<N>::CTAS * device_sms() / kDenseCluster);
-    const int grid = (int)std::min(total, clusters) * kDenseCluster;
+    const long long clusters = std::max(1, DGeo<N>::CTAS * device_sms() / DGeo<N>::CLUSTER);
+    const int grid = (int)std::min(total, clusters) * DGeo<N>::CLUSTER;
     k5_dense_f32<N><<<grid, G::NT, DGeo<N>::SMEM, s>>>(V, gE, blocks, T, X, Y, bnd, t_begin, t_step, t_count, wtab,
                                                  f32::make_tw<N>(t), make_exact2f<N>(0),
                                                  make_vanish_tab(N, T, X, Y, bnd, 0), g, dense);

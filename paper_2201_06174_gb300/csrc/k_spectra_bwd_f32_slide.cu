@@ -15,8 +15,8 @@
 //   which replaces the tile's G1; after all tiles the adjoint of stage 1 writes the brick's block.
 // Small bins (|F| <= 2^-16 of the window's L1 norm) take Gamma = 0 in the tile loop and go to the brick's list; at the
 // end, in the order of their codes, its warps recompute them as direct float-float sums, and their rank-one gradients
-// are added to the gradient of G1 (256 terms each; at the block they would be 4096).  A brick with more than kList
-// such bins (constant regions: every bin) is marked and left to k5_dense_f32.
+// are added to the gradient of G1 (256 terms each; at the block they would be 4096).  A brick with more than
+// list_max such bins (constant regions: every bin) is marked and left to k5_dense_f32.
 // The instruction cache sets how far the loop over outputs is unrolled: by R, and not at all in tile 0, whose packed rows
 // need the most code for an eighth of the work (there every window is an FFT).
 // Bound: issue slots, about 500 per thread and output of 16 bins with the FFTs and the small bins (128 MUFU cycles), by 12
@@ -44,7 +44,7 @@ using f32::vanish_mask;
 using f32::VanishTab;
 
 constexpr int kRun = 16;     // outputs of a brick along y
-constexpr int kList = 1024;  // small bins a brick can list
+constexpr int kList = 1024;  // small bins a brick can list at most
 constexpr int kChunk = 64;   // small bins whose Gamma is held at a time
 
 // n = 8: a brick of 16 x0 per CTA of 128 threads, four CTAs an SM.  n = 16: bricks of 12 x0 in groups of 192 threads,
@@ -95,7 +95,7 @@ template <int N, bool EN, int GROUPS>
 __global__ void __launch_bounds__(Adj<N, GROUPS>::NT, AGeo<N>::CTAS)
 k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __restrict__ blocks, int T, int X, int Y,
          int bnd, int t_begin, int t_step, const float* __restrict__ wtab, const __grid_constant__ Exact2f<N> ex,
-         const __grid_constant__ VanishTab vt, int* __restrict__ dense) {
+         const __grid_constant__ VanishTab vt, int* __restrict__ dense, int list_max) {
     using G = Adj<N, GROUPS>;
     using B = Bins<N, false>;
     constexpr int RX = G::RX, R = AGeo<N>::R, XH = G::XH, YH = G::YH, GT = G::GT, H = G::H, TILES = G::TILES, NW = B::NW;
@@ -438,8 +438,8 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
     if (!EN) {
         group_sync();
         const int total = *s_count;
-        if (tid == 0) dense[id] = total > kList;
-        if (total > kList) return;   // whole group: this brick's block comes from k5_dense_f32
+        if (tid == 0) dense[id] = total > list_max;
+        if (total > list_max) return;   // whole group: this brick's block comes from k5_dense_f32
         int* s_list = reinterpret_cast<int*>(s_g2);   // the codes in increasing order (G2 is free)
         for (int i = tid; i < total; i += GT) {
             const int c = s_small[i];
@@ -563,26 +563,34 @@ template <int N, int GROUPS> cudaError_t prepare_g() {
 
 template <int N, int GROUPS>
 void launch_g(const float* wtab, const float* V, const float* gE, float* blocks, int T, int X, int Y, int bnd, int feat,
-              int t_begin, int t_step, int t_count, int bricks, int* dense, cudaStream_t s) {
+              int t_begin, int t_step, int t_count, int bricks, int* dense, int list_max, cudaStream_t s) {
     using G = Adj<N, GROUPS>;
     const dim3 grid((bricks + GROUPS - 1) / GROUPS, 1, t_count);
     const Exact2f<N> ex = f32::make_exact2f<N>(0);
     if (feat == 1)
         k5_slide<N, true, GROUPS><<<grid, G::NT, G::SMEM, s>>>(V, gE, blocks, T, X, Y, bnd, t_begin, t_step, wtab, ex,
-                                                               VanishTab{}, dense);
+                                                               VanishTab{}, dense, list_max);
     else
         k5_slide<N, false, GROUPS><<<grid, G::NT, G::SMEM, s>>>(V, gE, blocks, T, X, Y, bnd, t_begin, t_step, wtab, ex,
-                                                                f32::make_vanish_tab(N, T, X, Y, bnd, 0), dense);
+                                                                f32::make_vanish_tab(N, T, X, Y, bnd, 0), dense,
+                                                                list_max);
 }
 
 template <int N>
 cudaError_t launch_n(const float* wtab, const float* V, const float* gE, float* blocks, int T, int X, int Y, int bnd,
                      int feat, int t_begin, int t_step, int t_count, int* dense, cudaStream_t s) {
     const int bricks = ((Y + kRun - 1) / kRun) * ((X + AGeo<N>::RX - 1) / AGeo<N>::RX);
-    if ((long long)bricks * t_count <= device_sms())
-        launch_g<N, 1>(wtab, V, gE, blocks, T, X, Y, bnd, feat, t_begin, t_step, t_count, bricks, dense, s);
+    // n = 8: a listed bin takes 0.4 us of its brick's time, k5_dense_f32 about 100 us for all of them, but many bricks side by
+    // side 6.6 us each against 0.4 for a full list.  So the list ends early where the bricks leave SMs idle (one sample set
+    // in 12 x 16 x 20: 590 -> 140 us; 5 % of them 440 -> 195), and at half in larger launches (a lone spike in 64^3
+    // 640 -> 207 us, 1 % of the samples 1170 -> 1114).  n = 16, k5_dense_f32 about 1 ms: at its end.
+    const bool few = (long long)bricks * t_count <= device_sms();
+    const int list_max = N == 8 ? (few ? 128 : 512) : kList;
+    if (few)
+        launch_g<N, 1>(wtab, V, gE, blocks, T, X, Y, bnd, feat, t_begin, t_step, t_count, bricks, dense, list_max, s);
     else
-        launch_g<N, AGeo<N>::GROUPS>(wtab, V, gE, blocks, T, X, Y, bnd, feat, t_begin, t_step, t_count, bricks, dense, s);
+        launch_g<N, AGeo<N>::GROUPS>(wtab, V, gE, blocks, T, X, Y, bnd, feat, t_begin, t_step, t_count, bricks, dense,
+                                     list_max, s);
     note_launches(1);
     return cudaGetLastError();
 }

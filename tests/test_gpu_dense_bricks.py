@@ -68,7 +68,9 @@ def test_dense_bricks_match_oracle(sal, n, shape, boundary, stride, planes):
 @pytest.mark.parametrize("n", [8, 16])
 def test_dense_bricks_are_spread_over_the_device(sal, n):
     """A few constant bricks against a textured volume of the same size: 3 (n = 8) and 8 (n = 16) times as long with separable
-    float-float spectra, 23 and 430 with a direct sum per bin, 100 and 2900 with those by one CTA per brick."""
+    float-float spectra, 23 and 430 with a direct sum per bin, 100 and 2900 with those by one CTA per brick.  And bricks
+    with a few hundred to a thousand small bins (a lone sample): 2 and 7 times as long, 6 and 150 with a CTA per x position,
+    20 and 700 with one per brick."""
     shape = (6, 8, 10)
     gE = torch.from_numpy(synth.random_volume((3,) + shape, seed=1)).cuda()
     gV = torch.empty(shape, device="cuda")
@@ -87,6 +89,25 @@ def test_dense_bricks_are_spread_over_the_device(sal, n):
     try:
         textured = run(torch.from_numpy(synth.random_volume(shape, seed=2)).cuda())
         constant = run(torch.full(shape, 0.375, device="cuda"))
+        lone = torch.zeros(shape, device="cuda")
+        lone[0, 0, 0] = 1.0
+        lone = run(lone)
     finally:
         eng.close()
     assert constant <= 50 * textured
+    assert lone <= (5 if n == 8 else 50) * textured
+
+
+@pytest.mark.parametrize("n,shape,boundary,share", [(8, (12, 16, 20), "symmetric", 0.05), (8, (12, 16, 20), "zero", 0.01),
+                                                    (8, (9, 18, 40), "periodic", 0.02), (16, (12, 16, 20), "symmetric", 0.01),
+                                                    (16, (18, 13, 35), "zero", 0.002)])
+def test_bricks_of_sparse_volumes_match_oracle(sal, n, shape, boundary, share):
+    """Isolated samples: cubes that hold few of them have many bins that are zero, of which some bricks list up to the
+    limit and others more."""
+    r = np.random.RandomState(n)
+    V = (r.randn(*shape) * (r.rand(*shape) < share)).astype(np.float32)
+    V[0, 0, 0] = 1.0
+    assert oracle.band_count(V, n, boundary, lo=2.0 ** -40, hi=2.0 ** -36).sum() == 0
+    gE = synth.random_volume((3,) + shape, seed=n + 9)
+    got, want = _adjoint(sal, V, gE, n=n, boundary=boundary), oracle.features_adjoint(V, gE, n, boundary=boundary)
+    assert np.linalg.norm(got - want) <= RTOL * np.linalg.norm(want)
