@@ -20,10 +20,10 @@
 // The instruction cache sets how far the loop over outputs is unrolled: by R, and not at all in tile 0, whose packed rows
 // need the most code for an eighth of the work (there every window is an FFT).
 // Bound: issue slots, about 500 per thread and output of 16 bins with the FFTs and the small bins (128 MUFU cycles), by 12
-// warps an SM at 168 registers.  The adjoint call, 128^3: n = 16 25.0 -> 6.9 ms, n = 8 2.54 -> 0.87
+// warps an SM at 168 registers.  The adjoint call, 128^3: n = 16 25.0 -> 6.9 ms, n = 8 2.54 -> 0.91
 // (before: one x0 per brick, direct DFTs in stages 1 and 2 and both of their adjoints, 31 point evaluations of 32
 // multiply-adds per run of 8 outputs, and two passes over the grid for the small bins, 0.1 per voxel here); 24^3, n = 16:
-// 353 -> 186 us.  Error against FP64 9.7e-7 -> 9.8e-7 (n = 16), 8.0e-7 -> 8.3e-7 (n = 8), most of it in the directions
+// 353 -> 186 us.  Error against FP64 9.8e-7 -> 9.7e-7 (n = 16), 7.9e-7 -> 7.6e-7 (n = 8), most of it in the directions
 // of the weak bins just above the small-bin level.
 #include "spectra_f32_exact.cuh"
 #include "spectra_f32_fft.cuh"
@@ -100,6 +100,7 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
     using B = Bins<N, false>;
     constexpr int RX = G::RX, R = AGeo<N>::R, XH = G::XH, YH = G::YH, GT = G::GT, H = G::H, TILES = G::TILES, NW = B::NW;
     constexpr size_t TILE_W = (size_t)3 * H * N;   // weights of a tile, [map][k][row] (f32_slide_table_fill)
+    constexpr bool ALT = N == 8;                   // the directions of weak bins (at n = 16 no further off than direct sums)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float s_ex[4][N];   // cos, sin (2 pi m / n) as float-float pairs, indexed by the lanes' own phases
     const int grp = threadIdx.x / GT, tid = threadIdx.x % GT, lane = threadIdx.x & 31, warp = tid >> 5;
@@ -166,7 +167,7 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
             for (int u = 0; u < N; ++u) a += fabsf(v[u]);
             s_col[it] = a;
         }
-        f32::rfft<N>(v, o);
+        f32::rfft<N, ALT>(v, o);
 #pragma unroll
         for (int k = 0; k < TILES; ++k) s_g1[(size_t)k * XH * YH + it] = o[k];
     }
@@ -201,7 +202,7 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
             float2 v[N];
 #pragma unroll
             for (int u = 0; u < N; ++u) v[u] = src[u * YH];
-            f32::fft<N>(v);
+            f32::fft<N, ALT>(v);
             float2* dst = s_g2 + (size_t)x * N * YH + y;
             if (tile != 0) {
 #pragma unroll
@@ -258,7 +259,7 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
             const float pk = packed ? 1.f : 0.f, qk = 1.f - 2.f * pk;
 #pragma unroll 1
             for (int h = 0; h < kRun; h += R) {
-                f.template first<N>(row + h);   // phases are those of the run's first window
+                f.template first<N, ALT>(row + h);   // phases are those of the run's first window
 #pragma unroll
                 for (int q = 0; q < N / 2; ++q) P.r[q] = P.i[q] = make_float2(0.f, 0.f);
                 if (tile != 0) {
@@ -315,7 +316,7 @@ k5_slide(const float* __restrict__ V, const float* __restrict__ gE, float* __res
 #pragma unroll 1
                     for (int b = 0; b < R; ++b) {
                         const int j = h + b;
-                        if (b > 0) f.template first<N>(row + j);
+                        if (b > 0) f.template first<N, ALT>(row + j);
                         float rho[NW];
                         weights(j, rho);
                         const float g0 = ge[j], g1 = ge[RX * kRun + j], g2 = ge[2 * RX * kRun + j];
