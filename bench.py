@@ -79,7 +79,7 @@ def op_rates():
                      for k, v in PEAKS["mufu"].items())
 # K1 DRAM traffic per launch (bytes) from an ncu capture of the same kernel and workload;
 # None until captured for the current kernel.
-K1_TRAFFIC = {("salt128", 16, "fp32"): 8498688,   # profiles/kernels_128cubed_n16.md (per launch)
+K1_TRAFFIC = {("salt128", 16, "fp32"): 8498176,   # profiles/kernels_128cubed_n16.md (per launch)
               ("salt128", 16, "bf16"): 8518400,
               # one-pass capture of the full-scale launch (1.56 GB read + 3.39 GB written: ncu's 3-digit
               # figures); profiles/full462x951x651_n16_bf16_fwd_bwd.md
@@ -88,7 +88,7 @@ K1_TRAFFIC = {("salt128", 16, "fp32"): 8498688,   # profiles/kernels_128cubed_n1
 # bricks (profiles/kernels_128cubed_n16.md); a brick's traffic does not depend on the volume, so the
 # full-scale call (2,254,098 bricks over its t-slab launches) is that per-brick figure times its bricks.
 K5_TRAFFIC = {("salt128", 16, "bf16"): 727448576,
-              ("salt128", 16, "fp32"): 579679232,
+              ("salt128", 16, "fp32"): 619414784,
               ("full462x951x651", 16, "bf16"): 100081810319}
 
 

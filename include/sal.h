@@ -192,7 +192,8 @@ sal_status sal_combine_noalloc(int T, int X, int Y, const float* S3, const float
  *   RLS:  k = P x / (lambda + x'P x); W += k e; P = (P - k x'P) / lambda   (W0 = 0, P0 = I / delta)
  * in FP64.  sections = 0: one recursion over the whole volume; sections = N > 0: the weights are
  * re-adapted for every block of N inline sections (each block its own recursion from W0), as the
- * paper allows.  The recursion is sequential by nature: one warp per block.
+ * paper allows.  Long chains (RLS: with lambda = 1) are regrouped into segments that run side by side, with the filters'
+ * results up to FP64 rounding; the others run step by step, one warp per block.
  * S3: [3][T][X][Y] raw maps; D: [T][X][Y]; W_out: device [ceil(Y / N)][3] (one row when
  * sections = 0); err2 (nullable): device [T*X*Y], the squared error e^2 of every step in filter
  * order.  The weights of a block can be passed to sal_combine as W_in. */

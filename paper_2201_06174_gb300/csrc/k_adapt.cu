@@ -16,7 +16,7 @@
 // since each one is an affine map of the weights (LMS, NLMS: W -> (I - g x x') W + g d x) or adds to a sum
 // (RLS with lambda = 1: R += x x', z += x d, with P = R^-1 and W = R^-1 z), and both compose associatively:
 //   k3_adapt_segments  a thread per segment of L steps of one section: the segment's map, then by a tree
-//                      the map of the block's 32 segments of each section (FP64 throughput: about 30
+//                      the map of the block's 32 segments of each section (FP64 throughput: about 40
 //                      operations a step at 2 per clock and SM);
 //   k3_adapt_chain     a block per chain: the weights at the start of each group of 32 segments, and W_out;
 //   k3_adapt_errors    (only for err2) each segment's steps again from its own starting weights, all at once.
@@ -123,8 +123,9 @@ k3_adapt(const float* __restrict__ S3, const float* __restrict__ D, int T, int X
 }
 
 // ---- The regrouped form -------------------------------------------------------------------------
-constexpr int kSegY = 4;               // sections of a block: with 8 (a whole 32-byte sector of S3 and D) the 216 blocks of
-                                       // a 96^3 volume left half of the SMs with two and the others waiting
+constexpr int kSegY = 4;               // sections of a block: with 8 (a whole 32-byte sector of S3 and D) too few blocks to
+                                       // share the SMs evenly, NLMS with errors on 48^3, 96^3, 128^3: 139, 255 and 432 us against
+                                       // 175, 293 and 528 (200^3 1545 against 1489)
 constexpr int kSegS = 32;              // segments of each section in a block
 constexpr int kSegThreads = kSegY * kSegS;
 constexpr int kMinSeg = 16;            // steps of a segment at least: the maps' composition costs what ~1.5 steps cost

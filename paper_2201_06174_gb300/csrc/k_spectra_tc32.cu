@@ -19,7 +19,7 @@
 // those of P - 3 and before are.
 // Bound: latency between the passes (about 12 k cycles a k_t tile, of which the MUFU pipe needs 4.1 k for the 17,408
 // square roots a voxel, the MMAs 3 to 4 k, and a group's four epilogues take 6.4 k); stage 1 takes 30 k of 235 k cycles a
-// brick.  64 x 96 x 96: 12.4 -> 6.3 ms (before: CTA-wide barriers around every pass, the FP32 sums of stage 1 again for
+// brick.  64 x 96 x 96: 12.4 -> 6.3 ms, the call 6.4 (before: CTA-wide barriers around every pass, the FP32 sums of stage 1 again for
 // every k_t, a maximum pass over every brick, operands laid out in 2-byte pieces with a division each).
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
